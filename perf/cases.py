@@ -18,6 +18,7 @@ N(0, 1).  Mixed bit-widths are drawn per matrix, nested configurations per modul
 """
 import random
 
+import numpy as np
 import torch
 
 import paper_2501_07139_b200 as P
@@ -279,3 +280,59 @@ def tolerance(case):
     if case["kind"] == "prefill":
         return {"rel": 5e-3, "max": 0.05}
     return {"rel": 1e-3, "max": 5e-3}
+
+
+# ------------------------------------------------------------------------------------------------ the same in 64 bits
+def _weights64(n, k, bits, fmt, gen):
+    """float64 [N][K]: the dequantised weights of a layer, from the real-valued ones that `_add_layer` draws."""
+    w = torch.randn((n, k), device="cuda", generator=gen).mul_(0.02).double().view(n, k // GROUP, GROUP)
+    width = 8 if fmt == "nested" else bits
+    qmax = 2 ** width - 1
+    low, high = w.amin(2, keepdim=True), w.amax(2, keepdim=True)
+    s = ((high - low) / qmax).cpu().numpy().astype(np.float16)              # one rounding, to nearest
+    s = torch.from_numpy(np.where(s == 0, np.float16(2.0 ** -14), s)).double().cuda()
+    z = (-low / s).round().clamp(0, qmax)
+    q = ((w / s).round() + z).clamp(0, qmax)
+    if bits < width:                                                        # the child: high bits, mid-point fill
+        step = 2 ** (width - bits)
+        q = torch.floor(q / step) * step + step / 2
+    return ((q - z) * s).view(n, k)
+
+
+def exact(case, seed):
+    """What `run` returns, in float64 with weights that are not rounded; quantising has whole numbers only."""
+    kind = case["kind"]
+    if kind == "quantize":
+        return None
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    if kind == "gemv":
+        w = _weights64(case["n"], case["k"], case["bits"], case["fmt"], gen)
+        return torch.randn((case["batch"], case["k"]), device="cuda", generator=gen).half().double() @ w.T
+    layers, bits = _blocks(case), _bits(case)
+    both = bits if kind == "switch" else (bits,)
+
+    def products(inputs):
+        """One list of outputs per configuration; the weights are drawn again from the seed, as often as they are needed."""
+        out = []
+        for widths in both:
+            again = torch.Generator(device="cuda")
+            again.manual_seed(seed)
+            out.append([inputs[i] @ _weights64(n, k, widths[i], case["fmt"], again).T for i, (_, n, k, _, _) in enumerate(layers)])
+        return out
+
+    for _, n, k, _, _ in layers:                                            # `prepare` draws every weight before the activations
+        torch.randn((n, k), device="cuda", generator=gen)
+    if kind == "prefill":
+        m = case["tokens"]
+        x = {k: torch.randn((m, k), device="cuda", generator=gen).bfloat16().double() for k in sorted({l[2] for l in layers})}
+        return products([x[l[2]] for l in layers])[0]
+    b = case["batch"]
+    got = products([torch.randn((b, l[2]), device="cuda", generator=gen).half().double() for l in layers])
+    outs = []
+    for ys in got:
+        buf, views = _views([(b, l[1]) for l in layers], torch.float64)
+        for v, y in zip(views, ys):
+            v.copy_(y)
+        outs.append(buf)
+    return {"footprints": [None, None], "high": outs[0], "low": outs[1]} if kind == "switch" else outs[0]
