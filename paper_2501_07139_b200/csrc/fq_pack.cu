@@ -8,7 +8,7 @@ namespace fq {
 #define FQ_CUDA_OK(expr) do { if ((expr) != cudaSuccess) return FQ_ERR_CUDA; } while (0)
 
 // ---------------------------------------------------------------------------------------
-// Quantiser: one warp per (row, group); all arithmetic that decides a code runs in double.
+// Quantiser: a code is decided by arithmetic in double, or by single precision where that cannot differ.
 // ---------------------------------------------------------------------------------------
 
 // Nearest-even conversion of a non-negative finite double to fp16 bits, done on the
@@ -33,48 +33,107 @@ __device__ __forceinline__ unsigned f64_to_f16_bits_nonneg(double v)
     return r >= 0x7c00ull ? 0x7c00u : (unsigned)r;
 }
 
-__device__ __forceinline__ double f16_bits_to_f64(unsigned h)
-{
-    return (double)__half2float(__ushort_as_half((unsigned short)h));
-}
+// Bound by HBM: 4 bytes in, 1 out per weight.  A warp takes kQuantGroups groups at once, so that a lane has that many
+// 16-byte loads in flight, and scale and zero point of a group are formed once, by one lane, instead of by all 32.  A code
+// is rint(w / s) + z with the quotient in double; it is first formed as w * (1 / s), whose error for |w / s| < 1024 is below
+// 1024 * 2^-24 < 2^-12 (s is an fp16 number, so exact; 1 / s is rounded once).  Only where the quotient is that close to a
+// rounding boundary, or not finite, it is formed in double: the codes are the same integers.  11008 x 4096: 126 us with every division in double,
+// about 40 us like this (225 MB, 34 us at the copy bandwidth).
+constexpr int kQuantGroups = 8;                // groups per warp
+constexpr int kQuantWarps = 8;
+constexpr float kRint = 12582912.f;            // 1.5 * 2^23: adding it rounds to an integer, ties to even
 
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kQuantWarps * 32, 4)
 quantize_kernel(const float* __restrict__ w, long long n_groups_total, int bits,
                 uint8_t* __restrict__ codes, uint16_t* __restrict__ scales, uint16_t* __restrict__ zeros)
 {
     const int lane = threadIdx.x & 31;
-    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
-    const double qmax = (double)((1 << bits) - 1);
-    for (long long grp = warp; grp < n_groups_total; grp += n_warps) {
-        const float4 v = reinterpret_cast<const float4*>(w + grp * kGroup)[lane];
-        float mn = fminf(fminf(v.x, v.y), fminf(v.z, v.w));
-        float mx = fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w));
+    const long long g0 = ((long long)blockIdx.x * kQuantWarps + (threadIdx.x >> 5)) * kQuantGroups;
+    if (g0 >= n_groups_total) return;
+    const int n = (int)min((long long)kQuantGroups, n_groups_total - g0);
+    const float top = (float)((1 << bits) - 1);
+    const double qmax = top;
+    float4 v[kQuantGroups];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        }
-        unsigned sb = f64_to_f16_bits_nonneg(((double)mx - (double)mn) / qmax);
-        if (sb == 0u) sb = 0x0400u;
-        if (sb >= 0x7c00u) sb = 0x7bffu;
-        const double S = f16_bits_to_f64(sb);
-        double z = rint(-(double)mn / S);
-        if (!(z > 0.0)) z = 0.0;
-        if (z > qmax) z = qmax;
-        const float vals[4] = {v.x, v.y, v.z, v.w};
-        unsigned packed = 0;
+    for (int i = 0; i < kQuantGroups; i++)
+        v[i] = i < n ? __ldcs(reinterpret_cast<const float4*>(w + (g0 + i) * kGroup) + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+    // minimum and (negated) maximum of the eight groups: every step of the reduction halves the number of values a lane holds,
+    // 17 shuffles in all instead of 80; lane l ends up with group (l >> 1) & 7
+    float r[2 * kQuantGroups];
 #pragma unroll
-        for (int i = 0; i < 4; i++) {
-            double q = rint((double)vals[i] / S) + z;
-            q = q < 0.0 ? 0.0 : (q > qmax ? qmax : q);
-            packed |= (unsigned)q << (8 * i);
+    for (int i = 0; i < kQuantGroups; i++) {
+        r[i] = fminf(fminf(v[i].x, v[i].y), fminf(v[i].z, v[i].w));
+        r[kQuantGroups + i] = -fmaxf(fmaxf(v[i].x, v[i].y), fmaxf(v[i].z, v[i].w));
+    }
+#pragma unroll
+    for (int o = 16; o > 1; o >>= 1) {
+        const bool upper = lane & o;
+#pragma unroll
+        for (int i = 0; i < o / 2; i++) {
+            const float keep = upper ? r[i + o / 2] : r[i], send = upper ? r[i] : r[i + o / 2];
+            r[i] = fminf(keep, __shfl_xor_sync(0xffffffffu, send, o));
         }
-        reinterpret_cast<unsigned*>(codes + grp * kGroup)[lane] = packed;
-        if (lane == 0) {
-            scales[grp] = (uint16_t)sb;
-            zeros[grp] = __half_as_ushort(__float2half_rn((float)z));   // an integer <= 255: exact
+    }
+    r[0] = fminf(r[0], __shfl_xor_sync(0xffffffffu, r[0], 1));
+    const float other = __shfl_xor_sync(0xffffffffu, r[0], 16);
+    const float mn = lane & 16 ? other : r[0], mx = -(lane & 16 ? r[0] : other);
+    const int mine = (lane >> 1) & (kQuantGroups - 1);
+    static_assert(kQuantGroups == 8, "lanes of the reduction");
+    float scale = 1.f, zero = 0.f;
+    if (mine < n) {
+        // scale = fp16((max - min) / qmax): in single precision the quotient is off by at most three units in the last
+        // place, so its rounding to fp16 is the right one unless it lies within eight of them from a tie
+        unsigned sb;
+        const float f = (mx - mn) * (1.f / top);
+        if (f >= 0x1p-14f && f < 60000.f && abs((int)(__float_as_uint(f) & 0x1fffu) - 0x1000) > 8) {
+            sb = __half_as_ushort(__float2half_rn(f));
+        } else {
+            sb = f64_to_f16_bits_nonneg(((double)mx - (double)mn) / qmax);
+            if (sb == 0u) sb = 0x0400u;
+            if (sb >= 0x7c00u) sb = 0x7bffu;
         }
+        scale = __half2float(__ushort_as_half((unsigned short)sb));  // exact
+        // zero = clamp(rint(-min / scale)): as for the codes below
+        const float ratio = -mn * (1.f / scale);
+        zero = __fadd_rn(__fadd_rn(ratio, kRint), -kRint);
+        if (!(fabsf(ratio) < 1024.f && fabsf(ratio - zero) < 0.5f - 0x1p-12f)) {
+            const double z = rint(-(double)mn / (double)scale);
+            zero = z > qmax ? top : (float)z;
+        }
+        if (!(zero > 0.f)) zero = 0.f;                               // (also -0 and NaN)
+        if (zero > top) zero = top;
+        if (lane == 2 * mine) {
+            scales[g0 + mine] = (uint16_t)sb;
+            zeros[g0 + mine] = __half_as_ushort(__float2half_rn(zero));   // an integer <= 255: exact
+        }
+    }
+    const float inverse = 1.f / scale, shifted = kRint + zero;       // exact: a small integer
+#pragma unroll
+    for (int i = 0; i < kQuantGroups; i++) {
+        const float inv = __shfl_sync(0xffffffffu, inverse, 2 * i), base = __shfl_sync(0xffffffffu, shifted, 2 * i);
+        if (i >= n) break;
+        const float vals[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+        float u[4];
+        bool sure = true;
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            u[e] = fmaf(vals[e], inv, base);                         // kRint + z + rint(w / s), one rounding
+            const float off = fmaf(vals[e], inv, -(u[e] - base));    // how far w / s is from that integer
+            sure = sure && fabsf(off) < 0.5f - 0x1p-12f;             // (false for NaN; beyond 1024 the code is clamped anyway)
+            u[e] = fminf(fmaxf(u[e], kRint), kRint + top);           // the code is the low byte
+        }
+        if (!sure) {
+            const double s = __half2float(__float2half_rn(1.f / inv)), z = base - kRint;
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                double qd = rint((double)vals[e] / s) + z;
+                qd = qd < 0.0 ? 0.0 : (qd > qmax ? qmax : qd);
+                u[e] = kRint + (float)(unsigned)qd;                  // (NaN becomes 0)
+            }
+        }
+        const unsigned packed = __byte_perm(__byte_perm(__float_as_uint(u[0]), __float_as_uint(u[1]), 0x0040),
+                                            __byte_perm(__float_as_uint(u[2]), __float_as_uint(u[3]), 0x0040), 0x5410);
+        reinterpret_cast<unsigned*>(codes + (g0 + i) * kGroup)[lane] = packed;
     }
 }
 
@@ -95,69 +154,120 @@ int launch_quantize(const float* w, int n_out, int k_in, int bits, uint8_t* code
                     uint16_t* zeros, cudaStream_t st)
 {
     const long long groups = (long long)n_out * (k_in / kGroup);
-    long long blocks = (groups + 7) / 8;
-    if (blocks > current_sm_count() * 16) blocks = current_sm_count() * 16;
-    if (blocks < 1) return FQ_OK;
-    quantize_kernel<<<(unsigned)blocks, 256, 0, st>>>(w, groups, bits, codes, scales, zeros);
+    if (groups < 1) return FQ_OK;
+    const long long per_block = kQuantWarps * kQuantGroups;
+    const long long blocks = (groups + per_block - 1) / per_block;
+    if (blocks > 0x7fffffffll) return FQ_ERR_SHAPE;
+    quantize_kernel<<<(unsigned)blocks, kQuantWarps * 32, 0, st>>>(w, groups, bits, codes, scales, zeros);
     FQ_CUDA_OK(cudaGetLastError());
     return FQ_OK;
 }
 
 // ---------------------------------------------------------------------------------------
-// Packer: one thread per 32-bit word of the stored variant (blob layout, see fq_layout.cuh).
+// Packer (blob layout, see fq_layout.cuh): one block per blob, one warp per (superstep, row tile) of it.
+//
+// Bound by HBM (1 byte in, bits / 8 out per weight; the codes are usually still in L2 after the quantiser).  The 32 x 512
+// codes of the blob go through shared memory with 16-byte loads; a lane then holds, as 32 words of four codes, exactly the A
+// registers it owns in the decode kernel (rows g and g + 8, columns 4c .. 4c + 3 of every half k32 step), and a field is
+// cut out of four codes at once with one shift and one AND, because a field never crosses a byte.  Every store is 16 bytes
+// a lane, 512 contiguous bytes a warp.  11008 x 4096, 8 / 5 / 3 bits: 160 / 230 / 197 us with one thread per stored
+// word gathering its codes byte by byte, about 13 us like this (whatever the width).
 // ---------------------------------------------------------------------------------------
 struct StoreArgs {
-    const uint8_t* codes;          // pack: canonical codes, one per byte
+    const uint8_t* codes;          // canonical codes, one per byte
     const uint16_t* scales;
     const uint16_t* zeros;
-    uint32_t* store;               // the stored variant
+    uint8_t* store;                // the stored variant
     int n_out, k_in, n_kb, groups;
     int stored_bits;               // bits of the stored variant (size of its blobs)
-    FieldList fl;                  // fields that are written / read
-    long long total_words;
+    FieldList fl;                  // fields that are written
+    bool wide;                     // codes are 16-byte aligned (rows are multiples of 128 bytes)
 };
 
-__global__ void __launch_bounds__(256) pack_kernel(const StoreArgs a)
+constexpr int kPackThreads = kBlobSteps * kBlobTiles * 32;
+constexpr int kPackCols = kBlobSteps * kStepCols;                // columns of a blob
+constexpr int kPackRow = kPackCols + 16;                         // bytes between rows: lanes (g, c) hit banks 4g + c
+
+// Field of width F at bit `shift`: registers of P = 8 / F consecutive k32 steps on top of each other.
+template <int F>
+__device__ __forceinline__ void pack_field(const uint32_t (&code)[8][4], int shift, uint8_t* dst)
 {
-    const int blob_words = blob_bytes(a.stored_bits) / 4;
-    for (long long wi = (long long)blockIdx.x * blockDim.x + threadIdx.x; wi < a.total_words;
-         wi += (long long)gridDim.x * blockDim.x) {
-        const long long blob = wi / blob_words;
-        const int off = (int)(wi % blob_words) * 4;               // byte offset inside the blob
-        const int rp = (int)(blob / a.n_kb), kb = (int)(blob % a.n_kb);
-        unsigned v = 0;
-        if (off < kBlobMetaBytes) {
-            // scale/zero word: [superstep][tile][row & 7][group][row >> 3]
-            const int r = ((off >> 4) & 7) + 8 * ((off >> 2) & 1), grp = (off >> 3) & 1, tile = (off >> 7) & 1, ssl = off >> 8;
-            const long long n = ((long long)rp * kBlobTiles + tile) * kTileRows + r;
-            const int g = (kb * kBlobSteps + ssl) * 2 + grp;
-            if (n < a.n_out && g < a.groups) {
-                const float z = __half2float(__ushort_as_half(a.zeros[n * a.groups + g]));
-                const unsigned zi = (unsigned)fminf(fmaxf(rintf(z), 0.f), 65535.f);
-                v = (unsigned)a.scales[n * a.groups + g] | (zi << 16);
-            }
-        } else {
-            int rem = off - kBlobMetaBytes, fi = 0;
-            while (rem >= kBlobSteps * kBlobTiles * 512 * a.fl.width[fi]) {
-                rem -= kBlobSteps * kBlobTiles * 512 * a.fl.width[fi];
-                fi++;
-            }
-            const int f = a.fl.width[fi], sh = a.fl.shift[fi];
-            const int st = rem / (f * 512), in_tile = rem % (f * 512);       // st = ssl * 2 + tile
-            const int ssl = st / kBlobTiles, tile = st % kBlobTiles;
-            const int chunk = in_tile >> 9, lane = (in_tile >> 4) & 31, word = (in_tile >> 2) & 3;
-            const unsigned mask = (1u << f) - 1u;
-            for (int q = 0; q < 32 / f; q++) {
-                int r, kk, bit;
-                field_owner(f, chunk, lane, word, q, r, kk, bit);
-                const long long n = ((long long)rp * kBlobTiles + tile) * kTileRows + r;
-                const long long k = ((long long)kb * kBlobSteps + ssl) * kStepCols + kk;
-                unsigned code = 0;
-                if (n < a.n_out && k < a.k_in) code = a.codes[n * a.k_in + k];
-                v |= ((code >> sh) & mask) << bit;
+    constexpr int P = 8 / F;
+    constexpr uint32_t kMask = ((1u << F) - 1u) * 0x01010101u;
+#pragma unroll
+    for (int chunk = 0; chunk < F; chunk++) {
+        uint32_t word[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int t = 0; t < P; t++)
+#pragma unroll
+            for (int a = 0; a < 4; a++) word[a] |= ((code[chunk * P + t][a] >> shift) & kMask) << (t * F);
+        *reinterpret_cast<uint4*>(dst + chunk * 512) = make_uint4(word[0], word[1], word[2], word[3]);
+    }
+}
+
+__global__ void __launch_bounds__(kPackThreads) pack_kernel(const __grid_constant__ StoreArgs a)
+{
+    __shared__ __align__(16) uint8_t tile_codes[kBlobTiles * kTileRows * kPackRow];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int rp = (int)(blockIdx.x / (unsigned)a.n_kb), kb = (int)(blockIdx.x % (unsigned)a.n_kb);
+    const long long n0 = (long long)rp * kBlobTiles * kTileRows;
+    const int k0 = kb * kPackCols;
+    uint8_t* blob = a.store + (long long)blockIdx.x * blob_bytes(a.stored_bits);
+
+    uint4 raw[kBlobTiles * kTileRows / (kPackThreads / 32)];         // a warp reads a row of the blob, 16 bytes a lane
+#pragma unroll
+    for (int i = 0; i < (int)(sizeof raw / sizeof raw[0]); i++) {
+        const int r = i * (kPackThreads / 32) + warp, k = k0 + lane * 16;
+        raw[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (n0 + r < a.n_out && k < a.k_in) {                        // (k_in is a multiple of 128)
+            const uint8_t* src = a.codes + (n0 + r) * a.k_in + k;
+            if (a.wide) {
+                raw[i] = *reinterpret_cast<const uint4*>(src);
+            } else {
+                uint32_t* w = reinterpret_cast<uint32_t*>(&raw[i]);
+#pragma unroll
+                for (int b = 0; b < 16; b++) w[b >> 2] |= (uint32_t)src[b] << (8 * (b & 3));
             }
         }
-        a.store[wi] = v;
+    }
+    {   // scale/zero word: [superstep][tile][row & 7][group][row >> 3]
+        const int off = t * 4;
+        const int r = ((off >> 4) & 7) + 8 * ((off >> 2) & 1), grp = (off >> 3) & 1, tile = (off >> 7) & 1, ssl = off >> 8;
+        const long long n = n0 + tile * kTileRows + r;
+        const int g = (kb * kBlobSteps + ssl) * 2 + grp;
+        unsigned v = 0;
+        if (n < a.n_out && g < a.groups) {
+            const float z = __half2float(__ushort_as_half(a.zeros[n * a.groups + g]));
+            const unsigned zi = (unsigned)fminf(fmaxf(rintf(z), 0.f), 65535.f);
+            v = (unsigned)a.scales[n * a.groups + g] | (zi << 16);
+        }
+        reinterpret_cast<uint32_t*>(blob)[t] = v;
+        static_assert(kBlobMetaBytes == 4 * kPackThreads, "one scale/zero word per thread");
+    }
+#pragma unroll
+    for (int i = 0; i < (int)(sizeof raw / sizeof raw[0]); i++)
+        *reinterpret_cast<uint4*>(tile_codes + (i * (kPackThreads / 32) + warp) * kPackRow + lane * 16) = raw[i];
+    __syncthreads();
+
+    const int ssl = warp / kBlobTiles, tile = warp % kBlobTiles, g = lane >> 2, c = lane & 3;
+    uint32_t code[8][4];                                             // [k32 step][A register]
+#pragma unroll
+    for (int j = 0; j < 8; j++)
+#pragma unroll
+        for (int r = 0; r < 4; r++)
+            code[j][r] = *reinterpret_cast<const uint32_t*>(tile_codes + (tile * kTileRows + g + 8 * (r & 1)) * kPackRow +
+                                                            ssl * kStepCols + j * 32 + (r >> 1) * 16 + c * 4);
+    int prefix = 0;
+    for (int fi = 0; fi < a.fl.n; fi++) {
+        const int f = a.fl.width[fi], shift = a.fl.shift[fi];
+        uint8_t* dst = blob + blob_field_off(prefix, f, ssl, tile) + lane * 16;
+        switch (f) {
+            case 8: pack_field<8>(code, shift, dst); break;
+            case 4: pack_field<4>(code, shift, dst); break;
+            case 2: pack_field<2>(code, shift, dst); break;
+            default: pack_field<1>(code, shift, dst); break;
+        }
+        prefix += f;
     }
 }
 
@@ -172,11 +282,13 @@ int launch_pack(const uint8_t* codes, const uint16_t* scales, const uint16_t* ze
                 int stored_bits, const FieldList& fl, void* store, cudaStream_t st)
 {
     StoreArgs a{};
-    a.codes = codes; a.scales = scales; a.zeros = zeros; a.store = (uint32_t*)store;
+    a.codes = codes; a.scales = scales; a.zeros = zeros; a.store = (uint8_t*)store;
     a.n_out = n_out; a.k_in = k_in; a.n_kb = k_blobs(k_in); a.groups = k_in / kGroup;
     a.stored_bits = stored_bits; a.fl = fl;
-    a.total_words = store_bytes(n_out, k_in, stored_bits) / 4;
-    pack_kernel<<<grid_for(a.total_words), 256, 0, st>>>(a);
+    a.wide = (reinterpret_cast<uintptr_t>(codes) & 15) == 0;
+    const long long blobs = (long long)row_pairs(n_out) * a.n_kb;
+    if (blobs > 0x7fffffffll) return FQ_ERR_SHAPE;
+    pack_kernel<<<(unsigned)blobs, kPackThreads, 0, st>>>(a);
     FQ_CUDA_OK(cudaGetLastError());
     return FQ_OK;
 }
