@@ -83,7 +83,7 @@ int fill_op(const Ctx* ctx, int layer, const uint16_t* x, uint16_t* y, int batch
     op.n_kb = k_blobs(L.k_in);
     op.n_rp = row_pairs(L.n_out);
     op.chunk_blobs = one ? gemv1_chunk_blobs(op.blob_read)
-                                : gemv_chunk_blobs(L.fmt == FQ_FMT_PLANES ? plane_read_bits(bits) : bits, batch);
+                                : gemv_chunk_blobs(L.fmt == FQ_FMT_PLANES ? plane_read_bits(bits) : bits);
     op.n_chunks = (op.n_kb + op.chunk_blobs - 1) / op.chunk_blobs;
     op.batch = batch;
     // nested child: codes are the parent's top bits; the dropped bits are filled with their mid-point

@@ -6,22 +6,18 @@
 //                     active variant plus the scale/zero words) from HBM into a shared-memory
 //                     ring with bulk asynchronous copies (cp.async.bulk + mbarrier tx counts)
 //                     and writes a small descriptor next to each stage;
-//   x-prep warps    : once per (op, K chunk) that this CTA touches, wait -- bounded -- for the
-//                     previous dependency phase, load the activations of that chunk and turn
-//                     them into 16-bit fixed point per group of 128 columns
-//                     (x_int = rint(x * 2^e), |x_int| < 2^14, stored as two signed byte digits);
-//   consumer warps  : two warps share a unit, one 16-row tile each.  Stored words become 8-bit
-//                     mma.m16n8k32 A operands with ONE AND each (no shift: a word holds 8/f
-//                     registers on top of each other, see fq_layout.cuh), the activation digits
-//                     are the B operand, accumulation is exact in s32.  At batch 1 the eight B
-//                     columns carry (low digit, high digit) for up to four bit-offset classes,
-//                     so no register ever has to be shifted.  The loops are compiled once per
-//                     field list (14 variants) and chosen per unit.
-//   output warp     : finishes row pairs (see below) and is the only warp that writes y.
-//   Per group:  y += s * 2^-e * ( sum_fields 2^shift * sum_k field_k * x_int_k  -  z * sum_k x_int_k ).
+//   activation warp : once per (op, K chunk) that this CTA touches, waits -- bounded -- for the
+//                     previous dependency phase and fetches the activations of that chunk, one bulk copy per batch row;
+//   consumer warps  : two warps share a unit, one 16-row tile each.  Stored words become fp16 integers q - z, the fp16
+//                     activations are the other operand of mma.m16n8k16, sums are fp32 and scaled once per group of 128
+//                     columns (fq_batch_core.cuh).  The loops are compiled once per field list (14 variants) and chosen
+//                     per unit.  13B nested at 4 bits, four blocks, no
+//                     dependencies: 4 / 8 entries 189 / 238 us, against 330 / 600 us with one 8-bit integer MMA per field and digit
+//                     of fixed-point activations.
+//   output warps    : finish row pairs (see below) and are the only warps that write y.
 // The K chunks of one row pair are computed by different CTAs.  Each unit publishes its row sums
 // as 64-bit words (fp32 value, launch tag) with plain stores; the unit whose chunk index is
-// (row pair mod chunks) hands its own sums to the output warp, which polls the other chunks'
+// (row pair mod chunks) hands its own sums to an output warp, which polls the other chunks'
 // words until they carry this launch's tag and adds them in chunk order, so results do not
 // depend on scheduling and no fence or atomic sits on the consumers' path.
 //
@@ -32,8 +28,7 @@
 // computing, drains its copies and returns.
 #include <cuda_fp16.h>
 
-#include <type_traits>
-
+#include "fq_batch_core.cuh"
 #include "fq_internal.cuh"
 #include "fq_ptx.cuh"
 
@@ -41,34 +36,19 @@ namespace fq {
 
 #define FQ_CUDA_OK(expr) do { if ((expr) != cudaSuccess) return FQ_ERR_CUDA; } while (0)
 
-#ifndef FQ_GEMV_WARPS
-#define FQ_GEMV_WARPS 18
-#endif
-#ifndef FQ_GEMV_TPW
-#define FQ_GEMV_TPW 1
-#endif
-#ifndef FQ_GEMV_UNIT_BYTES
-#define FQ_GEMV_UNIT_BYTES 17408
-#endif
-constexpr int kConsumerWarps = FQ_GEMV_WARPS;
-constexpr int kTilesPerWarp = FQ_GEMV_TPW;             // 16-row tiles of a unit that one consumer warp computes
-constexpr int kWarpsPerUnit = kUnitRowTiles / kTilesPerWarp;
+constexpr int kConsumerWarps = 20;
+constexpr int kWarpsPerUnit = kUnitRowTiles;           // one 16-row tile each
 constexpr int kUnitsInFlight = kConsumerWarps / kWarpsPerUnit;
-static_assert(kTilesPerWarp == 1 || kTilesPerWarp == 2, "a warp computes one or both row tiles of a unit");
 static_assert(kConsumerWarps % kWarpsPerUnit == 0, "consumer warps come in groups of one unit");
 constexpr int kProducerWarp = kConsumerWarps;          // warp index of the producer
-constexpr int kPrepWarp = kConsumerWarps + 1;          // first warp of the activation pre-processors
-constexpr int kPrepWarps = 4;                          // they share the items of a segment
-constexpr int kOutputWarp = kPrepWarp + kPrepWarps;    // the warp that owns every global store of results
-constexpr int kGemvThreads = (kConsumerWarps + 1 + kPrepWarps + 1) * 32;
-constexpr int kUnitBytes = FQ_GEMV_UNIT_BYTES;         // bytes of one unit (whole blobs), at most: 2 x 4-bit or 1 x 8-bit blob
-constexpr int kXSlots = 3;                             // activation chunks kept in shared memory
-
-template <int MAXB> struct GemvCfg;
-// kBlobsMax: k blobs (512 columns) per chunk, at most.  kOutSlots: finished units waiting for the output
-// warp (it scans one slot per lane: at most 32).
-template <> struct GemvCfg<1> { static constexpr int kBlobsMax = 3, kOutSlots = 32; };
-template <> struct GemvCfg<8> { static constexpr int kBlobsMax = 2, kOutSlots = 16; };
+constexpr int kActWarp = kConsumerWarps + 1;           // the warp that fetches activations
+constexpr int kOutputWarp = kActWarp + 1;              // the warps that own every global store of results
+constexpr int kOutputWarps = 2;                        // each takes every other place of the output queue
+constexpr int kGemvThreads = (kConsumerWarps + 2 + kOutputWarps) * 32;     // 24 warps: 80 registers each
+constexpr int kUnitBytes = 17408;                      // bytes of one unit (whole blobs), at most: 2 x 4-bit or 1 x 8-bit blob
+constexpr int kBlobsMax = kXCols / 512;                // k blobs (512 columns) per chunk, at most
+constexpr int kOutSlots = 16;                          // finished units waiting for an output warp (it scans one slot per lane)
+constexpr int kXSlots = 4;                             // activation chunks kept in shared memory
 
 // What the producer tells the consumers: once per op a copy of the op descriptor in a ring ...
 constexpr int kOpRing = 16;                            // > stages + 1: an op slot outlives the start of its last unit
@@ -90,22 +70,13 @@ struct OutDesc {
 };
 static_assert(sizeof(OutDesc) == 48, "descriptor layout");
 
-template <int MAXB> struct GemvSmem {
-    static constexpr int kCMax = GemvCfg<MAXB>::kBlobsMax * kBlobSteps;     // supersteps per chunk, at most
-    static constexpr int kOutSlots = GemvCfg<MAXB>::kOutSlots;
+template <int BP> struct GemvSmem {
     static constexpr int kStageBytes = kUnitBytes;
-    // activation slot: low digits, high digits (rows padded so that LDS.64 of a quarter warp is
-    // conflict free), then per (row, group) the integer sum and the power-of-two scale
-    static constexpr int kXRow = MAXB == 1 ? kCMax * 256 : kCMax * 256 + 32;
-    static constexpr int kDigitOff = MAXB == 1 ? kXRow : MAXB * kXRow + 64;
-    static constexpr int kXsumOff = kDigitOff + MAXB * kXRow;
-    static constexpr int kXscaleOff = kXsumOff + MAXB * kCMax * 2 * 4;
-    static constexpr int kXSlotBytes = (kXscaleOff + MAXB * kCMax * 2 * 4 + 127) / 128 * 128;
-    static constexpr int kZeroBytes = kCMax * 256 + 64;
+    static constexpr int kXSlotBytes = BP * kXRowBytes;              // one chunk's activations
     static constexpr int kOpBytes = (int)((sizeof(GemvOp) + 15) / 16 * 16);
-    static constexpr int kOutFloats = 32 * (MAXB == 1 ? 1 : 8);              // row sums of one unit
+    static constexpr int kOutFloats = 32 * BP;                               // row sums of one unit
     static constexpr int kOutBytes = kOutSlots * (kOutFloats * 4 + (int)sizeof(OutDesc));
-    static constexpr int kFixed = kXSlots * kXSlotBytes + kZeroBytes + kOpRing * kOpBytes + (2 + 2 * kPrepWarps) * kOpBytes +
+    static constexpr int kFixed = kXSlots * kXSlotBytes + kOpRing * kOpBytes + 4 * kOpBytes +
                                   kOutBytes + 512;
     static constexpr int kPerStage = kStageBytes + (int)sizeof(UnitDesc) + 16 + 4;
     static constexpr int kAuto = (232448 - kFixed) / kPerStage;
@@ -113,10 +84,9 @@ template <int MAXB> struct GemvSmem {
     static constexpr int oStages = 0;
     static constexpr int oDesc = oStages + kStages * kStageBytes;
     static constexpr int oX = oDesc + kStages * (int)sizeof(UnitDesc);
-    static constexpr int oZero = oX + kXSlots * kXSlotBytes;
-    static constexpr int oOpRing = oZero + kZeroBytes;               // GemvOp[kOpRing]
-    static constexpr int oOpBuf = oOpRing + kOpRing * kOpBytes;   // GemvOp[2] producer, GemvOp[2] per x-prep warp
-    static constexpr int oOutData = oOpBuf + (2 + 2 * kPrepWarps) * kOpBytes;   // float[kOutSlots][kOutFloats]
+    static constexpr int oOpRing = oX + kXSlots * kXSlotBytes;       // GemvOp[kOpRing]
+    static constexpr int oOpBuf = oOpRing + kOpRing * kOpBytes;   // GemvOp[2] producer, GemvOp[2] activation warp
+    static constexpr int oOutData = oOpBuf + 4 * kOpBytes;   // float[kOutSlots][kOutFloats]
     static constexpr int oOutDesc = oOutData + kOutSlots * kOutFloats * 4;     // OutDesc[kOutSlots]
     static constexpr int oBars = oOutDesc + kOutSlots * (int)sizeof(OutDesc);  // full[S], empty[S]
     static constexpr int oReleased = oBars + 2 * kStages * 8;        // u32[S]: consumer warps that released a stage, ever
@@ -131,28 +101,17 @@ template <int MAXB> struct GemvSmem {
 };
 
 // K blobs (512 columns) per K chunk for a variant of which `bits` bits are read.
-int gemv_chunk_blobs(int bits, int batch)
+int gemv_chunk_blobs(int bits)
 {
-    const int cmax = batch <= 1 ? GemvCfg<1>::kBlobsMax : GemvCfg<8>::kBlobsMax;
     int c = kUnitBytes / blob_bytes(bits);
-    if (c > cmax) c = cmax;
+    if (c > kBlobsMax) c = kBlobsMax;
     if (c < 1) c = 1;
     return c;
 }
 static_assert(kUnitBytes >= kBlobMetaBytes + kBlobSteps * kBlobTiles * 512 * 8, "a unit must hold an 8-bit blob");
 
 // A split-K partial is one 64-bit word per (row, batch entry): fp32 sum in the low half, launch tag in the high half.
-size_t gemv_partial_bytes_per_unit(int batch) { return (batch <= 1 ? 32 : 256) * sizeof(unsigned long long); }
-
-// D += A(u8, 16x32, row) * B(s8, 32x8, col), s32 accumulate.
-__device__ __forceinline__ void mma_u8s8(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                         uint32_t b0, uint32_t b1)
-{
-    asm volatile(
-        "mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-        : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
+size_t gemv_partial_bytes_per_unit(int batch) { return (size_t)(32 * batch_pad(batch)) * sizeof(unsigned long long); }
 
 // ------------------------------------------------------------------------------- per-CTA work split
 // (this kernel numbers the units of an op chunk-major, u = ch * n_rp + rp, and deals them with cta_range)
@@ -191,276 +150,11 @@ struct OpFetch {
 };
 static_assert(sizeof(GemvOp) <= 256, "op descriptor too large for the two-word fetch");
 
-// ------------------------------------------------------------------------------- the arithmetic of one unit
-// Shared memory is addressed with 32-bit shared-window addresses and explicit ld.shared: the inner
-// loops then carry no 64-bit pointer arithmetic.
-// (OFF is a compile-time byte offset: it goes into the instruction's address field instead of costing an add)
-template <int OFF = 0>
-__device__ __forceinline__ uint4 lds128(uint32_t a)
-{
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4+%5];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a), "n"(OFF));
-    return v;
-}
-template <int OFF = 0>
-__device__ __forceinline__ uint2 lds64(uint32_t a)
-{
-    uint2 v;
-    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2+%3];" : "=r"(v.x), "=r"(v.y) : "r"(a), "n"(OFF));
-    return v;
-}
-template <int OFF = 0>
-__device__ __forceinline__ uint32_t lds32(uint32_t a)
-{
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(a), "n"(OFF));
-    return v;
-}
-// Loop whose index is a compile-time constant in the body (so that it can be a load's immediate offset).
-template <int I, int N, class Fn>
-__device__ __forceinline__ void static_for(Fn&& fn)
-{
-    if constexpr (I < N) {
-        fn(std::integral_constant<int, I>{});
-        static_for<I + 1, N>(fn);
-    }
-}
-// D = A(u8, 16x32, row) * B(s8, 32x8, col): first link of an accumulation chain (C = 0).
-__device__ __forceinline__ void mma_u8s8_first(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                               uint32_t b0, uint32_t b1)
-{
-    asm volatile(
-        "mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
-        : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "r"(0));
-}
-
-#ifndef FQ_GEMV_NA
-#define FQ_GEMV_NA 1
-#endif
-
-// One field of width F (at bit SHIFT of the code) of TILES row tiles, one superstep: eight k32 steps, the
-// first four belong to the first group of 128 columns, the last four to the second.  Adds (FIRSTF: stores),
-// per tile / pass / row / group, the integer  2^SHIFT * sum_k field_k * x_int_k  into v.
-//   fa     : shared address of this lane's 16-byte chunk in the first tile's field array
-//   MAXB 1 : B columns (2t, 2t+1) carry the activation digits for bit-offset class t; lane (g, c) ends up
-//            with the partial sum of class c, still scaled by 2^(c*F); xa[t] is the shared address of this
-//            lane's B data for class t (or of zeros)
-//   MAXB 8 : every register is shifted down to class 0; B columns (2b, 2b+1) carry batch entry
-//            4*pass + b; xa[pass] is this lane's B data
-// With one tile per warp and batch 1 the k32 steps of a group may alternate between FQ_GEMV_NA accumulators.
-template <int F, int KEEP, int SHIFT, bool FIRSTF, int MAXB, int TILES>
-__device__ __forceinline__ void field_step(uint32_t fa, const uint32_t (&xa)[4], uint32_t xoff, bool two_pass, int c,
-                                           int (&v)[TILES][MAXB == 1 ? 1 : 2][2][2])
-{
-    constexpr int P = 8 / F;                                   // A registers stacked in one word
-    constexpr uint32_t kMask = field_keep_mask(F, KEEP) * 0x01010101u;
-    constexpr int NP = MAXB == 1 ? 1 : 2;
-    constexpr int NA = (TILES == 1 && MAXB == 1) ? FQ_GEMV_NA : 1;   // accumulators per (tile, pass, group)
-    int acc[TILES][NP][2][NA][4];
-
-    static_for<0, F>([&](auto JB) {
-        constexpr int jb = decltype(JB)::value;
-        uint4 w[TILES], h[TILES];
-        static_for<0, TILES>([&](auto TLI) {
-            constexpr int tl = decltype(TLI)::value;
-            w[tl] = lds128<tl * F * 512 + jb * 512>(fa);
-            h[tl] = w[tl];                                     // F == 1: classes 4..7 come down by one shift
-            if (F == 1 && MAXB == 1) h[tl] = make_uint4(w[tl].x >> 4, w[tl].y >> 4, w[tl].z >> 4, w[tl].w >> 4);
-        });
-        static_for<0, P>([&](auto TI) {
-            constexpr int t = decltype(TI)::value;
-            constexpr int j = P * jb + t;                      // k32 step inside the superstep
-            constexpr int grp = j >> 2;
-            [[maybe_unused]] constexpr int ai = (j & 3) % NA;
-            constexpr bool first = (j & 3) < NA;               // first link of this accumulator's chain
-            if constexpr (MAXB == 1) {
-                constexpr int tc = (F == 1) ? (t & 3) : t;     // bit-offset class = B column pair
-                constexpr uint32_t m = kMask << (tc * F);
-                const uint2 x = lds64<j * 32>(xa[tc] + xoff);
-#pragma unroll
-                for (int tl = 0; tl < TILES; tl++) {
-                    const uint4& a = (F == 1 && t >= 4) ? h[tl] : w[tl];
-                    if (F == 8) {
-                        if (first) mma_u8s8_first(acc[tl][0][grp][ai], a.x, a.y, a.z, a.w, x.x, x.y);
-                        else mma_u8s8(acc[tl][0][grp][ai], a.x, a.y, a.z, a.w, x.x, x.y);
-                    } else {
-                        if (first) mma_u8s8_first(acc[tl][0][grp][ai], a.x & m, a.y & m, a.z & m, a.w & m, x.x, x.y);
-                        else mma_u8s8(acc[tl][0][grp][ai], a.x & m, a.y & m, a.z & m, a.w & m, x.x, x.y);
-                    }
-                }
-            } else {
-                constexpr int sh = t * F;
-                const uint2 x = lds64<j * 32>(xa[0] + xoff);
-                uint2 x2 = make_uint2(0u, 0u);
-                if (two_pass) x2 = lds64<j * 32>(xa[1] + xoff);
-#pragma unroll
-                for (int tl = 0; tl < TILES; tl++) {
-                    const uint32_t a0 = (w[tl].x >> sh) & kMask, a1 = (w[tl].y >> sh) & kMask;
-                    const uint32_t a2 = (w[tl].z >> sh) & kMask, a3 = (w[tl].w >> sh) & kMask;
-                    if (first) {
-                        mma_u8s8_first(acc[tl][0][grp][0], a0, a1, a2, a3, x.x, x.y);
-                        if (two_pass) mma_u8s8_first(acc[tl][NP - 1][grp][0], a0, a1, a2, a3, x2.x, x2.y);
-                        else if (NP > 1) {
-#pragma unroll
-                            for (int i = 0; i < 4; i++) acc[tl][NP - 1][grp][0][i] = 0;
-                        }
-                    } else {
-                        mma_u8s8(acc[tl][0][grp][0], a0, a1, a2, a3, x.x, x.y);
-                        if (two_pass) mma_u8s8(acc[tl][NP - 1][grp][0], a0, a1, a2, a3, x2.x, x2.y);
-                    }
-                }
-            }
-        });
-    });
-    // digits -> integer, undo the class scaling (exact: every term is a multiple of 2^(c*F)),
-    // apply the field's position inside the code
-    const int down = MAXB == 1 ? c * F : 0;
-#pragma unroll
-    for (int tl = 0; tl < TILES; tl++)
-#pragma unroll
-        for (int p = 0; p < NP; p++)
-#pragma unroll
-            for (int grp = 0; grp < 2; grp++) {
-                int a[4];
-#pragma unroll
-                for (int i = 0; i < 4; i++) {
-                    a[i] = acc[tl][p][grp][0][i];
-#pragma unroll
-                    for (int n = 1; n < NA; n++) a[i] += acc[tl][p][grp][n][i];
-                }
-                const int v0 = ((a[0] + (a[1] << 8)) >> down) << SHIFT, v1 = ((a[2] + (a[3] << 8)) >> down) << SHIFT;
-                if (FIRSTF) { v[tl][p][0][grp] = v0; v[tl][p][1][grp] = v1; }      // the first field starts the sums
-                else { v[tl][p][0][grp] += v0; v[tl][p][1][grp] += v1; }
-            }
-}
-
-// The fields of one superstep, unrolled at compile time from the variant's field list.
-template <int VARIANT, int FI, int PREFIX, int MAXB, int TILES>
-struct FieldLoop {
-    static __device__ __forceinline__ void run(uint32_t fbase, int st_tile, const uint32_t (&xa)[4], uint32_t xoff,
-                                               bool two_pass, int c, int (&v)[TILES][MAXB == 1 ? 1 : 2][2][2])
-    {
-        constexpr FieldList FL = variant_fields(VARIANT);
-        if constexpr (FI < FL.n) {
-            constexpr int F = FL.width[FI], SHIFT = FL.shift[FI], KEEP = FL.keep[FI];
-            // field array of width F after fields adding up to PREFIX bits; tile (superstep, row tile) = st_tile
-            const uint32_t fa = fbase + kBlobSteps * kBlobTiles * 512 * PREFIX + st_tile * (F * 512);
-            field_step<F, KEEP, SHIFT, FI == 0, MAXB, TILES>(fa, xa, xoff, two_pass, c, v);
-            FieldLoop<VARIANT, FI + 1, PREFIX + F, MAXB, TILES>::run(fbase, st_tile, xa, xoff, two_pass, c, v);
-        }
-    }
-};
-
-// All supersteps of one unit for this warp's row tiles: tot[tile][pass][row half] += the dequantised dot products.
-//   st    : shared address of the stage          cnt : supersteps in the unit (whole blobs)
-//   xs    : shared address of the activation slot (digits, group sums, group scales)
-template <int VARIANT, int MAXB, int TILES, class S>
-__device__ __forceinline__ void unit_compute(uint32_t st, int cnt, int blob_read, uint32_t xs, uint32_t zero_page,
-                                             int B, int lane, int tile0, float (&tot)[TILES][MAXB == 1 ? 1 : 2][2])
-{
-    constexpr int NP = MAXB == 1 ? 1 : 2;
-    // a nested child reads the parent's top bits; the dropped bits are filled with their mid-point, which
-    // is the same as lowering every zero point by that amount
-    constexpr int kAdjust = (VARIANT >= 7 && VARIANT < 13) ? 1 << (7 - (VARIANT - 5)) : 0;
-    const int g = lane >> 2, c = lane & 3;
-    const bool two_pass = MAXB > 1 && B > 4;
-    // this lane's B-operand sources.  B column n = g holds digit (g & 1) of
-    //   batch 1: bit-offset class g >> 1            batch > 1: batch entry 4 * pass + (g >> 1)
-    uint32_t xa[4];
-    if (MAXB == 1) {
-#pragma unroll
-        for (int t = 0; t < 4; t++) xa[t] = (g >> 1) == t ? xs + (g & 1) * S::kDigitOff + c * 8 : zero_page + c * 8;
-    } else {
-#pragma unroll
-        for (int p = 0; p < 2; p++) {
-            const int b = 4 * p + (g >> 1);
-            xa[p] = b < B ? xs + b * S::kXRow + (g & 1) * S::kDigitOff + c * 8 : zero_page + c * 8;
-        }
-        xa[2] = xa[3] = zero_page + c * 8;
-    }
-    const uint32_t xsum = xs + S::kXsumOff, xscale = xs + S::kXscaleOff;
-    uint32_t blob = st;
-    for (int s = 0; s < cnt; s += kBlobSteps, blob += blob_read) {
-#ifdef FQ_GEMV_UNROLL_SSL
-#pragma unroll
-#else
-#pragma unroll 1                                                             // (keeps the 14 specialised loops small)
-#endif
-        for (int ssl = 0; ssl < kBlobSteps; ssl++) {
-            const int st_tile = ssl * kBlobTiles + tile0;
-            int v[TILES][NP][2][2];
-            FieldLoop<VARIANT, 0, 0, MAXB, TILES>::run(blob + kBlobMetaBytes + lane * 16, st_tile, xa, (s + ssl) * 256, two_pass, c, v);
-            // group epilogue: y += s * 2^-e * (v - z * sum x_int)
-            const uint32_t meta = blob + st_tile * 128 + g * 16;          // words of (group, row half) at + group * 8 + half * 4
-            if constexpr (MAXB == 1) {
-                // both groups' activation sums and scales in one load each; only the class-0 lane of a quad
-                // subtracts the zero-point term
-                const uint2 xs2 = lds64(xsum + (s + ssl) * 8), sc2 = lds64(xscale + (s + ssl) * 8);
-                const int nx[2] = {c == 0 ? -(int)xs2.x : 0, c == 0 ? -(int)xs2.y : 0};
-                const float sc[2] = {__uint_as_float(sc2.x), __uint_as_float(sc2.y)};
-                static_for<0, TILES * 2>([&](auto I) {
-                    constexpr int tl = decltype(I)::value / 2, grp = decltype(I)::value % 2;
-                    const uint32_t m0 = lds32<tl * 128 + grp * 8>(meta);
-                    const uint32_t m1 = lds32<tl * 128 + grp * 8 + 4>(meta);
-                    const float s0 = __low2float(*reinterpret_cast<const __half2*>(&m0));
-                    const float s1 = __low2float(*reinterpret_cast<const __half2*>(&m1));
-                    // v - (z - adjust) * X  =  v + z * (-X) - adjust * (-X)
-                    const int base = kAdjust ? -kAdjust * nx[grp] : 0;
-                    const int t0 = v[tl][0][0][grp] + (int)(m0 >> 16) * nx[grp] + base;
-                    const int t1 = v[tl][0][1][grp] + (int)(m1 >> 16) * nx[grp] + base;
-                    tot[tl][0][0] = fmaf((float)t0, s0 * sc[grp], tot[tl][0][0]);
-                    tot[tl][0][1] = fmaf((float)t1, s1 * sc[grp], tot[tl][0][1]);
-                });
-            } else {
-#pragma unroll
-                for (int tl = 0; tl < TILES; tl++) {
-#pragma unroll
-                    for (int grp = 0; grp < 2; grp++) {
-                        const uint32_t m0 = lds32(meta + tl * 128 + grp * 8);
-                        const uint32_t m1 = lds32(meta + tl * 128 + grp * 8 + 4);
-                        const float s0 = __low2float(*reinterpret_cast<const __half2*>(&m0));
-                        const float s1 = __low2float(*reinterpret_cast<const __half2*>(&m1));
-                        const int z0 = (int)(m0 >> 16) - kAdjust;
-                        const int z1 = (int)(m1 >> 16) - kAdjust;
-#pragma unroll
-                        for (int p = 0; p < NP; p++) {
-                            const int b = 4 * p + c;
-                            const bool has = b < B;
-                            const uint32_t gi = (uint32_t)(b * (S::kCMax * 2) + (s + ssl) * 2 + grp) * 4u;
-                            const int xsm = has ? (int)lds32(xsum + gi) : 0;
-                            const float scb = has ? __uint_as_float(lds32(xscale + gi)) : 0.f;
-                            tot[tl][p][0] = fmaf((float)(v[tl][p][0][grp] - z0 * xsm), s0 * scb, tot[tl][p][0]);
-                            tot[tl][p][1] = fmaf((float)(v[tl][p][1][grp] - z1 * xsm), s1 * scb, tot[tl][p][1]);
-                        }
-                    }
-                }
-            }
-        }
-    }
-}
-
-template <int MAXB, int TILES, class S>
-__device__ __forceinline__ void unit_dispatch(int variant, uint32_t st, int cnt, int blob_read, uint32_t xs, uint32_t zero_page,
-                                              int B, int lane, int tile0, float (&tot)[TILES][MAXB == 1 ? 1 : 2][2])
-{
-#define FQ_VARIANT_CASE(V) case V: unit_compute<V, MAXB, TILES, S>(st, cnt, blob_read, xs, zero_page, B, lane, tile0, tot); break;
-    switch (variant) {
-        FQ_VARIANT_CASE(0) FQ_VARIANT_CASE(1) FQ_VARIANT_CASE(2) FQ_VARIANT_CASE(3) FQ_VARIANT_CASE(4)
-        FQ_VARIANT_CASE(5) FQ_VARIANT_CASE(6) FQ_VARIANT_CASE(7) FQ_VARIANT_CASE(8) FQ_VARIANT_CASE(9)
-        FQ_VARIANT_CASE(10) FQ_VARIANT_CASE(11) FQ_VARIANT_CASE(12) FQ_VARIANT_CASE(13)
-        default: break;
-    }
-#undef FQ_VARIANT_CASE
-    static_assert(kVariants == 14, "one case per variant");
-}
-
-template <int MAXB>
+template <int BP>
 __global__ void __launch_bounds__(kGemvThreads, 1)
 gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
 {
-    using S = GemvSmem<MAXB>;
-    constexpr int NP = MAXB == 1 ? 1 : 2;
+    using S = GemvSmem<BP>;
     extern __shared__ __align__(1024) uint8_t smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t bars = smem_u32(smem + S::oBars);                          // full[0..S), empty[0..S)
@@ -469,10 +163,9 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
     const uint32_t xbars = smem_u32(smem + S::oXBars);                         // completes a phase per publication of a slot
     volatile int* x_pending = x_ready + kXSlots;                               // units that still need the slot
     volatile int* flags = x_pending + kXSlots;                                 // [0]: stop computing, [1]: stop everything
-    volatile int* prep_cmd = flags + 2;                                        // decision shared by the pre-processing warps
     volatile unsigned* out_fill = reinterpret_cast<volatile unsigned*>(smem + S::oOutCtl);   // consumer warps that filled a slot
-    volatile unsigned* out_gen = out_fill + S::kOutSlots;                         // times the output warp drained a slot
-    volatile int* out_total = reinterpret_cast<volatile int*>(out_gen + S::kOutSlots);   // finishing units of this CTA (-1: not known yet)
+    volatile unsigned* out_gen = out_fill + kOutSlots;                         // times the output warp drained a slot
+    volatile int* out_total = reinterpret_cast<volatile int*>(out_gen + kOutSlots);   // finishing units of this CTA (-1: not known yet)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S::kStages; s++) {
@@ -481,14 +174,12 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
             released[s] = 0u;
         }
         for (int i = 0; i < kXSlots; i++) { x_ready[i] = 0; x_pending[i] = 0; mbar_init(xbars + 8 * i, 1); }
-        for (int i = 0; i < S::kOutSlots; i++) { out_fill[i] = 0u; out_gen[i] = 0u; }
+        for (int i = 0; i < kOutSlots; i++) { out_fill[i] = 0u; out_gen[i] = 0u; }
         out_total[0] = -1;
         flags[0] = 0; flags[1] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    for (int i = threadIdx.x; i < S::kZeroBytes / 4; i += blockDim.x)
-        reinterpret_cast<uint32_t*>(smem + S::oZero)[i] = 0u;
     __syncthreads();
 
     const int grid = gridDim.x, cta = blockIdx.x;
@@ -595,13 +286,12 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
             fetch.store(&opbuf[(oi + 1) & 1], lane);
             __syncwarp();
         }
-        if (lane == 0 && !stop) out_total[0] = oseq;                // the output warp may leave after this many
-    } else if (warp >= kPrepWarp && warp < kPrepWarp + kPrepWarps) {
-        // ================================================================== activation pre-processing
-        // All pre-processing warps walk the same list of (op, K chunk) segments and split the
-        // (batch row, superstep) items of each segment among them; named barrier 1 keeps them in step.
-        const int pw = warp - kPrepWarp;
-        GemvOp* opbuf = reinterpret_cast<GemvOp*>(smem + S::oOpBuf) + 2 + 2 * pw;
+        if (lane == 0 && !stop) out_total[0] = oseq;                // the output warps may leave after this many
+    } else if (warp == kActWarp) {
+        // ================================================================== activations
+        // One (op, K chunk) segment after the other: wait until a slot is free and the phase that produces the activations is
+        // complete, then one bulk copy per batch row; the consumers sleep on the slot's barrier.
+        GemvOp* opbuf = reinterpret_cast<GemvOp*>(smem + S::oOpBuf) + 2;
         OpFetch fetch;
         fetch.issue(ops, 0, sa.n_ops, lane);
         fetch.store(&opbuf[0], lane);
@@ -625,8 +315,9 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                 seg++;
                 const int units = min(hi, (ch + 1) * op.n_rp) - max(lo, ch * op.n_rp);
                 const int slot = seg % kXSlots;
-                uint8_t* xs = smem + S::oX + slot * S::kXSlotBytes;
-                if (pw == 0 && lane == 0) {
+                const uint32_t xs = smem_u32(smem + S::oX) + (uint32_t)slot * S::kXSlotBytes, bar = xbars + 8 * slot;
+                int go = 1;                                            // 0: stop, 1: fetch, 2: publish without fetching
+                if (lane == 0) {
                     // the slot is free when every unit of the segment that used it before is done
                     if (!smem_wait([&] { return x_pending[slot] == 0 || flags[1]; })) {
                         atomicCAS(sa.status, 0, FQ_ERR_TIMEOUT); flags[0] = 1; flags[1] = 1;
@@ -642,105 +333,51 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                                  flags[0])) { atomicCAS(sa.status, 0, FQ_ERR_TIMEOUT); flags[0] = 1; break; }
                         }
                     }
-                    prep_cmd[0] = flags[1] ? 0 : (flags[0] ? 2 : 1);   // one decision for all pre-processing warps
+                    // other SMs' plain stores (y of the previous phase) and this SM's reads of the slot before the copies below
                     __threadfence_block();
+                    asm volatile("fence.proxy.async;" ::: "memory");
+                    go = flags[1] ? 0 : (flags[0] ? 2 : 1);
                 }
-                asm volatile("bar.sync 1, %0;" ::"n"(kPrepWarps * 32) : "memory");
-                const int go = prep_cmd[0];                            // 0: stop, 1: compute, 2: publish without computing
+                go = __shfl_sync(0xffffffffu, go, 0);
                 if (op.phase > 0) phase_known = op.phase - 1;          // (meaningless after an abort; unused then)
                 if (go == 0) { stop = true; break; }
-                if (go == 1) {
-                    const int ss0 = ch * op.chunk_blobs * kBlobSteps;
-                    const int cnt = min(op.chunk_blobs, op.n_kb - ch * op.chunk_blobs) * kBlobSteps;
-                    int* xsum = reinterpret_cast<int*>(xs + S::kXsumOff);
-                    float* xscale = reinterpret_cast<float*>(xs + S::kXscaleOff);
-                    const int n_items = cnt * op.batch;                // item = (batch row, superstep)
-                    for (int i0 = pw; i0 < n_items; i0 += 4 * kPrepWarps) {
-                        uint4 raw[4];                                  // all loads of up to four items first
-#pragma unroll
-                        for (int q = 0; q < 4; q++) {
-                            raw[q] = make_uint4(0u, 0u, 0u, 0u);
-                            const int item = i0 + q * kPrepWarps;
-                            if (item < n_items) {
-                                const int b = item / cnt, s_ = item % cnt;
-                                const int k = (ss0 + s_) * kStepCols + lane * 8;   // this lane: 8 columns of the superstep
-                                if (k < op.k_in)
-                                    raw[q] = __ldcg(reinterpret_cast<const uint4*>(
-                                        reinterpret_cast<const __half*>(op.x) + (long long)b * op.k_in + k));
-                            }
-                        }
-#pragma unroll
-                        for (int q = 0; q < 4; q++) {
-                            const int item = i0 + q * kPrepWarps;
-                            if (item >= n_items) break;
-                            const int b = item / cnt, s_ = item % cnt;
-                            const __half2* h2 = reinterpret_cast<const __half2*>(&raw[q]);
-                            float f[8];
-#pragma unroll
-                            for (int i = 0; i < 4; i++) {
-                                const float2 t2 = __half22float2(h2[i]);
-                                f[2 * i] = t2.x; f[2 * i + 1] = t2.y;
-                            }
-                            float amax = 0.f;
-#pragma unroll
-                            for (int i = 0; i < 8; i++) amax = fmaxf(amax, fabsf(f[i]));
-#pragma unroll
-                            for (int o = 8; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-                            // group of 128 columns = 16 lanes.  x_int = rint(x * 2^(13 - E)), 2^E <= amax < 2^(E+1)
-                            const int eb = (__float_as_int(amax) >> 23) & 0xff;       // biased exponent of amax
-                            const bool fin = amax > 0.f && eb < 255;
-                            const float mult = fin ? __int_as_float((267 - eb) << 23) : 0.f;
-                            const float back = fin ? __int_as_float((eb - 13) << 23) : 0.f;
-                            int xi[8], sum = 0;
-#pragma unroll
-                            for (int i = 0; i < 8; i++) { xi[i] = __float2int_rn(f[i] * mult); sum += xi[i]; }
-#pragma unroll
-                            for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-                            // signed digits base 256 of four values at a time: low byte as is, high byte + carry
-                            uint32_t lo4[2], hi4[2];
-#pragma unroll
-                            for (int r = 0; r < 2; r++) {
-                                const uint32_t p01 = __byte_perm((uint32_t)xi[4 * r + 0], (uint32_t)xi[4 * r + 1], 0x5410);
-                                const uint32_t p23 = __byte_perm((uint32_t)xi[4 * r + 2], (uint32_t)xi[4 * r + 3], 0x5410);
-                                const uint32_t h01 = (((p01 >> 8) & 0x00ff00ffu) + ((p01 >> 7) & 0x00010001u)) & 0x00ff00ffu;
-                                const uint32_t h23 = (((p23 >> 8) & 0x00ff00ffu) + ((p23 >> 7) & 0x00010001u)) & 0x00ff00ffu;
-                                lo4[r] = __byte_perm(p01, p23, 0x6420);
-                                hi4[r] = __byte_perm(h01, h23, 0x6420);
-                            }
-                            // B-fragment order: per k32 step 32 bytes = [c][k 4c..4c+3 | k 16+4c..16+4c+3]
-                            const int j = lane >> 2, q4 = lane & 3;
-                            const int half = q4 >> 1, c0 = 2 * (q4 & 1);
-                            uint8_t* row = xs + b * S::kXRow + s_ * 256 + j * 32 + half * 4;
-                            *reinterpret_cast<uint32_t*>(row + c0 * 8) = lo4[0];
-                            *reinterpret_cast<uint32_t*>(row + (c0 + 1) * 8) = lo4[1];
-                            *reinterpret_cast<uint32_t*>(row + S::kDigitOff + c0 * 8) = hi4[0];
-                            *reinterpret_cast<uint32_t*>(row + S::kDigitOff + (c0 + 1) * 8) = hi4[1];
-                            if ((lane & 15) == 0) {
-                                xsum[b * (S::kCMax * 2) + s_ * 2 + (lane >> 4)] = sum;
-                                xscale[b * (S::kCMax * 2) + s_ * 2 + (lane >> 4)] = back;
-                            }
-                        }
+                const int k0 = ch * op.chunk_blobs * (kBlobSteps * kStepCols);
+                const int cols = min(op.chunk_blobs * (kBlobSteps * kStepCols), op.n_kb * (kBlobSteps * kStepCols) - k0);
+                const int have = min(cols, op.k_in - k0);              // (a multiple of 128, at least 128)
+                // columns beyond k_in have weights of zero: their activations must be numbers
+                if (have < cols)
+                    for (int i = lane; i < op.batch * ((cols - have) / 8); i += 32) {
+                        const int b = i / ((cols - have) / 8), k = have + i % ((cols - have) / 8) * 8;
+                        sts128(xs + (uint32_t)(b * kXRowBytes + k * 2), make_uint4(0u, 0u, 0u, 0u));
                     }
-                }
                 __threadfence_block();
-                asm volatile("bar.sync 1, %0;" ::"n"(kPrepWarps * 32) : "memory");
-                if (pw == 0 && lane == 0) {
+                __syncwarp();
+                if (lane == 0) {
                     x_pending[slot] = units * kWarpsPerUnit;
                     __threadfence_block();
                     x_ready[slot] = seg + 1;
                     __threadfence_block();
-                    mbar_arrive(xbars + 8 * slot);                     // wakes the consumers that sleep on this slot
+                    if (go == 1) mbar_expect_tx(bar, (uint32_t)(op.batch * have * 2));
+                    else mbar_arrive(bar);
                 }
+                __syncwarp();
+                if (go == 1 && lane < op.batch && FQ_IN_BOUNDS(k0 + have <= op.k_in && have <= kXCols, sa.status))
+                    bulk_g2s(xs + (uint32_t)(lane * kXRowBytes), reinterpret_cast<const __half*>(op.x) + (long long)lane * op.k_in + k0,
+                             (uint32_t)have * 2u, bar);
             }
         }
-    } else if (warp == kOutputWarp) {
-        // ================================================================== output warp
+        // copies that are still in flight land before the CTA may exit (their units wait for them unless the kernel is aborting)
+        if (lane == 0 && flags[1])
+            for (int i = max(0, seg + 1 - kXSlots); i <= seg; i++)
+                if (x_ready[i % kXSlots] == i + 1) mbar_wait(xbars + 8 * (i % kXSlots), (unsigned)(i / kXSlots) & 1u, 1000000ull);
+    } else if (warp >= kOutputWarp) {
+        // ================================================================== output warps
         // Finishes row pairs.  The unit whose K chunk is (row pair mod chunks) adds up its row pair: its own
         // sums arrive through the queue in shared memory, the other chunks' sums are tagged 64-bit words in
         // global memory (value, launch tag) that their consumers stored without any fence -- a word counts
         // once its tag is this launch's.  The sums are added in chunk order, so results do not depend on
         // timing.  One fence per batch of finished row pairs orders y before the phase counter.
-        constexpr int BW = MAXB == 1 ? 1 : 8;                            // result floats per row
+        const int ow = warp - kOutputWarp;                               // takes the places congruent to ow
         const float* odata = reinterpret_cast<const float*>(smem + S::oOutData);
         const OutDesc* odesc = reinterpret_cast<const OutDesc*>(smem + S::oOutDesc);
         int processed = 0;
@@ -748,7 +385,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
         unsigned idle_it = 0u;
         for (;;) {
             // every decision that ends the loop is taken by lane 0 and broadcast: the lanes must leave together
-            const bool filled = lane < S::kOutSlots && out_fill[lane] == (unsigned)kWarpsPerUnit;
+            const bool filled = lane < kOutSlots && lane % kOutputWarps == ow && out_fill[lane] == (unsigned)kWarpsPerUnit;
             const unsigned m = __ballot_sync(0xffffffffu, filled);
             unsigned done = 0u;
             if (m) {
@@ -757,48 +394,50 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                     const int s = __ffs(mm) - 1;
                     const OutDesc& d = odesc[s];
                     const float* o = odata + s * S::kOutFloats;
-                    // a few chunks per round trip, every batch entry of them in flight at once; a round whose
-                    // words are not all there ends the attempt
-                    constexpr int QS = MAXB == 1 ? 24 : 2;
-                    float sum[BW];
+                    // lane = row; a few chunks per round trip, every batch entry of them in flight at once; a round
+                    // whose words are not all there ends the attempt
+                    constexpr int QS = 16 / BP;
+                    float sum[BP];
 #pragma unroll
-                    for (int i = 0; i < BW; i++) sum[i] = 0.f;
+                    for (int i = 0; i < BP; i++) sum[i] = 0.f;
                     bool ok = true;
-                    const unsigned long long* pt = d.partial + (long long)d.rp * d.n_chunks * (32 * BW) + lane;
+                    const unsigned long long* pt = d.partial + (long long)d.rp * d.n_chunks * (32 * BP) + lane * BP;
                     for (int q0 = 0; q0 < d.n_chunks; q0 += QS) {
-                        unsigned long long w[QS][BW];
+                        ulonglong2 w[QS][BP / 2];
 #pragma unroll
                         for (int j = 0; j < QS; j++) {
                             const int q = q0 + j;
 #pragma unroll
-                            for (int i = 0; i < BW; i++) {                // element e = lane + 32 i = local row * BW + batch entry
-                                w[j][i] = 0ull;
-                                if (q < d.n_chunks && q != d.ch) w[j][i] = ld_relaxed_u64(pt + (long long)q * (32 * BW) + 32 * i);
+                            for (int i = 0; i < BP / 2; i++) {
+                                w[j][i] = make_ulonglong2(0ull, 0ull);
+                                if (q < d.n_chunks && q != d.ch) w[j][i] = ld_relaxed_u64x2(pt + (long long)q * (32 * BP) + 2 * i);
                             }
                         }
 #pragma unroll
                         for (int j = 0; j < QS; j++) {
                             const int q = q0 + j;
                             if (q >= d.n_chunks) break;
+                            if (q == d.ch) {
 #pragma unroll
-                            for (int i = 0; i < BW; i++) {
-                                if (q == d.ch) sum[i] += o[lane + 32 * i];
-                                else {
-                                    ok = ok && (unsigned)(w[j][i] >> 32) == sa.epoch;
-                                    sum[i] += __uint_as_float((unsigned)w[j][i]);
+                                for (int i = 0; i < BP; i++) sum[i] += o[lane * BP + i];
+                            } else {
+#pragma unroll
+                                for (int i = 0; i < BP / 2; i++) {
+                                    ok = ok && (unsigned)(w[j][i].x >> 32) == sa.epoch && (unsigned)(w[j][i].y >> 32) == sa.epoch;
+                                    sum[2 * i] += __uint_as_float((unsigned)w[j][i].x);
+                                    sum[2 * i + 1] += __uint_as_float((unsigned)w[j][i].y);
                                 }
                             }
                         }
                         if (!__all_sync(0xffffffffu, ok)) break;
                     }
                     if (!__all_sync(0xffffffffu, ok)) continue;          // some chunk has not arrived yet: look again later
-                    const int row_base = d.rp * (kUnitRowTiles * kTileRows);
+                    const int row = d.rp * (kUnitRowTiles * kTileRows) + lane;
                     __half* y = reinterpret_cast<__half*>(d.y);
+                    if (row < d.n_out) {
 #pragma unroll
-                    for (int i = 0; i < BW; i++) {
-                        const int e = lane + 32 * i;
-                        const int row = row_base + e / BW, b = e % BW;
-                        if (row < d.n_out && b < d.batch) y[(long long)b * d.n_out + row] = __float2half_rn(sum[i]);
+                        for (int b = 0; b < BP; b++)
+                            if (b < d.batch) y[(long long)b * d.n_out + row] = __float2half_rn(sum[b]);
                     }
                     done |= 1u << s;
                 }
@@ -820,7 +459,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
             int leave = 0;
             if (lane == 0) {
                 const int want = out_total[0];
-                if (flags[0] || (want >= 0 && processed >= want)) leave = 1;
+                if (flags[0] || (want >= 0 && processed >= (want + kOutputWarps - 1 - ow) / kOutputWarps)) leave = 1;
                 else if ((++idle_it & 127u) == 0u) {
                     const unsigned long long now = global_ns();
                     if (last_progress == 0ull) last_progress = now;
@@ -835,11 +474,10 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
         }
     } else {
         // ================================================================== consumers
-        // kWarpsPerUnit warps share a unit, each computes kTilesPerWarp of its two 16-row tiles.
+        // Two warps share a unit, each computes one of its two 16-row tiles.
         const int g = lane >> 2, c = lane & 3;
         const int uidx = warp / kWarpsPerUnit;                       // which of the units in flight
-        const int tile0 = (warp % kWarpsPerUnit) * kTilesPerWarp;    // first row tile of this warp
-        constexpr int TL = kTilesPerWarp;
+        const int tile = warp % kWarpsPerUnit;                       // this warp's row tile
         int total = 0;                               // units of this CTA over the whole launch
         if (sa.cta_units) total = sa.cta_units[cta];
         else {
@@ -882,16 +520,16 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
             }
             // a unit that finishes its row pair needs a place in the output queue: that place must be free
             // again; the descriptor goes there now, while the op's slot in the op ring is certainly still valid
-            const int oslot = d.oseq % S::kOutSlots;
+            const int oslot = d.oseq % kOutSlots;
             if (d.oseq >= 0) {
-                const unsigned ogen = (unsigned)(d.oseq / S::kOutSlots);
+                const unsigned ogen = (unsigned)(d.oseq / kOutSlots);
                 if (!smem_wait([&] { return out_gen[oslot] == ogen || flags[1]; })) {
                     if (lane == 0) { atomicCAS(sa.status, 0, FQ_ERR_TIMEOUT); flags[0] = 1; flags[1] = 1; }
                     stop = true;
                     break;
                 }
                 if (flags[1]) { stop = true; break; }
-                if (tile0 == 0 && lane == 0) {
+                if (tile == 0 && lane == 0) {
                     const GemvOp& od = *reinterpret_cast<const GemvOp*>(opring + d.op_slot * S::kOpBytes);
                     OutDesc& q = odesc[oslot];
                     q.rp = d.rp; q.ch = d.ch; q.n_chunks = od.n_chunks; q.n_out = od.n_out; q.phase = od.phase; q.batch = od.batch;
@@ -900,24 +538,21 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
             }
             const int slot = d.seg % kXSlots;
             // sleep on the slot's barrier (a hardware wake-up: this wait is on the critical path of every
-            // dependency phase); the flag has the last word, because a warp that is several publications
-            // ahead would read a stale parity
-            if (x_ready[slot] != d.seg + 1 && !flags[1]) mbar_wait(xbars + 8 * slot, (unsigned)(d.seg / kXSlots) & 1u);
-            if (!smem_wait([&] { return x_ready[slot] == d.seg + 1 || flags[1]; })) {
+            // dependency phase); a warp that is several publications ahead would read a stale parity, so only a barrier that
+            // belongs to this segment counts
+            const unsigned xpar = (unsigned)(d.seg / kXSlots) & 1u;
+            if (x_ready[slot] != d.seg + 1 && !flags[1]) mbar_wait(xbars + 8 * slot, xpar);
+            if (!smem_wait([&] { return x_ready[slot] == d.seg + 1 || flags[1]; }) || (!flags[1] && !mbar_wait(xbars + 8 * slot, xpar))) {
                 if (lane == 0) { atomicCAS(sa.status, 0, FQ_ERR_TIMEOUT); flags[0] = 1; }
             }
             __threadfence_block();
             __syncwarp();
             const bool live = !flags[0];
 
-            float tot[TL][NP][2];
-#pragma unroll
-            for (int i = 0; i < TL * NP * 2; i++) (&tot[0][0][0])[i] = 0.f;
-
+            float tot[4] = {0.f, 0.f, 0.f, 0.f};
             if (live)
-                unit_dispatch<MAXB, TL, S>(d.variant, smem_u32(smem + S::oStages) + (uint32_t)stage * S::kStageBytes, d.cnt,
-                                           d.blob_read, smem_u32(smem + S::oX) + (uint32_t)slot * S::kXSlotBytes,
-                                           smem_u32(smem + S::oZero), d.batch, lane, tile0, tot);
+                unit_dispatch<BP>(d.variant, smem_u32(smem + S::oStages) + (uint32_t)stage * S::kStageBytes, d.cnt, (uint32_t)d.blob_read,
+                                  smem_u32(smem + S::oX) + (uint32_t)slot * S::kXSlotBytes, lane, tile, tot);
             __syncwarp();
             if (lane == 0) {
                 atomicAdd(const_cast<unsigned*>(&released[stage]), 1u);
@@ -929,58 +564,24 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
             while (stage >= S::kStages) { stage -= S::kStages; use++; }
             if (!live) continue;
 
-            if (MAXB == 1) {                                     // add up the bit-offset classes held by the quad
-#pragma unroll
-                for (int tl = 0; tl < TL; tl++)
-#pragma unroll
-                    for (int r = 0; r < 2; r++) {
-                        float t = tot[tl][0][r];
-                        t += __shfl_xor_sync(0xffffffffu, t, 1);
-                        t += __shfl_xor_sync(0xffffffffu, t, 2);
-                        tot[tl][0][r] = t;
-                    }
-            }
-
-            // ---- the row sums: value (tile, pass, r) of lane (g, c) belongs to local row tile * 16 + g + 8 r,
-            //      batch entry 0 (batch 1: every lane of the quad holds it) or 4 pass + c
-            constexpr int BW = MAXB == 1 ? 1 : 8;
+            // ---- the row sums: tot[2 r + i] of lane (g, c) belongs to local row tile * 16 + g + 8 r, batch entry 2 c + i
+            const int lr = tile * kTileRows + g;
             if (d.oseq >= 0) {
-                // this unit finishes its row pair: hand the sums to the output warp
+                // this unit finishes its row pair: hand the sums to the output warps
                 float* o = odata + oslot * S::kOutFloats;
-#pragma unroll
-                for (int tl = 0; tl < TL; tl++)
-#pragma unroll
-                    for (int p = 0; p < NP; p++)
-#pragma unroll
-                        for (int r = 0; r < 2; r++) {
-                            const int lr = (tile0 + tl) * 16 + g + 8 * r;
-                            if (MAXB == 1) { if (c == 0) o[lr] = tot[tl][0][r]; }
-                            else o[lr * BW + 4 * p + c] = tot[tl][p][r];
-                        }
+                if (2 * c < BP) {
+                    *reinterpret_cast<float2*>(o + lr * BP + 2 * c) = make_float2(tot[0], tot[1]);
+                    *reinterpret_cast<float2*>(o + (lr + 8) * BP + 2 * c) = make_float2(tot[2], tot[3]);
+                }
                 __threadfence_block();
                 __syncwarp();
                 if (lane == 0) atomicAdd(const_cast<unsigned*>(&out_fill[oslot]), 1u);
-            } else {
+            } else if (2 * c < BP) {
                 // another unit finishes it: publish tagged words (value, launch tag), fire and forget
-                unsigned long long* pu = d.partial + ((long long)d.rp * d.n_chunks + d.ch) * (32 * BW);
+                unsigned long long* pu = d.partial + ((long long)d.rp * d.n_chunks + d.ch) * (32 * BP) + lr * BP + 2 * c;
                 const unsigned long long tag = (unsigned long long)sa.epoch << 32;
-#pragma unroll
-                for (int tl = 0; tl < TL; tl++) {
-                    if (MAXB == 1) {
-                        if (c < 2) {                                 // lane c of the quad stores row g + 8 c
-                            const float v = c == 0 ? tot[tl][0][0] : tot[tl][0][1];
-                            st_relaxed_u64(pu + (tile0 + tl) * 16 + g + 8 * c, tag | __float_as_uint(v));
-                        }
-                    } else {
-#pragma unroll
-                        for (int p = 0; p < NP; p++)
-#pragma unroll
-                            for (int r = 0; r < 2; r++) {
-                                const int lr = (tile0 + tl) * 16 + g + 8 * r;
-                                st_relaxed_u64(pu + lr * BW + 4 * p + c, tag | __float_as_uint(tot[tl][p][r]));
-                            }
-                    }
-                }
+                st_relaxed_u64x2(pu, tag | __float_as_uint(tot[0]), tag | __float_as_uint(tot[1]));
+                st_relaxed_u64x2(pu + 8 * BP, tag | __float_as_uint(tot[2]), tag | __float_as_uint(tot[3]));
             }
         }
     }
@@ -1000,20 +601,20 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
 // ------------------------------------------------------------------------------- launchers
 // The launch is always cooperative: a CTA that finishes a row pair waits (bounded) for sums that other
 // CTAs produce, so all CTAs of the grid have to be resident together.
-template <int MAXB>
+template <int BP>
 static int launch_impl(Ctx* ctx, const GemvOp& single, const StackArgs& sa, long long total_units, cudaStream_t st)
 {
-    using S = GemvSmem<MAXB>;
+    using S = GemvSmem<BP>;
     static bool configured[64] = {};
     if (ctx->device < 64 && !configured[ctx->device]) {
-        FQ_CUDA_OK(cudaFuncSetAttribute(gemv_kernel<MAXB>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kTotal));
+        FQ_CUDA_OK(cudaFuncSetAttribute(gemv_kernel<BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kTotal));
         configured[ctx->device] = true;
     }
     long long blocks = ctx->sm_count;
     if (total_units < blocks) blocks = total_units;
     if (blocks < 1) return FQ_OK;
     void* args[] = {(void*)&single, (void*)&sa};
-    FQ_CUDA_OK(cudaLaunchCooperativeKernel((const void*)gemv_kernel<MAXB>, dim3((unsigned)blocks), dim3(kGemvThreads),
+    FQ_CUDA_OK(cudaLaunchCooperativeKernel((const void*)gemv_kernel<BP>, dim3((unsigned)blocks), dim3(kGemvThreads),
                                            args, S::kTotal, st));
     return FQ_OK;
 }
@@ -1034,7 +635,7 @@ int launch_gemv_single(Ctx* ctx, const GemvOp& op, cudaStream_t st)
     sa.n_phases = 0;
     sa.epoch = next_epoch(ctx->launch_epoch);
     const long long units = (long long)op.n_rp * op.n_chunks;
-    return launch_impl<8>(ctx, op, sa, units, st);
+    return batch_pad(op.batch) == 4 ? launch_impl<4>(ctx, op, sa, units, st) : launch_impl<8>(ctx, op, sa, units, st);
 }
 
 int launch_gemv_stack(Ctx* ctx, const StackHeader& hdr, const char* table_dev, int max_batch, cudaStream_t st)
@@ -1051,8 +652,7 @@ int launch_gemv_stack(Ctx* ctx, const StackHeader& hdr, const char* table_dev, i
     sa.n_phases = hdr.n_phases;
     sa.epoch = next_epoch(ctx->launch_epoch);
     GemvOp dummy{};
-    (void)max_batch;
-    return launch_impl<8>(ctx, dummy, sa, hdr.total_units, st);
+    return batch_pad(max_batch) == 4 ? launch_impl<4>(ctx, dummy, sa, hdr.total_units, st) : launch_impl<8>(ctx, dummy, sa, hdr.total_units, st);
 }
 
 }  // namespace fq

@@ -135,11 +135,6 @@ __device__ __forceinline__ void prefetch_ops(const GemvOp* ops, int oi, int n_op
         asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
     }
 }
-__device__ __forceinline__ void sts128(uint32_t a, uint4 v)
-{
-    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
-
 // The strips of one op for one CTA: rp_first .. rp_last; the first starts at blob c_first, the last ends
 // before blob c_last (see cta_work).  Packed into two words per (CTA, op) by the host for a stack call.
 constexpr uint32_t kRangeEmpty = 0xffffffffu;

@@ -13,45 +13,10 @@
 #pragma once
 #include <cuda_fp16.h>
 
-#include <type_traits>
-
 #include "fq_layout.cuh"
+#include "fq_ptx.cuh"
 
 namespace fq {
-
-// ------------------------------------------------------------------------------- shared-memory loads
-// Shared memory is addressed with 32-bit shared-window addresses and explicit ld.shared; OFF is a
-// compile-time byte offset that goes into the instruction's address field.
-template <int OFF = 0>
-__device__ __forceinline__ uint4 lds128(uint32_t a)
-{
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4+%5];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a), "n"(OFF));
-    return v;
-}
-template <int OFF = 0>
-__device__ __forceinline__ uint2 lds64(uint32_t a)
-{
-    uint2 v;
-    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2+%3];" : "=r"(v.x), "=r"(v.y) : "r"(a), "n"(OFF));
-    return v;
-}
-template <int OFF = 0>
-__device__ __forceinline__ uint32_t lds32(uint32_t a)
-{
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(a), "n"(OFF));
-    return v;
-}
-// Loop whose index is a compile-time constant in the body (so that it can be a load's immediate offset).
-template <int I, int N, class Fn>
-__device__ __forceinline__ void static_for(Fn&& fn)
-{
-    if constexpr (I < N) {
-        fn(std::integral_constant<int, I>{});
-        static_for<I + 1, N>(fn);
-    }
-}
 
 // D = A(u8, 16x32, row) * B(s8, 32x8, col) + C, s32.  Not volatile: a pure function of its registers,
 // the compiler may interleave independent chains.

@@ -125,7 +125,7 @@ int current_sm_count();
 int launch_stream_read(const void* src, size_t bytes, unsigned* sink, int sm_count, cudaStream_t st);
 
 // Chunking policy of the decode kernel: k blobs (512 columns) per K chunk.
-int gemv_chunk_blobs(int bits, int batch);
+int gemv_chunk_blobs(int bits);
 size_t gemv_partial_bytes_per_unit(int batch);
 int launch_gemv_single(Ctx* ctx, const GemvOp& op, cudaStream_t st);                 // batch 2..8
 int launch_gemm_fused(Ctx* ctx, const void* store, int blob_stride, const FieldList& fl, int zero_adjust, int n_out, int k_in,
