@@ -121,6 +121,23 @@ size_t layer_partial_bytes(int n_out, int k_in)
 
 namespace fq {
 
+// Status word, and behind it the prefill's counters and slots (29 MB): an allocation costs about 0.4 ms whatever its size, and
+// the first prompt of a context should not pay for one.  Without that much memory prefill keeps its tiles whole.
+static bool allocate_status(Ctx* ctx)
+{
+    constexpr size_t kHead = 256;
+    const size_t counts = gemm_split_flag_bytes(ctx->sm_count);
+    char* p = nullptr;
+    if (cudaMalloc(&p, kHead + counts + gemm_split_part_bytes(ctx->sm_count)) == cudaSuccess) {
+        ctx->fused_ws = p + kHead;
+    } else {
+        cudaGetLastError();
+        if (cudaMalloc(&p, kHead) != cudaSuccess) return false;
+    }
+    ctx->status_dev = reinterpret_cast<int*>(p);
+    return cudaMemset(p, 0, kHead + (ctx->fused_ws ? counts : 0)) == cudaSuccess;
+}
+
 int ensure_workspace(Ctx* ctx, size_t bytes)
 {
     if (bytes <= ctx->ws_bytes) return FQ_OK;
@@ -175,8 +192,7 @@ int fq_create(fq_ctx** out, int device, int n_layers)
     ctx->device = device;
     ctx->layers.resize(n_layers);
     if (cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
-        cudaMalloc(&ctx->status_dev, sizeof(int)) != cudaSuccess ||
-        cudaMemset(ctx->status_dev, 0, sizeof(int)) != cudaSuccess ||
+        !allocate_status(ctx) ||
         ensure_workspace(ctx, kPartialBase + (1 << 20)) != FQ_OK) {
         if (ctx->status_dev) cudaFree(ctx->status_dev);
         delete ctx;
@@ -200,7 +216,6 @@ int fq_destroy(fq_ctx* ctx)
             if (ctx->stage_done[i]) cudaEventDestroy(ctx->stage_done[i]);
         }
         if (ctx->gemm_ws) cudaFree(ctx->gemm_ws);
-        if (ctx->fused_ws) cudaFree(ctx->fused_ws);
         for (void* p : ctx->owned) cudaFree(p);
         for (Layer& L : ctx->layers)
             for (Variant& v : L.var)
@@ -582,6 +597,7 @@ int fq_status(fq_ctx* ctx)
         // counters may have been left half-way: start from a clean workspace
         FQ_CUDA_OK(cudaMemset(ctx->status_dev, 0, sizeof(int)));
         FQ_CUDA_OK(cudaMemset(ctx->ws, 0, ctx->ws_bytes));
+        if (ctx->fused_ws) FQ_CUDA_OK(cudaMemset(ctx->fused_ws, 0, gemm_split_flag_bytes(ctx->sm_count)));
         FQ_CUDA_OK(cudaDeviceSynchronize());
     }
     return st;
@@ -810,6 +826,32 @@ int fq_gemv_stack(fq_ctx* ctx, int n_ops, const int* layers_host, const uint16_t
                       : launch_gemv_stack(ctx, ctx->stack_hdr, ctx->stack_dev, batch, st);
 }
 
+static bool may_allocate(cudaStream_t st)
+{
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone) return true;
+    cudaGetLastError();
+    return false;
+}
+
+// Room for the bf16 copy of one layer; the first call asks for that of the largest layer of the context.
+static bool dequant_workspace(fq_ctx* ctx, cudaStream_t st, size_t need)
+{
+    if (need <= ctx->gemm_ws_bytes) return true;
+    if (!may_allocate(st) || cudaDeviceSynchronize() != cudaSuccess) return false;
+    size_t most = need;
+    for (const Layer& L : ctx->layers)
+        if (L.registered && (size_t)L.n_out * L.k_in * 2 > most) most = (size_t)L.n_out * L.k_in * 2;
+    if (ctx->gemm_ws) cudaFree(ctx->gemm_ws);
+    ctx->gemm_ws = nullptr; ctx->gemm_ws_bytes = 0;
+    for (const size_t bytes : {most, need}) {
+        if (cudaMalloc(&ctx->gemm_ws, bytes) == cudaSuccess) { ctx->gemm_ws_bytes = bytes; return true; }
+        cudaGetLastError();
+        ctx->gemm_ws = nullptr;
+    }
+    return false;
+}
+
 static int gemm_common(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int ldx, uint16_t* Y_dev, int ldy, void* stream,
                        bool fused)
 {
@@ -826,36 +868,20 @@ static int gemm_common(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int
     if (!guard.ok) return FQ_ERR_CUDA;
     const int zero_adjust = (L.fmt == FQ_FMT_PLANES && bits < 8) ? (1 << (7 - bits)) : 0;
     const int stride = blob_bytes(L.fmt == FQ_FMT_PLANES ? 8 : bits);
-    if (fused) {
-        float* parts = nullptr;
-        unsigned* flags = nullptr;
-        if (gemm_fused_wants_balance(M, L.n_out, ctx->sm_count)) {
-            // partial-sum slots of the tiles that two CTAs share: [flags 4 x (SMs + 1), padded][slot x (SMs + 1)];
-            // allocated the first time a shape asks for balanced runs
-            const size_t flag_bytes = (size_t)round_up((int64_t)((ctx->sm_count + 1) * 4 * sizeof(unsigned)), 256);
-            if (!ctx->fused_ws) {
-                const size_t bytes = flag_bytes + (size_t)(ctx->sm_count + 1) * gemm_fused_part_bytes();
-                FQ_CUDA_OK(cudaMalloc(&ctx->fused_ws, bytes));
-                FQ_CUDA_OK(cudaMemset(ctx->fused_ws, 0, flag_bytes));
-                ctx->fused_epoch = 0;
-            }
-            if (++ctx->fused_epoch == 0) ctx->fused_epoch = 1;               // (0 is the cleared flag)
-            flags = reinterpret_cast<unsigned*>(ctx->fused_ws);
-            parts = reinterpret_cast<float*>(ctx->fused_ws + flag_bytes);
-        }
-        return launch_gemm_fused(ctx, v->store, stride, active_fields(L, bits), zero_adjust, L.n_out, L.k_in, X_dev, M, ldx,
-                                 Y_dev, ldy, parts, flags, ctx->fused_epoch, (cudaStream_t)stream);
-    }
-    const size_t need = (size_t)L.n_out * L.k_in * 2;
-    if (need > ctx->gemm_ws_bytes) {
-        FQ_CUDA_OK(cudaDeviceSynchronize());
-        if (ctx->gemm_ws) cudaFree(ctx->gemm_ws);
-        ctx->gemm_ws = nullptr; ctx->gemm_ws_bytes = 0;
-        FQ_CUDA_OK(cudaMalloc(&ctx->gemm_ws, need));
-        ctx->gemm_ws_bytes = need;
-    }
-    return launch_gemm(ctx, v->store, stride, active_fields(L, bits), zero_adjust, L.n_out, L.k_in, X_dev, M, ldx, Y_dev, ldy,
-                       ctx->gemm_ws, (cudaStream_t)stream);
+    const cudaStream_t st = (cudaStream_t)stream;
+    const FieldList fl = active_fields(L, bits);
+    // Two ways to the same product, whichever the shape makes the faster one: converting the weights inside the GEMM, once for
+    // every tile of up to 192 tokens, or once for all tokens in a pass of their own.  Both estimates are fits to measured times
+    // (within about 15 %); the second way needs room for a bf16 copy of the layer.
+    const bool two_pass = !fused || gemm_two_pass_us(ctx, M, L.n_out, L.k_in) < gemm_split_us(ctx, M, L.n_out, L.k_in);
+    if (two_pass && dequant_workspace(ctx, st, (size_t)L.n_out * L.k_in * 2))
+        return launch_gemm(ctx, v->store, stride, fl, zero_adjust, L.n_out, L.k_in, X_dev, M, ldx, Y_dev, ldy, ctx->gemm_ws, st);
+    if (!fused) return FQ_ERR_CUDA;
+    // counters and slots for the sums of tiles that several CTAs share; without them the tiles stay whole
+    unsigned* arrived = reinterpret_cast<unsigned*>(ctx->fused_ws);
+    float* parts = ctx->fused_ws ? reinterpret_cast<float*>(ctx->fused_ws + gemm_split_flag_bytes(ctx->sm_count)) : nullptr;
+    const int read = L.fmt == FQ_FMT_PLANES ? blob_bytes(plane_read_bits(bits)) : stride;
+    return launch_gemm_split(ctx, v->store, stride, read, fl, zero_adjust, L.n_out, L.k_in, X_dev, M, ldx, Y_dev, ldy, parts, arrived, st);
 }
 
 int fq_gemm(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int ldx, uint16_t* Y_dev, int ldy, void* stream)

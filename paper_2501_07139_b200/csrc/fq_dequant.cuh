@@ -74,6 +74,54 @@ __device__ __forceinline__ void merge_codes(const uint4 (&raw)[fields_loads(vari
     });
 }
 
+// The same for a whole group of 128 columns (k32 steps 4 * grp .. + 3): every 16-byte chunk once.
+FQ_HDC int group_loads(const FieldList fl, int fi) { int n = 0; for (int i = 0; i < fi; i++) n += fl.width[i] >= 2 ? fl.width[i] / 2 : 1; return n; }
+
+template <int VARIANT, int TL>
+__device__ __forceinline__ void load_group_words(const uint8_t* blob_lane, int ssl, int grp,
+                                                 uint4 (&raw)[group_loads(variant_fields(VARIANT), variant_fields(VARIANT).n)])
+{
+    constexpr FieldList FL = variant_fields(VARIANT);
+    unrolled<0, FL.n>([&](auto FI) {
+        constexpr int fi = decltype(FI)::value, F = FL.width[fi], base = group_loads(FL, fi), n = F >= 2 ? F / 2 : 1;
+        const uint8_t* tb = blob_lane + blob_field_off(fields_prefix(FL, fi), F, 0, TL) + ssl * (kBlobTiles * F * 512) +
+                            (F >= 2 ? grp * (n * 512) : 0);
+#pragma unroll
+        for (int i = 0; i < n; i++) raw[base + i] = __ldg(reinterpret_cast<const uint4*>(tb + i * 512));
+    });
+}
+// A 1-bit field's chunk holds both groups: the second one's bits come down once, so that every other shift is a constant.
+template <int VARIANT>
+__device__ __forceinline__ void align_group_words(uint4 (&raw)[group_loads(variant_fields(VARIANT), variant_fields(VARIANT).n)], int grp)
+{
+    constexpr FieldList FL = variant_fields(VARIANT);
+    unrolled<0, FL.n>([&](auto FI) {
+        constexpr int fi = decltype(FI)::value, F = FL.width[fi], base = group_loads(FL, fi);
+        if constexpr (F == 1) {
+            raw[base].x >>= 4 * grp; raw[base].y >>= 4 * grp; raw[base].z >>= 4 * grp; raw[base].w >>= 4 * grp;
+        }
+    });
+}
+// The A registers of k32 step J (0 .. 3) of the group.
+template <int VARIANT, int J>
+__device__ __forceinline__ void merge_group_codes(const uint4 (&raw)[group_loads(variant_fields(VARIANT), variant_fields(VARIANT).n)],
+                                                  uint32_t (&code)[4])
+{
+    constexpr FieldList FL = variant_fields(VARIANT);
+    unrolled<0, FL.n>([&](auto FI) {
+        constexpr int fi = decltype(FI)::value, F = FL.width[fi], P = 8 / F, SH = FL.shift[fi], at = (J % P) * F, base = group_loads(FL, fi);
+        constexpr uint32_t kM = (field_keep_mask(F, FL.keep[fi]) * 0x01010101u) << SH;
+        constexpr int down = at >= SH ? at - SH : 0, up = at >= SH ? 0 : SH - at;      // (one of the two is zero)
+        const uint4 w = raw[base + J / P];
+        const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int r = 0; r < 4; r++) {
+            const uint32_t v = F == 8 ? ww[r] : ((ww[r] >> down) << up) & kM;
+            code[r] = fi == 0 ? v : (code[r] | v);
+        }
+    });
+}
+
 // Four codes of one row (one A register) -> four bf16 weights w^ = (q - z) * s, each rounded once.
 //   Codes up to 255: a byte q under the exponent byte 0x64 is the fp16 number 1024 + q; subtracting zz = 1024 + z
 //   in fp16 is exact (integers below 2048), the product with the fp16 scale is exact in fp32 (9 x 11 bits).

@@ -75,8 +75,7 @@ struct Ctx {
     // prefill: dequantised bf16 copy of the layer being multiplied
     char* gemm_ws = nullptr;
     size_t gemm_ws_bytes = 0;
-    char* fused_ws = nullptr;            // fused GEMM, balanced runs: flags, then one fp32 tile slot per SM (+ 1)
-    unsigned fused_epoch = 0;
+    char* fused_ws = nullptr;            // prefill: counters, then two fp32 tile slots per SM (part of the allocation of status_dev)
     std::vector<void*> owned;    // device buffers allocated by fq_load, freed by fq_destroy
     uint64_t config_epoch = 0;
     unsigned launch_epoch = 0;   // tag of the split-K partials of the latest decode launch (never 0)
@@ -128,11 +127,14 @@ int launch_stream_read(const void* src, size_t bytes, unsigned* sink, int sm_cou
 int gemv_chunk_blobs(int bits);
 size_t gemv_partial_bytes_per_unit(int batch);
 int launch_gemv_single(Ctx* ctx, const GemvOp& op, cudaStream_t st);                 // batch 2..8
-int launch_gemm_fused(Ctx* ctx, const void* store, int blob_stride, const FieldList& fl, int zero_adjust, int n_out, int k_in,
-                      const uint16_t* X, int M, int ldx, uint16_t* Y, int ldy, float* parts, unsigned* part_flags, unsigned epoch,
-                      cudaStream_t st);                   // parts == nullptr: whole tiles; else balanced runs through these slots
-size_t gemm_fused_part_bytes();          // bytes of one CTA's partial-sum slot
-bool gemm_fused_wants_balance(int M, int n_out, int sm_count);
+// parts == nullptr: whole tiles only; else tiles may be shared between CTAs through these slots
+int launch_gemm_split(Ctx* ctx, const void* store, int blob_stride, int blob_read, const FieldList& fl, int zero_adjust, int n_out,
+                      int k_in, const uint16_t* X, int M, int ldx, uint16_t* Y, int ldy, float* parts, unsigned* arrived,
+                      cudaStream_t st);
+size_t gemm_split_flag_bytes(int sm_count);
+size_t gemm_split_part_bytes(int sm_count);
+double gemm_split_us(const Ctx* ctx, int M, int n_out, int k_in);       // estimates of the time of a call
+double gemm_two_pass_us(const Ctx* ctx, int M, int n_out, int k_in);
 struct CtaWork;
 int launch_gemv1_single(Ctx* ctx, const GemvOp& op, cudaStream_t st);                // batch 1
 // table_dev: [GemvOp x n_ops][int phase_total x max(n_phases,1)][uint2 strips x sm_count x n_ops]
