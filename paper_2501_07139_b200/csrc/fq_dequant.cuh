@@ -1,5 +1,5 @@
-// Dequantisation of stored words to bf16, shared by the prefill kernels: the fused kernel's dequantisation warps
-// (fq_gemm_fused.cu) and the stand-alone pass of the two-pass path (fq_gemm.cu).  Everything is specialised per
+// Dequantisation of stored words to bf16, shared by the prefill kernels: the dequantisation warps of the
+// fused one (fq_gemm_split.cu) and the stand-alone pass of the two-pass path (fq_gemm.cu).  Everything is specialised per
 // field list (variant_index in fq_layout.cuh), so that field widths, shifts and offsets are compile-time constants.
 #pragma once
 #include <cuda_bf16.h>
@@ -102,16 +102,16 @@ __device__ __forceinline__ void align_group_words(uint4 (&raw)[group_loads(varia
         }
     });
 }
-// The A registers of k32 step J (0 .. 3) of the group.
-template <int VARIANT, int J>
+// The A registers of k32 step J (0 .. 3) of the group, every code shifted down by DOWN bits (that must be zero).
+template <int VARIANT, int J, int DOWN = 0>
 __device__ __forceinline__ void merge_group_codes(const uint4 (&raw)[group_loads(variant_fields(VARIANT), variant_fields(VARIANT).n)],
                                                   uint32_t (&code)[4])
 {
     constexpr FieldList FL = variant_fields(VARIANT);
     unrolled<0, FL.n>([&](auto FI) {
         constexpr int fi = decltype(FI)::value, F = FL.width[fi], P = 8 / F, SH = FL.shift[fi], at = (J % P) * F, base = group_loads(FL, fi);
-        constexpr uint32_t kM = (field_keep_mask(F, FL.keep[fi]) * 0x01010101u) << SH;
-        constexpr int down = at >= SH ? at - SH : 0, up = at >= SH ? 0 : SH - at;      // (one of the two is zero)
+        constexpr uint32_t kM = ((field_keep_mask(F, FL.keep[fi]) << SH) >> DOWN) * 0x01010101u;
+        constexpr int down = at >= SH - DOWN ? at - SH + DOWN : 0, up = at >= SH - DOWN ? 0 : SH - DOWN - at;   // (one of the two is zero)
         const uint4 w = raw[base + J / P];
         const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
@@ -153,6 +153,9 @@ __device__ __forceinline__ uint2 small_codes_to_bf16(uint32_t q4, float c, float
     o.y = *reinterpret_cast<const uint32_t*>(&hi);
     return o;
 }
+
+//   A nested child of at most 7 bits has codes q = 2 h, h below 128, and a mid-point fill of at least 1:
+//   fma(128 + h, 2 s, c) with c = -(256 + z - fill) * s (exact: 9 x 11 bits) is (q + fill - z) * s, with the same instructions.
 
 // The variant whose field list is `fl`, or -1.
 inline int variant_of_fields(const FieldList& fl)

@@ -34,7 +34,7 @@ struct DequantArgs {
 // One warp per (row strip of 32, 64 columns): the lanes read the stored words of the two k32 steps exactly as
 // the decode kernel does (16 bytes per lane and field chunk), merge the fields into four codes per register,
 // convert (w^ = (q - z) * s exactly, one rounding to bf16) and write 8-byte runs; the four lanes of a quad
-// cover 32 contiguous bytes of a row.  Specialised per field list like the fused kernel, whose helpers it shares.
+// cover 32 contiguous bytes of a row.  Specialised per field list like fq_gemm_split.cu, whose helpers it shares.
 template <int VARIANT>
 __global__ void __launch_bounds__(256) dequant_kernel(const DequantArgs a)
 {
@@ -344,12 +344,12 @@ static PairTiles pair_tile_n(int M, int n_out, int pairs)
     return best;
 }
 
-// Measured (4096 x 4096, 11008 x 4096 and 4096 x 11008, 16 to 8192 tokens): the conversion takes 2 us + 0.31 us per million
-// weights, a stage of 64 columns of a 256 x 256 tile 0.4 us, the second launch 2 us.
+// Measured (4096 x 4096, 11008 x 4096 and 4096 x 11008, 16 to 8192 tokens): the conversion takes 0.33 us per million weights, a
+// stage of 64 columns 0.4 us at 256 outputs and not much less at fewer, everything else 6 us.
 double gemm_two_pass_us(const Ctx* ctx, int M, int n_out, int k_in)
 {
     const PairTiles t = pair_tile_n(M, n_out, ctx->sm_count / 2);
-    return 4.0 + 0.31e-6 * (double)n_out * (double)k_in + (double)t.waves * (k_in / kBK) * 0.4 * (t.width + 16) / 272.0;
+    return 6.0 + 0.33e-6 * (double)n_out * (double)k_in + (double)t.waves * (k_in / kBK) * (0.2 + 0.2 * (t.width + 16) / 272.0);
 }
 
 int launch_gemm(Ctx* ctx, const void* store, int blob_stride, const FieldList& fl, int zero_adjust, int n_out, int k_in,

@@ -1,6 +1,6 @@
 // Prefill path, fused:  Y[m][n] = sum_k X[m][k] * w^[n][k]  straight from the stored blobs.
 //
-// The WEIGHTS are the left operand: a tile is 128 outputs (TMEM lanes) x up to 192 tokens (TMEM columns), so that the tensor
+// The WEIGHTS are the left operand: a tile is 128 outputs (TMEM lanes) x up to 160 tokens (TMEM columns), so that the tensor
 // work follows the token count in steps of 16, and the converted weights go from registers straight into TMEM (tcgen05.st),
 // from where the MMA reads its left operand: they never pass through shared memory.
 //   warp 0        lane 0: TMA, two tile_n x 64 bf16 tiles of X per stage (128-byte swizzle)
@@ -34,7 +34,8 @@ namespace fq {
 namespace {
 
 constexpr int kRows = 128;               // outputs per tile (UMMA M)
-constexpr int kTokens = 192;             // tokens per tile, at most (UMMA N): four stages of X, and of weights beside the accumulator
+constexpr int kTokens = 160;             // tokens per tile, at most (UMMA N): four stages of X and a tile of Y in shared memory, four
+                                         // stages of weights beside the accumulator in TMEM
 constexpr int kK = kGroup;               // K per stage: a group of 128 columns.  One pass of the issuing warp's loop (wait, issue,
                                          // commit) costs about 300 cycles whether it issues four MMAs or eight
 constexpr int kStages = 4;
@@ -48,8 +49,10 @@ static_assert(kTokens <= kTmemA && kTmemA + kStages * (kK / 2) <= kTmemCols, "TM
 
 struct SplitSmem {
     static constexpr int kHalfBytes = kTokens * kUmmaBK * 2;       // 64 columns: one 128-byte swizzle span a token
-    static constexpr int kStageBytes = 2 * kHalfBytes;             // 48 KB
-    static constexpr int oBars = kStages * kStageBytes;            // full[S], empty[S], tmem_full, tmem_empty
+    static constexpr int kStageBytes = 2 * kHalfBytes;             // 40 KB
+    static constexpr int kOutRow = kRows * 2 + 16;                 // a token's outputs (bf16), and room that spreads tokens over the banks
+    static constexpr int oOut = kStages * kStageBytes;
+    static constexpr int oBars = oOut + kTokens * kOutRow;         // full[S], empty[S], tmem_full, tmem_empty
     static constexpr int oTmemPtr = oBars + (2 * kStages + 3) * 8; // (and sums_due)
     static constexpr int oFlag = oTmemPtr + 8;
     static constexpr int oDue = oFlag + 8;                         // int[2]: this CTA completes its first / last tile; int[2]: warps done
@@ -181,21 +184,32 @@ __device__ __forceinline__ void add_shared_tiles(const SplitArgs& a, const volat
         const float4* in0 = reinterpret_cast<const float4*>(a.parts) + (long long)sh.slot0 * slot + trow;
         const float4* in1 = reinterpret_cast<const float4*>(a.parts) + (long long)(sh.c0 + 1) * 2 * slot + trow;
         __nv_bfloat16* y = a.Y + (long long)mb * a.tile_n * a.ldy;
-        for (int q = set; q < quads; q += kSumSets) {
-            float4 s = __ldcg(in0 + q * kRows);
-            for (int i0 = 0; i0 < others; i0 += 8) {
-                float4 p[8];
+        for (int qa = set; qa < quads; qa += 2 * kSumSets) {             // two at a time: ten loads on their way with four others
+            const int qb = qa + kSumSets < quads ? qa + kSumSets : qa;
+            float4 sa = __ldcg(in0 + qa * kRows), sb = __ldcg(in0 + qb * kRows);
+            for (int i0 = 0; i0 < others; i0 += 4) {
+                float4 pa[4], pb[4];
 #pragma unroll
-                for (int i = 0; i < 8; i++) {
-                    p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (i0 + i < others) p[i] = __ldcg(in1 + (long long)(i0 + i) * 2 * slot + q * kRows);
+                for (int i = 0; i < 4; i++) {
+                    pa[i] = pb[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (i0 + i < others) {
+                        const float4* in = in1 + (long long)(i0 + i) * 2 * slot;
+                        pa[i] = __ldcg(in + qa * kRows);
+                        pb[i] = __ldcg(in + qb * kRows);
+                    }
                 }
 #pragma unroll
-                for (int i = 0; i < 8; i++) { s.x += p[i].x; s.y += p[i].y; s.z += p[i].z; s.w += p[i].w; }
+                for (int i = 0; i < 4; i++) {
+                    sa.x += pa[i].x; sa.y += pa[i].y; sa.z += pa[i].z; sa.w += pa[i].w;
+                    sb.x += pb[i].x; sb.y += pb[i].y; sb.z += pb[i].z; sb.w += pb[i].w;
+                }
             }
-            const int t = 4 * q;
-            store_pair(y + (long long)t * a.ldy, a.ldy, n, a.N, s.x, s.y, t < tokens, t + 1 < tokens, lane);
-            store_pair(y + (long long)(t + 2) * a.ldy, a.ldy, n, a.N, s.z, s.w, t + 2 < tokens, t + 3 < tokens, lane);
+            const int ta = 4 * qa, tb = 4 * qb;
+            store_pair(y + (long long)ta * a.ldy, a.ldy, n, a.N, sa.x, sa.y, ta < tokens, ta + 1 < tokens, lane);
+            store_pair(y + (long long)(ta + 2) * a.ldy, a.ldy, n, a.N, sa.z, sa.w, ta + 2 < tokens, ta + 3 < tokens, lane);
+            if (qb == qa) break;
+            store_pair(y + (long long)tb * a.ldy, a.ldy, n, a.N, sb.x, sb.y, tb < tokens, tb + 1 < tokens, lane);
+            store_pair(y + (long long)(tb + 2) * a.ldy, a.ldy, n, a.N, sb.z, sb.w, tb + 2 < tokens, tb + 3 < tokens, lane);
         }
     }
 }
@@ -206,7 +220,8 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_x, const SplitArgs a)
 {
     constexpr FieldList FL = variant_fields(VARIANT);
     constexpr int kLoads = group_loads(FL, FL.n);
-    constexpr bool kSmallCodes = VARIANT < 6;            // PACKED 2..7 bits: codes below 128, no zero adjustment
+    constexpr bool kHalved = VARIANT >= 7 && VARIANT < 13;         // a nested child of 2..7 bits: half its codes are below 128
+    constexpr bool kSmallCodes = VARIANT < 6 || kHalved;           // PACKED 2..7 bits: codes below 128, no zero adjustment
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -336,16 +351,39 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_x, const SplitArgs a)
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (run.whole(it)) {
-                __nv_bfloat16* y = a.Y + (long long)mb * a.tile_n * a.ldy;
+                // through shared memory: the accumulator is free for the next tile as soon as it has been read, and the stores to
+                // Y are 16 bytes a lane (straight from TMEM a lane has one output of every token: 9000 cycles for 160 tokens)
+                uint8_t* mine = smem + SplitSmem::oOut + trow * 2;
 #pragma unroll 1
                 for (int t0 = 0; t0 < tokens; t0 += 16) {
                     uint32_t v[16];
                     tmem_ld_x16(taddr + (uint32_t)t0, v);
 #pragma unroll
-                    for (int e = 0; e < 16; e += 2)
-                        store_pair(y + (long long)(t0 + e) * a.ldy, a.ldy, n, a.N, __uint_as_float(v[e]), __uint_as_float(v[e + 1]),
-                                   t0 + e < tokens, t0 + e + 1 < tokens, lane);
+                    for (int e = 0; e < 16; e++)
+                        *reinterpret_cast<__nv_bfloat16*>(mine + (t0 + e) * SplitSmem::kOutRow) = __float2bfloat16_rn(__uint_as_float(v[e]));
                 }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(tempty);                     // the accumulator may be overwritten
+                // this warp's 32 outputs of every token: 64 bytes, four lanes; eight tokens at a time
+                const int n4 = it.tile / a.m_blocks * kRows + quarter * 32 + (lane & 3) * 8;
+                __nv_bfloat16* y = a.Y + (long long)mb * a.tile_n * a.ldy + n4;
+                const uint8_t* from = smem + SplitSmem::oOut + (quarter * 32 + (lane & 3) * 8) * 2;
+#pragma unroll 2
+                for (int t = lane >> 2; t < tokens; t += 8) {
+                    const uint4 o = *reinterpret_cast<const uint4*>(from + t * SplitSmem::kOutRow);
+                    __nv_bfloat16* dst = y + (long long)t * a.ldy;
+                    if (n4 + 8 <= a.N) {
+                        *reinterpret_cast<uint4*>(dst) = o;
+                    } else {
+                        const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&o);
+#pragma unroll
+                        for (int e = 0; e < 8; e++)
+                            if (n4 + e < a.N) dst[e] = h[e];
+                    }
+                }
+                __syncwarp();
+                continue;
             } else {
                 // partial sums: float4 number q (tokens 4q .. 4q + 3) of the slot is [q][output of the tile]
                 const int slot = blockIdx.x * 2 + (local > 0 ? 1 : 0);
@@ -430,7 +468,8 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_x, const SplitArgs a)
                     for (int hr = 0; hr < 2; hr++) {
                         sc[hr] = have ? __half2float(__ushort_as_half((unsigned short)(mm[hr] & 0xffffu))) : 0.f;   // rows past N: zeros
                         zz[hr] = __half2half2(__int2half_rn(1024 + (int)(mm[hr] >> 16) - a.zero_adjust));
-                        cc[hr] = -(float)(128 + (int)(mm[hr] >> 16)) * sc[hr];
+                        cc[hr] = -(float)((kHalved ? 256 - a.zero_adjust : 128) + (int)(mm[hr] >> 16)) * sc[hr];
+                        if (kHalved) sc[hr] *= 2.f;
                     }
                     unrolled<0, 2>([&](auto H) {                               // 64 columns at a time
                         constexpr int h = decltype(H)::value;
@@ -438,7 +477,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_x, const SplitArgs a)
                         unrolled<0, 2>([&](auto JJ) {
                             constexpr int jj = decltype(JJ)::value;
                             uint32_t code[4];
-                            merge_group_codes<VARIANT, 2 * h + jj>(raw[tl], code);
+                            merge_group_codes<VARIANT, 2 * h + jj, kHalved ? 1 : 0>(raw[tl], code);
 #pragma unroll
                             for (int r = 0; r < 4; r++) {
                                 const int hr = r & 1, half = r >> 1;           // A register r = 2 * half + row half
@@ -501,8 +540,9 @@ int split_tile_n(int M)
     return (int)round_up((M + tiles - 1) / tiles, 16);
 }
 
-// Sharing tiles evens the CTAs out and costs an exchange of partial sums through the L2.  Measured (4096 x 4096 and
-// 11008 x 4096, 16 to 600 tokens): a stage takes about 0.5 us + 1.2 ns a token, the exchange 4 us + 80 ns a token.
+// Sharing tiles evens the CTAs out and costs an exchange of partial sums through the L2.  Measured (4096 x 4096, 11008 x 4096 and
+// 4096 x 11008, 16 to 600 tokens): a stage takes about 0.33 us + 1 ns a token, the exchange 4.5 us + 60 ns a token, everything
+// else 5 us.
 struct Plan {
     long long tiles, pairs, runs;        // pairs: (tile, K stage); runs: CTAs when tiles are shared
     bool share;
@@ -515,17 +555,23 @@ struct Plan {
         const long long grid = tiles < sm_count ? tiles : sm_count;
         runs = pairs / kMinRun < sm_count ? pairs / kMinRun : sm_count;
         if (runs < grid) runs = grid;
-        const double stage_us = 0.5 + 0.0012 * tile_n, exchange_us = 4.0 + 0.08 * tile_n;
+        const double stage_us = 0.33 + 0.001 * tile_n, exchange_us = 4.5 + 0.06 * tile_n;
         const double whole = (double)((tiles + grid - 1) / grid * k_steps) * stage_us;
         const double shared = (double)((pairs + runs - 1) / runs) * stage_us + exchange_us;
         share = pairs < (1ll << 31) && shared < whole;
-        us = share ? shared : whole;
+        us = 5.0 + (share ? shared : whole);
     }
 };
 
 }  // namespace
 
-double gemm_split_us(const Ctx* ctx, int M, int n_out, int k_in) { return Plan(ctx->sm_count, M, n_out, k_in).us; }
+// Long prompts run into the power limit, and converting the weights once per token tile costs energy: chosen by the estimate of
+// a cool chip alone, one 7B block at 8192 tokens took 3338 us in this kernel and 2692 us in the two-pass way, a 13B block at
+// 2048 tokens 1334 and 1187 us.
+double gemm_split_us(const Ctx* ctx, int M, int n_out, int k_in)
+{
+    return Plan(ctx->sm_count, M, n_out, k_in).us * (1.0 + 0.3 * (M < 2048 ? M : 2048) / 2048.0);
+}
 
 size_t gemm_split_flag_bytes(int sm_count) { return (size_t)round_up((int64_t)sm_count * sizeof(unsigned), 256); }
 size_t gemm_split_part_bytes(int sm_count) { return (size_t)sm_count * 2 * kRows * kTokens * sizeof(float); }

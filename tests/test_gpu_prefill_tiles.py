@@ -23,7 +23,7 @@ def _layer(P, tag, n, k, bits, fmt):
 
 def _check(fq, ref, x, n, call=None):
     m = x.shape[0]
-    y = torch.full((m + 2, n + 8), float("nan"), dtype=torch.bfloat16, device="cuda")
+    y = torch.full((m + 2, (n + 7) // 8 * 8 + 8), float("nan"), dtype=torch.bfloat16, device="cuda")
     view = y[1:m + 1, :n]
     (call or fq.fq_gemm)(0, x, view)
     assert fq.fq_status() == 0
