@@ -106,51 +106,50 @@ __device__ __forceinline__ void group_mma(const uint32_t (&fa)[kMaxFields], uint
     });
 }
 
-// One 16-row tile of `steps` supersteps (whole blobs): tot[0..1] row g, tot[2..3] row g + 8, batch entries 2c, 2c + 1.
+// Supersteps first .. first + steps - 1 of a unit, one 16-row tile: tot[0..1] row g, tot[2..3] row g + 8, batch entries 2c, 2c + 1.
 //   stage : shared address of the unit's first blob        xs : of the activation slot
 template <int VARIANT, int BP>
-__device__ __forceinline__ void unit_compute(uint32_t stage, int steps, uint32_t blob_read, uint32_t xs, int lane, int tile, float (&tot)[4])
+__device__ __forceinline__ void unit_compute(uint32_t stage, int first, int steps, uint32_t blob_read, uint32_t xs, int lane, int tile, float (&tot)[4])
 {
     constexpr FieldList FL = variant_fields(VARIANT);
     const int g = lane >> 2, c = lane & 3;
     // batch entries beyond the padding read a valid entry's activations; nobody uses what they add up to
-    uint32_t xa = xs + (uint32_t)((g & (BP - 1)) * kXRowBytes + c * 8);
-    uint32_t blob = stage;
-    for (int s = 0; s < steps; s += kBlobSteps, blob += blob_read) {
+    uint32_t xa = xs + (uint32_t)((g & (BP - 1)) * kXRowBytes + c * 8 + first * kStepCols * 2);
 #pragma unroll 1                                                     // (keeps the specialised loops small)
-        for (int ssl = 0; ssl < kBlobSteps; ssl++, xa += kStepCols * 2) {
-            const int st_tile = ssl * kBlobTiles + tile;
-            uint32_t fa[kMaxFields];
-            static_for<0, FL.n>([&](auto FI) {
-                constexpr int fi = decltype(FI)::value;
-                constexpr int prefix = [] { int p = 0; for (int i = 0; i < fi; i++) p += variant_fields(VARIANT).width[i]; return p; }();
-                fa[fi] = blob + kBlobMetaBytes + kBlobSteps * kBlobTiles * 512 * prefix + st_tile * (FL.width[fi] * 512) + lane * 16;
-            });
-            const uint4 m4 = lds128(blob + st_tile * 128 + g * 16);   // scale/zero words: group 0 rows g, g + 8, group 1 rows g, g + 8
-            static_for<0, 2>([&](auto G) {
-                constexpr int grp = decltype(G)::value;
-                const uint32_t m[2] = {grp ? m4.z : m4.x, grp ? m4.w : m4.y};
-                __half2 nz[2];
-                float sc[2];
+    for (int s = first; s < first + steps; s++, xa += kStepCols * 2) {
+        const int ssl = s % kBlobSteps;
+        const uint32_t blob = stage + (uint32_t)(s / kBlobSteps) * blob_read;
+        const int st_tile = ssl * kBlobTiles + tile;
+        uint32_t fa[kMaxFields];
+        static_for<0, FL.n>([&](auto FI) {
+            constexpr int fi = decltype(FI)::value;
+            constexpr int prefix = [] { int p = 0; for (int i = 0; i < fi; i++) p += variant_fields(VARIANT).width[i]; return p; }();
+            fa[fi] = blob + kBlobMetaBytes + kBlobSteps * kBlobTiles * 512 * prefix + st_tile * (FL.width[fi] * 512) + lane * 16;
+        });
+        const uint4 m4 = lds128(blob + st_tile * 128 + g * 16);   // scale/zero words: group 0 rows g, g + 8, group 1 rows g, g + 8
+        static_for<0, 2>([&](auto G) {
+            constexpr int grp = decltype(G)::value;
+            const uint32_t m[2] = {grp ? m4.z : m4.x, grp ? m4.w : m4.y};
+            __half2 nz[2];
+            float sc[2];
 #pragma unroll
-                for (int r = 0; r < 2; r++) {
-                    sc[r] = __half2float(__ushort_as_half((unsigned short)(m[r] & 0xffffu)));
-                    nz[r] = __half2half2(__hneg(__ushort2half_rn((unsigned short)(m[r] >> 16))));
-                }
-                float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};      // two chains: an MMA waits long for its sums
-                group_mma<VARIANT, grp>(fa, xa, nz, acc);
+            for (int r = 0; r < 2; r++) {
+                sc[r] = __half2float(__ushort_as_half((unsigned short)(m[r] & 0xffffu)));
+                nz[r] = __half2half2(__hneg(__ushort2half_rn((unsigned short)(m[r] >> 16))));
+            }
+            float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};      // two chains: an MMA waits long for its sums
+            group_mma<VARIANT, grp>(fa, xa, nz, acc);
 #pragma unroll
-                for (int i = 0; i < 4; i++) tot[i] = fmaf(sc[i >> 1], acc[0][i] + acc[1][i], tot[i]);
-            });
-        }
+            for (int i = 0; i < 4; i++) tot[i] = fmaf(sc[i >> 1], acc[0][i] + acc[1][i], tot[i]);
+        });
     }
 }
 
 template <int BP>
-__device__ __forceinline__ void unit_dispatch(int variant, uint32_t stage, int steps, uint32_t blob_read, uint32_t xs, int lane, int tile,
+__device__ __forceinline__ void unit_dispatch(int variant, uint32_t stage, int first, int steps, uint32_t blob_read, uint32_t xs, int lane, int tile,
                                               float (&tot)[4])
 {
-#define FQ_VARIANT_CASE(V) case V: unit_compute<V, BP>(stage, steps, blob_read, xs, lane, tile, tot); break;
+#define FQ_VARIANT_CASE(V) case V: unit_compute<V, BP>(stage, first, steps, blob_read, xs, lane, tile, tot); break;
     switch (variant) {
         FQ_VARIANT_CASE(0) FQ_VARIANT_CASE(1) FQ_VARIANT_CASE(2) FQ_VARIANT_CASE(3) FQ_VARIANT_CASE(4)
         FQ_VARIANT_CASE(5) FQ_VARIANT_CASE(6) FQ_VARIANT_CASE(7) FQ_VARIANT_CASE(8) FQ_VARIANT_CASE(9)

@@ -8,12 +8,12 @@
 //                     and writes a small descriptor next to each stage;
 //   activation warp : once per (op, K chunk) that this CTA touches, waits -- bounded -- for the
 //                     previous dependency phase and fetches the activations of that chunk, one bulk copy per batch row;
-//   consumer warps  : two warps share a unit, one 16-row tile each.  Stored words become fp16 integers q - z, the fp16
+//   consumer warps  : two or four warps share a unit, one 16-row tile, or a half of its columns, each.  Stored words become fp16 integers q - z, the fp16
 //                     activations are the other operand of mma.m16n8k16, sums are fp32 and scaled once per group of 128
 //                     columns (fq_batch_core.cuh).  The loops are compiled once per field list (14 variants) and chosen
-//                     per unit.  13B nested at 4 bits, four blocks, no
-//                     dependencies: 4 / 8 entries 189 / 238 us, against 330 / 600 us with one 8-bit integer MMA per field and digit
-//                     of fixed-point activations.
+//                     per unit.  13B nested at 4 bits, four blocks in
+//                     dependency order: 4 / 8 entries 333 / 375 us, against 534 / 593 us with one 8-bit integer MMA per field and
+//                     digit of fixed-point activations.
 //   output warps    : finish row pairs (see below) and are the only warps that write y.
 // The K chunks of one row pair are computed by different CTAs.  Each unit publishes its row sums
 // as 64-bit words (fp32 value, launch tag) with plain stores; the unit whose chunk index is
@@ -37,9 +37,6 @@ namespace fq {
 #define FQ_CUDA_OK(expr) do { if ((expr) != cudaSuccess) return FQ_ERR_CUDA; } while (0)
 
 constexpr int kConsumerWarps = 20;
-constexpr int kWarpsPerUnit = kUnitRowTiles;           // one 16-row tile each
-constexpr int kUnitsInFlight = kConsumerWarps / kWarpsPerUnit;
-static_assert(kConsumerWarps % kWarpsPerUnit == 0, "consumer warps come in groups of one unit");
 constexpr int kProducerWarp = kConsumerWarps;          // warp index of the producer
 constexpr int kActWarp = kConsumerWarps + 1;           // the warp that fetches activations
 constexpr int kOutputWarp = kActWarp + 1;              // the warps that own every global store of results
@@ -71,13 +68,21 @@ struct OutDesc {
 static_assert(sizeof(OutDesc) == 48, "descriptor layout");
 
 template <int BP> struct GemvSmem {
+    // Warps that share a unit: one 16-row tile each, and for up to eight entries also one half of the columns each.  Their stage
+    // ring is the shorter one (more shared memory goes to activations), so a unit has to leave it sooner: 13B nested at
+    // 4 bits, four blocks in dependency order: 399 -> 375 us; up to four entries lose by it (333 -> 362 us).
+    static constexpr int kWarpsPerUnit = BP == 8 ? 2 * kUnitRowTiles : kUnitRowTiles;
+    static constexpr bool kHalves = kWarpsPerUnit > kUnitRowTiles;
+    static constexpr int kUnitsInFlight = kConsumerWarps / kWarpsPerUnit;
+    static_assert(kConsumerWarps % kWarpsPerUnit == 0, "consumer warps come in groups of one unit");
     static constexpr int kStageBytes = kUnitBytes;
     static constexpr int kXSlotBytes = BP * kXRowBytes;              // one chunk's activations
     static constexpr int kOpBytes = (int)((sizeof(GemvOp) + 15) / 16 * 16);
     static constexpr int kOutFloats = 32 * BP;                               // row sums of one unit
+    static constexpr int kHalfBytes = kHalves ? kUnitsInFlight * 2 * kOutFloats * 4 : 0;    // [unit in flight][half][row][batch entry]
     static constexpr int kOutBytes = kOutSlots * (kOutFloats * 4 + (int)sizeof(OutDesc));
     static constexpr int kFixed = kXSlots * kXSlotBytes + kOpRing * kOpBytes + 4 * kOpBytes +
-                                  kOutBytes + 512;
+                                  kOutBytes + kHalfBytes + 640;
     static constexpr int kPerStage = kStageBytes + (int)sizeof(UnitDesc) + 16 + 4;
     static constexpr int kAuto = (232448 - kFixed) / kPerStage;
     static constexpr int kStages = kAuto > 16 ? 16 : kAuto;
@@ -88,11 +93,13 @@ template <int BP> struct GemvSmem {
     static constexpr int oOpBuf = oOpRing + kOpRing * kOpBytes;   // GemvOp[2] producer, GemvOp[2] activation warp
     static constexpr int oOutData = oOpBuf + 4 * kOpBytes;   // float[kOutSlots][kOutFloats]
     static constexpr int oOutDesc = oOutData + kOutSlots * kOutFloats * 4;     // OutDesc[kOutSlots]
-    static constexpr int oBars = oOutDesc + kOutSlots * (int)sizeof(OutDesc);  // full[S], empty[S]
+    static constexpr int oHalf = oOutDesc + kOutSlots * (int)sizeof(OutDesc);   // float[kUnitsInFlight][2][kOutFloats]
+    static constexpr int oBars = oHalf + kHalfBytes;  // full[S], empty[S]
     static constexpr int oReleased = oBars + 2 * kStages * 8;        // u32[S]: consumer warps that released a stage, ever
     static constexpr int oCtl = oReleased + kStages * 4;             // x_ready[XS], x_pending[XS], flags[2], prep_cmd, pad
     static constexpr int oOutCtl = oCtl + 64;                        // out_fill[kOutSlots], out_gen[kOutSlots]
-    static constexpr int oXBars = (oOutCtl + 2 * kOutSlots * 4 + 16 + 7) / 8 * 8;   // (+ out_total) one mbarrier per activation slot
+    static constexpr int oHalfCtl = oOutCtl + 2 * kOutSlots * 4 + 16;          // u32 [unit in flight][tile]: halves delivered, units done
+    static constexpr int oXBars = (oHalfCtl + kUnitsInFlight * kUnitRowTiles * 8 + 7) / 8 * 8;   // (+ out_total) one mbarrier per activation slot
     static constexpr int kTotal = oXBars + 8 * kXSlots + 8;
     static_assert(kStages >= 4, "decode kernel: no room for a ring");
     static_assert(kOpRing >= kStages + 2, "an op's ring slot must outlive the units that refer to it");
@@ -165,16 +172,18 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
     volatile int* flags = x_pending + kXSlots;                                 // [0]: stop computing, [1]: stop everything
     volatile unsigned* out_fill = reinterpret_cast<volatile unsigned*>(smem + S::oOutCtl);   // consumer warps that filled a slot
     volatile unsigned* out_gen = out_fill + kOutSlots;                         // times the output warp drained a slot
+    volatile unsigned* half_ctl = reinterpret_cast<volatile unsigned*>(smem + S::oHalfCtl);
     volatile int* out_total = reinterpret_cast<volatile int*>(out_gen + kOutSlots);   // finishing units of this CTA (-1: not known yet)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S::kStages; s++) {
             mbar_init(bars + 8 * s, 1);
-            mbar_init(bars + 8 * (S::kStages + s), kWarpsPerUnit);
+            mbar_init(bars + 8 * (S::kStages + s), S::kWarpsPerUnit);
             released[s] = 0u;
         }
         for (int i = 0; i < kXSlots; i++) { x_ready[i] = 0; x_pending[i] = 0; mbar_init(xbars + 8 * i, 1); }
         for (int i = 0; i < kOutSlots; i++) { out_fill[i] = 0u; out_gen[i] = 0u; }
+        for (int i = 0; i < S::kUnitsInFlight * kUnitRowTiles * 2; i++) half_ctl[i] = 0u;
         out_total[0] = -1;
         flags[0] = 0; flags[1] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -353,7 +362,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                 __threadfence_block();
                 __syncwarp();
                 if (lane == 0) {
-                    x_pending[slot] = units * kWarpsPerUnit;
+                    x_pending[slot] = units * S::kWarpsPerUnit;
                     __threadfence_block();
                     x_ready[slot] = seg + 1;
                     __threadfence_block();
@@ -385,7 +394,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
         unsigned idle_it = 0u;
         for (;;) {
             // every decision that ends the loop is taken by lane 0 and broadcast: the lanes must leave together
-            const bool filled = lane < kOutSlots && lane % kOutputWarps == ow && out_fill[lane] == (unsigned)kWarpsPerUnit;
+            const bool filled = lane < kOutSlots && lane % kOutputWarps == ow && out_fill[lane] == (unsigned)kUnitRowTiles;
             const unsigned m = __ballot_sync(0xffffffffu, filled);
             unsigned done = 0u;
             if (m) {
@@ -474,10 +483,13 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
         }
     } else {
         // ================================================================== consumers
-        // Two warps share a unit, each computes one of its two 16-row tiles.
+        // Two or four warps share a unit (see GemvSmem), each computes one of its two 16-row tiles, over all or half of the columns.
         const int g = lane >> 2, c = lane & 3;
-        const int uidx = warp / kWarpsPerUnit;                       // which of the units in flight
-        const int tile = warp % kWarpsPerUnit;                       // this warp's row tile
+        const int uidx = warp / S::kWarpsPerUnit;                       // which of the units in flight
+        const int tile = warp % kUnitRowTiles, half = S::kHalves ? warp / kUnitRowTiles % 2 : 0;   // this warp's row tile and columns
+        volatile unsigned* delivered = half_ctl + (uidx * kUnitRowTiles + tile) * 2;   // halves of the unit at hand; [1]: units done
+        float* halves = reinterpret_cast<float*>(smem + S::oHalf) + uidx * 2 * S::kOutFloats;
+        unsigned turn = 0;                                           // units of this group so far
         int total = 0;                               // units of this CTA over the whole launch
         if (sa.cta_units) total = sa.cta_units[cta];
         else {
@@ -493,12 +505,12 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
         int stage = uidx % S::kStages;
         unsigned use = (unsigned)(uidx / S::kStages);
         const uint32_t opring_a = smem_u32(smem + S::oOpRing), desc_a = smem_u32(smem + S::oDesc);
-        for (int seq = uidx; seq < total && !stop; seq += kUnitsInFlight) {
+        for (int seq = uidx; seq < total && !stop; seq += S::kUnitsInFlight) {
             const uint32_t full = bars + 8 * stage, empty = bars + 8 * (S::kStages + stage);
             // a stage's uses are consumed strictly in order: wait for the release of the previous
             // use before trusting the parity of the full barrier
             bool ok = true;
-            if (use > 0) ok = smem_wait([&] { return released[stage] >= use * kWarpsPerUnit || flags[1]; });
+            if (use > 0) ok = smem_wait([&] { return released[stage] >= use * S::kWarpsPerUnit || flags[1]; });
             if (ok) ok = mbar_wait(full, use & 1u);
             if (!ok || flags[1]) {
                 if (lane == 0 && !ok) { atomicCAS(sa.status, 0, FQ_ERR_TIMEOUT); flags[0] = 1; flags[1] = 1; }
@@ -513,7 +525,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                 const uint32_t od = opring_a + u1.x * S::kOpBytes;
                 const uint4 o1 = lds128(od + 16);                                           // blob_read, variant, batch, n_chunks
                 const uint2 o0 = lds64(od + 8);                                             // partial
-                d.ch = (int)u0.x; d.rp = (int)u0.y; d.cnt = (int)u0.z * kBlobSteps; d.seg = (int)u0.w;
+                d.ch = (int)u0.x; d.rp = (int)u0.y; d.cnt = (int)u0.z * kBlobSteps / (S::kHalves ? 2 : 1); d.seg = (int)u0.w;
                 d.op_slot = (int)u1.x; d.oseq = (int)u1.y;
                 d.blob_read = (int)o1.x; d.variant = (int)o1.y; d.batch = (int)o1.z; d.n_chunks = (int)o1.w;
                 d.partial = reinterpret_cast<unsigned long long*>(((unsigned long long)o0.y << 32) | o0.x);
@@ -529,7 +541,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                     break;
                 }
                 if (flags[1]) { stop = true; break; }
-                if (tile == 0 && lane == 0) {
+                if (tile == 0 && half == 0 && lane == 0) {
                     const GemvOp& od = *reinterpret_cast<const GemvOp*>(opring + d.op_slot * S::kOpBytes);
                     OutDesc& q = odesc[oslot];
                     q.rp = d.rp; q.ch = d.ch; q.n_chunks = od.n_chunks; q.n_out = od.n_out; q.phase = od.phase; q.batch = od.batch;
@@ -551,7 +563,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
 
             float tot[4] = {0.f, 0.f, 0.f, 0.f};
             if (live)
-                unit_dispatch<BP>(d.variant, smem_u32(smem + S::oStages) + (uint32_t)stage * S::kStageBytes, d.cnt, (uint32_t)d.blob_read,
+                unit_dispatch<BP>(d.variant, smem_u32(smem + S::oStages) + (uint32_t)stage * S::kStageBytes, half * d.cnt, d.cnt, (uint32_t)d.blob_read,
                                   smem_u32(smem + S::oX) + (uint32_t)slot * S::kXSlotBytes, lane, tile, tot);
             __syncwarp();
             if (lane == 0) {
@@ -560,12 +572,43 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                 mbar_arrive(empty);                              // the stage may be refilled
                 atomicSub(const_cast<int*>(&x_pending[slot]), 1);   // one warp fewer needs the activation slot
             }
-            stage += kUnitsInFlight;
+            stage += S::kUnitsInFlight;
             while (stage >= S::kStages) { stage -= S::kStages; use++; }
             if (!live) continue;
 
             // ---- the row sums: tot[2 r + i] of lane (g, c) belongs to local row tile * 16 + g + 8 r, batch entry 2 c + i
             const int lr = tile * kTileRows + g;
+            // the two halves of the columns: whoever delivers the second one adds the first (the order does not change the sum)
+            if constexpr (S::kHalves) {
+                if (!smem_wait([&] { return delivered[1] >= turn || flags[1]; })) {        // the previous unit's have been taken
+                    if (lane == 0) { atomicCAS(sa.status, 0, FQ_ERR_TIMEOUT); flags[0] = 1; flags[1] = 1; }
+                }
+                if (__any_sync(0xffffffffu, flags[1] != 0)) { stop = true; break; }
+                turn++;
+                float* mine = halves + half * S::kOutFloats;
+                if (2 * c < BP) {
+                    *reinterpret_cast<float2*>(mine + lr * BP + 2 * c) = make_float2(tot[0], tot[1]);
+                    *reinterpret_cast<float2*>(mine + (lr + 8) * BP + 2 * c) = make_float2(tot[2], tot[3]);
+                }
+                __threadfence_block();
+                __syncwarp();
+                unsigned before = 0;
+                if (lane == 0) before = atomicAdd(const_cast<unsigned*>(&delivered[0]), 1u);
+                if (__shfl_sync(0xffffffffu, before, 0) == 0u) continue;
+                __threadfence_block();
+                const float* other = halves + (half ^ 1) * S::kOutFloats;
+                if (2 * c < BP) {
+                    const float2 o0 = *reinterpret_cast<const float2*>(other + lr * BP + 2 * c);
+                    const float2 o1 = *reinterpret_cast<const float2*>(other + (lr + 8) * BP + 2 * c);
+                    tot[0] += o0.x; tot[1] += o0.y; tot[2] += o1.x; tot[3] += o1.y;
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    delivered[0] = 0u;
+                    __threadfence_block();
+                    delivered[1] = turn;
+                }
+            }
             if (d.oseq >= 0) {
                 // this unit finishes its row pair: hand the sums to the output warps
                 float* o = odata + oslot * S::kOutFloats;
