@@ -49,6 +49,26 @@ const Variant* active_variant(const Layer& L, int bits)
 constexpr int kSplitBelowBlobsPerCta = 48;
 constexpr int kSplitAboveFields = 2;
 
+// Relative cost of a byte, x64, per variant (0..6 packed 2..8 bits, 7..13 nested 2..8 bits).
+unsigned deal_weight(int variant)
+{
+    static const unsigned w[kVariants] = {125, 112, 66, 78, 78, 84, 48,      // packed 2..8
+                                          108, 64, 64, 74, 74, 64, 64};      // nested 2..8 (per byte READ: whole 2-bit fields)
+    return variant >= 0 && variant < kVariants ? w[variant] : 64u;
+}
+
+// Time a CTA spends on one blob of an op, in arbitrary units: bytes x the relative cost of a byte of the op's
+// variant.  The 8-bit and 4-bit loops keep up with the CTA's share of HBM; variants with more fields per stored
+// bit are bound by the integer pipe and take longer per byte (per-CTA rates of uniform stacks, all CTAs busy:
+// 8 bits 48.8 GB/s, 4: 46.1, 5: 42.8, 6: 42.5, 7: 39.9, 3: 31.5, 2: 27.7; nested children 21 - 37 by field count).  The table
+// starts from the inverse rates; the 8-bit entry is lower than that because a CTA that streams 8-bit blobs speeds
+// up when its neighbours are compute-bound and leave it more of the HBM (tuned on the mixed 7B stack: the
+// unordered pass went from 4350 to 5380 GB/s, the ordered one from 1.525 to 1.465 ms).
+unsigned blob_cost(const GemvOp& op)
+{
+    return (unsigned)op.blob_read / 512u * deal_weight(op.variant);     // (blobs are multiples of 512 bytes)
+}
+
 // Fills the device descriptor of one decode op (everything except workspace pointers and unit_base).
 //   one : the op runs in the batch-1 kernel (gemv1); otherwise in the batch kernel, which also serves batch 1 for
 //         layers whose k_in exceeds what the batch-1 kernel keeps in shared memory
@@ -94,6 +114,7 @@ int fill_op(const Ctx* ctx, int layer, const uint16_t* x, uint16_t* y, int batch
     if (one && (batch != 1 || L.k_in > gemv1_max_k())) return FQ_ERR_SHAPE;                   // a strip's activations stay in shared memory
     op.phase = -1;
     op.rot = 0;
+    op.blob_cost = blob_cost(op);
     // a lone matrix is a few blobs per CTA: items of one 16-row tile spread them over twice as many consumer warps
     op.split = (one && fl.n > kSplitAboveFields && op.n_units < kSplitBelowBlobsPerCta * ctx->sm_count) ? 2 : 1;
     return FQ_OK;
@@ -617,7 +638,11 @@ int fq_gemv_batched(fq_ctx* ctx, int layer, const uint16_t* x_dev, int batch, ui
     rc = ensure_workspace(ctx, kPartialBase + pb + 256);
     if (rc != FQ_OK) return rc;
     op.partial = reinterpret_cast<unsigned long long*>(ctx->ws + kPartialBase);
-    return one ? launch_gemv1_single(ctx, op, (cudaStream_t)stream) : launch_gemv_single(ctx, op, (cudaStream_t)stream);
+    if (!one) return launch_gemv_single(ctx, op, (cudaStream_t)stream);
+    InlineOps ops;
+    ops.op[0] = op;
+    ops.op[0].blob_cost = 1;                               // one op: blobs are all alike
+    return launch_gemv1_inline(ctx, ops, 1, (cudaStream_t)stream);
 }
 
 int fq_gemv(fq_ctx* ctx, int layer, const uint16_t* x_dev, uint16_t* y_dev, void* stream)
@@ -634,26 +659,6 @@ int fq_gemv_static(fq_ctx* ctx, int layer, const uint16_t* x_dev, uint16_t* y_de
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return FQ_ERR_CUDA;
     return launch_gemv_static(ctx, op, op_partial_bytes(op, true, 1), (cudaStream_t)stream);
-}
-
-// Relative cost of a byte, x64, per variant (0..6 packed 2..8 bits, 7..13 nested 2..8 bits).
-static unsigned deal_weight(int variant)
-{
-    static const unsigned w[kVariants] = {125, 112, 66, 78, 78, 84, 48,      // packed 2..8
-                                          108, 64, 64, 74, 74, 64, 64};      // nested 2..8 (per byte READ: whole 2-bit fields)
-    return variant >= 0 && variant < kVariants ? w[variant] : 64u;
-}
-
-// Time a CTA spends on one blob of an op, in arbitrary units: bytes x the relative cost of a byte of the op's
-// variant.  The 8-bit and 4-bit loops keep up with the CTA's share of HBM; variants with more fields per stored
-// bit are bound by the integer pipe and take longer per byte (per-CTA rates of uniform stacks, all CTAs busy:
-// 8 bits 48.8 GB/s, 4: 46.1, 5: 42.8, 6: 42.5, 7: 39.9, 3: 31.5, 2: 27.7; nested children 21 - 37 by field count).  The table
-// starts from the inverse rates; the 8-bit entry is lower than that because a CTA that streams 8-bit blobs speeds
-// up when its neighbours are compute-bound and leave it more of the HBM (tuned on the mixed 7B stack: the
-// unordered pass went from 4350 to 5380 GB/s, the ordered one from 1.525 to 1.465 ms).
-static unsigned long long blob_cost(const GemvOp& op)
-{
-    return (unsigned long long)(unsigned)op.blob_read * deal_weight(op.variant);
 }
 
 int fq_gemv_stack(fq_ctx* ctx, int n_ops, const int* layers_host, const uint16_t* const* x_dev_host,
@@ -678,6 +683,36 @@ int fq_gemv_stack(fq_ctx* ctx, int n_ops, const int* layers_host, const uint16_t
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return FQ_ERR_CUDA;
     const cudaStream_t st = (cudaStream_t)stream;
+
+    // A few ops without dependencies (what a serving loop calls between its own kernels) travel as kernel parameters and are
+    // dealt to the CTAs on the device: no table to build, compare or upload.  Eight ops are 1.2 KB of parameters.
+    if (one && !phases_host && n_ops <= kInlineOps) {
+        InlineOps ops;
+        size_t ws_need = kPartialBase;
+        long long blobs = 0, cost = 0;
+        int strips = 0;
+        for (int i = 0; i < n_ops; i++) {
+            const int rc = fill_op(ctx, layers_host[i], x_dev_host[i], y_dev_host[i], 1, true, ops.op[i]);
+            if (rc != FQ_OK) return rc;
+            ws_need += (size_t)round_up((int64_t)op_partial_bytes(ops.op[i], true, 1), 256);
+            blobs += ops.op[i].n_units;
+            cost += (long long)ops.op[i].n_units * ops.op[i].blob_cost;
+            ops.op[i].rot = strips;                                // (the ops' first counters of shared strips)
+            strips += ops.op[i].n_rp;
+        }
+        if (cost < (1ll << 32)) {                                  // (the device deals in 32 bits)
+            const int rc = ensure_workspace(ctx, ws_need + 256);
+            if (rc != FQ_OK) return rc;
+            const long long grid = blobs < ctx->sm_count ? blobs : ctx->sm_count;
+            size_t poff = kPartialBase;
+            for (int i = 0; i < n_ops; i++) {
+                ops.op[i].partial = reinterpret_cast<unsigned long long*>(ctx->ws + poff);
+                poff += (size_t)round_up((int64_t)op_partial_bytes(ops.op[i], true, 1), 256);
+                ops.op[i].split = (ops.op[i].n_fields > kSplitAboveFields && blobs < (long long)kSplitBelowBlobsPerCta * grid) ? 2 : 1;
+            }
+            return launch_gemv1_inline(ctx, ops, n_ops, st);
+        }
+    }
 
     // The op table only depends on the arguments and the active configuration: the uploaded copy is
     // reused when every argument word is the same as in the call that built it.
@@ -752,7 +787,7 @@ int fq_gemv_stack(fq_ctx* ctx, int n_ops, const int* layers_host, const uint16_t
                 unsigned long long total = 0;
                 long long strips = 0;
                 for (int i = g0; i < g1; i++) {
-                    total += (unsigned long long)ops[i].n_units * blob_cost(ops[i]);
+                    total += (unsigned long long)ops[i].n_units * ops[i].blob_cost;
                     strips += ops[i].n_rp;
                 }
                 long long group_blobs = 0;
@@ -766,7 +801,7 @@ int fq_gemv_stack(fq_ctx* ctx, int n_ops, const int* layers_host, const uint16_t
                 const int rot = (int)((unsigned)group * 53u % (unsigned)grid);      // spreads the remainders
                 unsigned long long before = 0;
                 for (int i = g0; i < g1; i++) {
-                    const unsigned long long sz = blob_cost(ops[i]);
+                    const unsigned long long sz = ops[i].blob_cost;
                     const unsigned long long bytes = (unsigned long long)ops[i].n_units * sz;
                     const unsigned long long strip_bytes = (unsigned long long)ops[i].n_kb * sz;
                     for (int c = 0; c < grid; c++) {

@@ -11,6 +11,9 @@
 // its blobs of a strip in "units" of up to six (what one ring stage holds).  y[row] is always the sum of the per-blob sums in
 // blob order, whoever computed them, so results do not depend on how the op was dealt.
 //
+// (In a launch without dependency phases a shared strip is added up by whoever publishes its last blob sum instead, so that no
+// CTA waits for another; such launches need not be cooperative and overlap the previous kernel of the stream.)
+//
 // Roles of a CTA:
 //   producer warp   : walks the op list, streams units into a ring of shared-memory stages with bulk
 //                     asynchronous copies (cp.async.bulk + mbarrier tx counts; it runs ahead across op and
@@ -52,6 +55,7 @@ constexpr int kXSlots = 28;                            // activation blobs resid
 constexpr int kStripSlots = 5;                         // strips whose items are in flight
 constexpr int kMaxKb = 28;                             // blobs per strip, at most (k_in <= 14336)
 constexpr int kQD = 8;                                 // entries per consumer queue
+constexpr int kArrivedMax = 8192;                      // counters of shared strips (the area of the phase counters, not used at the same time)
 constexpr int kMaxPhasesDev = 1024;
 constexpr int kMaxOpsDev = 512;                        // ops of one launch (their per-CTA ranges sit in shared memory)
 
@@ -70,10 +74,11 @@ struct StripDesc {
     unsigned long long* partial;             // tagged blob sums of this strip in global memory: [blob][32 rows]
     int n_out, row_base;
     int n_kb, kb_lo, kb_hi;                  // blobs of the strip; [kb_lo, kb_hi) are computed by this CTA
-    int finish;                              // this CTA owns the first blob: it adds up and writes y
+    int finish;                              // this CTA owns the first blob (Args::arrived: all blobs): it adds up and writes y
     int phase;
     int expect;                              // items of this CTA in the strip
-    int pad[4];
+    int counter;                             // Args::arrived: which counter is this strip's
+    int pad[3];
 };
 static_assert(sizeof(StripDesc) == 64, "descriptor layout");
 
@@ -119,6 +124,8 @@ struct Args {
     int n_ops, n_phases;
     unsigned epoch;                        // tag of this launch's published blob sums (never 0)
     unsigned long long wait_ns;            // limit of every wait
+    bool whole_strips;                     // inline ops: no strip is cut
+    unsigned* arrived;                     // ops without dependencies (or null): blobs published, per shared strip
 };
 
 __device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n)
@@ -196,6 +203,32 @@ __device__ __forceinline__ bool wait_mbar(uint32_t bar, uint32_t parity, volatil
             if (mbar_try_wait(bar, parity)) return true;
         if (ctl[Smem::cAbort] || global_ns() - t0 > limit) return false;
     }
+}
+
+// The blobs of op oi that a CTA computes when the ops came as kernel parameters: the blobs of all ops are one sequence, every
+// CTA gets the same cost of it in one contiguous piece (the host deals longer lists by the same rule), rounded to whole
+// strips where that is asked for.
+__device__ CtaWork inline_work(const GemvOp* ops, int oi, int n_ops, int cta, int grid, bool whole_strips)
+{
+    unsigned before = 0, total = 0;                                      // (32 bits are enough: checked on the host)
+    for (int i = 0; i < n_ops; i++) {
+        const unsigned cost = (unsigned)ops[i].n_units * ops[i].blob_cost;
+        if (i < oi) before += cost;
+        total += cost;
+    }
+    const unsigned n_kb = (unsigned)ops[oi].n_kb, step = whole_strips ? n_kb : 1u, size = ops[oi].blob_cost * step;
+    const unsigned each = total / (unsigned)grid, rest = total - each * (unsigned)grid;
+    auto first_blob_at = [&](unsigned c) -> int {                        // first blob of the op in the pieces of CTAs c, c + 1, ...
+        const unsigned pos = each * c + rest * c / (unsigned)grid;
+        if (pos <= before) return 0;
+        return (int)min(((pos - before - 1u) / size + 1u) * step, (unsigned)ops[oi].n_units);
+    };
+    CtaWork w;
+    w.lo = first_blob_at((unsigned)cta);
+    w.hi = first_blob_at((unsigned)cta + 1);
+    w.rp_first = w.lo / ops[oi].n_kb;
+    w.rp_last = w.hi > w.lo ? (w.hi - 1) / ops[oi].n_kb : w.rp_first;
+    return w;
 }
 
 // ------------------------------------------------------------------------------- activation pre-processing
@@ -280,7 +313,7 @@ __device__ __forceinline__ void convert_blob(const uint4 (&raw)[2], uint8_t* xdi
 
 // ------------------------------------------------------------------------------- the kernel
 __global__ void __launch_bounds__(kThreads, 1)
-gemv1_kernel(const __grid_constant__ GemvOp single, const Args a)
+gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
 {
     using S = Smem;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -291,7 +324,7 @@ gemv1_kernel(const __grid_constant__ GemvOp single, const Args a)
     volatile unsigned* ctl = reinterpret_cast<volatile unsigned*>(smem + S::oCtl);
     unsigned char* fin_total = smem + S::oFinTot;
     const uint2* range = reinterpret_cast<const uint2*>(smem + S::oRange);
-    const GemvOp* ops = a.table ? a.table : &single;
+    const GemvOp* ops = a.table ? a.table : inl.op;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S::kStages; s++) {
@@ -310,7 +343,7 @@ gemv1_kernel(const __grid_constant__ GemvOp single, const Args a)
     for (int oi = threadIdx.x; oi < a.n_ops; oi += blockDim.x) {
         uint2 r;
         if (a.ranges) r = a.ranges[(long long)cta * a.n_ops + oi];
-        else r = pack_range(cta_work(ops[oi].n_units, ops[oi].n_kb, ops[oi].rot, cta, grid), ops[oi].n_kb);
+        else r = pack_range(inline_work(ops, oi, a.n_ops, cta, grid, a.whole_strips), ops[oi].n_kb);
         reinterpret_cast<uint2*>(smem + S::oRange)[oi] = r;
     }
     __syncthreads();
@@ -324,6 +357,24 @@ gemv1_kernel(const __grid_constant__ GemvOp single, const Args a)
         }
     }
     __syncthreads();
+    if (!a.table && warp < kCW) {
+        // launched while the previous kernel of the stream drains: ask for this CTA's blobs to be brought into the L2 meanwhile
+        for (int oi = 0; oi < a.n_ops; oi++) {
+            const GemvOp& op = ops[oi];
+            const StripOrder so(range[oi], op.n_kb);
+            for (int si = warp; si < so.n_strips; si += kCW) {
+                const int rp = so.strip(si);
+                int c0, c1;
+                so.chunks(rp, c0, c1);
+                if (c0 + lane < c1 && FQ_IN_BOUNDS(rp < op.n_rp && c1 <= op.n_kb, a.status))
+                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
+                                 ::"l"(op.store + ((long long)rp * op.n_kb + c0 + lane) * op.blob_stride), "r"(op.blob_read) : "memory");
+            }
+        }
+    }
+    // nothing above reads or writes what the previous kernel may still be working on
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (warp == kProducerWarp) {
         // ================================================================== producer
@@ -346,14 +397,14 @@ gemv1_kernel(const __grid_constant__ GemvOp single, const Args a)
             const uint8_t* store;
             unsigned long long* partial;
             uint16_t* y;
-            int blob_read, blob_stride, n_kb, cb, variant, n_out, phase, split;
+            int blob_read, blob_stride, n_kb, cb, variant, n_out, phase, split, rot;
             __device__ __forceinline__ void fetch(const GemvOp* ops, int oi, int n_ops)
             {
                 if (oi >= n_ops) return;
                 const GemvOp& o = ops[oi];
                 store = o.store; partial = o.partial; y = o.y; blob_read = o.blob_read; blob_stride = o.blob_stride;
                 n_kb = o.n_kb; cb = o.chunk_blobs; variant = o.variant; n_out = o.n_out; phase = o.phase;
-                split = o.split == 2 ? 2 : 1;
+                split = o.split == 2 ? 2 : 1; rot = o.rot;
             }
         };
         OpRegs nxt;
@@ -385,14 +436,16 @@ gemv1_kernel(const __grid_constant__ GemvOp single, const Args a)
                 }
                 if (!__shfl_sync(0xffffffffu, slot_ok, 0)) { stop = true; break; }   // (every loop exit is decided by lane 0)
                 {
-                    // the strip's descriptor: three lanes store 16 bytes each
+                    // the strip's descriptor: four lanes store 16 bytes each
                     unsigned long long* const sp = partial + (long long)rp * n_kb * 32;
                     uint4 d;
                     if (lane == 0) d = make_uint4((uint32_t)(uintptr_t)y, (uint32_t)((uintptr_t)y >> 32), (uint32_t)(uintptr_t)sp,
                                                   (uint32_t)((uintptr_t)sp >> 32));
                     else if (lane == 1) d = make_uint4((uint32_t)n_out, (uint32_t)(rp * (kBlobTiles * kTileRows)), (uint32_t)n_kb, (uint32_t)kb_lo);
-                    else d = make_uint4((uint32_t)kb_hi, c0 == 0 ? 1u : 0u, (uint32_t)phase, (uint32_t)((kb_hi - kb_lo) * split));
-                    if (lane < 3) sts128(sdesc_a + (uint32_t)sslot * 64u + (uint32_t)lane * 16u, d);
+                    else if (lane == 2) d = make_uint4((uint32_t)kb_hi, c0 == 0 && (!a.arrived || c1 == n_kb) ? 1u : 0u, (uint32_t)phase,
+                                                       (uint32_t)((kb_hi - kb_lo) * split));
+                    else d = make_uint4((uint32_t)(cur.rot + rp), 0u, 0u, 0u);
+                    if (lane < 4) sts128(sdesc_a + (uint32_t)sslot * 64u + (uint32_t)lane * 16u, d);
                     if (lane == 0) ctl[S::cStripBusy + sslot] = 1u;
                     __threadfence_block();                           // the descriptor before any item that refers to it
                     __syncwarp();
@@ -720,6 +773,30 @@ gemv1_kernel(const __grid_constant__ GemvOp single, const Args a)
                     if (row < d.n_out && FQ_IN_BOUNDS(row >= 0, a.status)) reinterpret_cast<__half*>(d.y)[row] = __float2half_rn(sum);
                 }
             }
+            if (!finish && a.arrived) {
+                // a shared strip of a launch without dependencies: whoever publishes the last blob sum adds all of them up, in
+                // blob order.  Nobody waits for a CTA that may not be running yet.
+                const int mine = d.kb_hi - d.kb_lo, n_kb = d.n_kb;
+                __threadfence();                                             // the sums of this CTA's items before the count
+                __syncwarp();
+                unsigned before = 0;
+                if (lane == 0 && FQ_IN_BOUNDS(d.counter >= 0 && d.counter < kArrivedMax, a.status)) before = atomicAdd(a.arrived + d.counter, (unsigned)mine);
+                before = __shfl_sync(0xffffffffu, before, 0);
+                if ((int)before + mine == n_kb) {
+                    __threadfence();
+                    float sum = 0.f;
+                    for (int q0 = 0; q0 < n_kb; q0 += 8) {
+                        unsigned long long wv[8];
+#pragma unroll
+                        for (int i = 0; i < 8; i++) wv[i] = q0 + i < n_kb ? ld_relaxed_u64(d.partial + (q0 + i) * 32 + lane) : 0ull;
+#pragma unroll
+                        for (int i = 0; i < 8; i++) if (q0 + i < n_kb) sum += __uint_as_float((unsigned)wv[i]);
+                    }
+                    const int row = d.row_base + lane;
+                    if (row < d.n_out && FQ_IN_BOUNDS(row >= 0, a.status)) reinterpret_cast<__half*>(d.y)[row] = __float2half_rn(sum);
+                    if (lane == 0) a.arrived[d.counter] = 0u;
+                }
+            }
             const int phase = d.phase;
             __syncwarp();
             if (lane == 0) {
@@ -754,7 +831,7 @@ gemv1_kernel(const __grid_constant__ GemvOp single, const Args a)
     }
 }
 
-int launch(Ctx* ctx, const GemvOp& single, const Args& a, long long total_units, cudaStream_t st)
+int launch(Ctx* ctx, const InlineOps& ops, const Args& a, long long total_units, cudaStream_t st)
 {
     static bool configured[64] = {};
     if (ctx->device >= 64) return FQ_ERR_ARG;
@@ -765,7 +842,17 @@ int launch(Ctx* ctx, const GemvOp& single, const Args& a, long long total_units,
     long long blocks = ctx->sm_count;
     if (total_units < blocks) blocks = total_units;
     if (blocks < 1) return FQ_OK;
-    void* args[] = {(void*)&single, (void*)&a};
+    if (a.arrived) {                                 // no CTA waits for another: set up while the previous kernel drains
+        cudaLaunchAttribute overlap{};
+        overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        overlap.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)blocks); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = Smem::kTotal;
+        cfg.stream = st; cfg.attrs = &overlap; cfg.numAttrs = 1;
+        FQ_CUDA_OK(cudaLaunchKernelEx(&cfg, gemv1_kernel, ops, a));
+        return FQ_OK;
+    }
+    void* args[] = {(void*)&ops, (void*)&a};
     // cooperative: CTAs wait (bounded) for each other's phase counts and published sums, so all of them
     // have to be resident together
     FQ_CUDA_OK(cudaLaunchCooperativeKernel((const void*)gemv1_kernel, dim3((unsigned)blocks), dim3(kThreads), args,
@@ -791,14 +878,27 @@ int gemv1_chunk_blobs(int blob_read_bytes)
     return c > kBlobsMax ? kBlobsMax : (c < 1 ? 1 : c);
 }
 
-int launch_gemv1_single(Ctx* ctx, const GemvOp& op, cudaStream_t st)
+int launch_gemv1_inline(Ctx* ctx, const InlineOps& ops, int n_ops, cudaStream_t st)
 {
     Args a{};
     a.status = ctx->status_dev;
-    a.n_ops = 1;
+    a.n_ops = n_ops;
     a.epoch = next_epoch(ctx->launch_epoch);
     a.wait_ns = ctx->wait_limit_ns;
-    return launch(ctx, op, a, op.n_units, st);
+    long long units = 0, strips = 0;
+    double bytes = 0;
+    for (int i = 0; i < n_ops; i++) {
+        units += ops.op[i].n_units;
+        strips += ops.op[i].n_rp;
+        bytes += (double)ops.op[i].n_units * ops.op[i].blob_read;
+    }
+    // Whole strips leave the CTAs less even, strips that are cut cost the exchange of their sums at the end of the launch (about
+    // 2.5 us): whole ones where the unevenness, streamed at 6.5 TB/s by all SMs, is less than that.  One matrix of 4096 x 11008 at
+    // 4 bits: 14.0 us cut, 10.6 us whole.
+    const double per_cta = (double)strips / ctx->sm_count, uneven = (double)((strips + ctx->sm_count - 1) / ctx->sm_count) - per_cta;
+    a.whole_strips = uneven / per_cta * bytes / 6.5e6 < 2.5;
+    if (strips <= kArrivedMax) a.arrived = reinterpret_cast<unsigned*>(ctx->ws);
+    return launch(ctx, ops, a, units, st);
 }
 
 int launch_gemv1_stack(Ctx* ctx, const StackHeader& hdr, const char* table_dev, cudaStream_t st)
@@ -816,8 +916,8 @@ int launch_gemv1_stack(Ctx* ctx, const StackHeader& hdr, const char* table_dev, 
     a.n_phases = hdr.n_phases;
     a.epoch = next_epoch(ctx->launch_epoch);
     a.wait_ns = ctx->wait_limit_ns;
-    GemvOp dummy{};
-    return launch(ctx, dummy, a, hdr.total_units, st);
+    static const InlineOps none{};
+    return launch(ctx, none, a, hdr.total_units, st);
 }
 
 // ------------------------------------------------------------------------------- allocation-free variant
@@ -858,7 +958,10 @@ int launch_gemv_static(Ctx* ctx, GemvOp op, size_t partial_bytes, cudaStream_t s
     if (e == 0u) e = epoch[ctx->device].fetch_add(1u) + 1u;      // 0 marks words that no launch has written
     a.epoch = e;
     a.wait_ns = ctx->wait_limit_ns;
-    return launch(ctx, op, a, op.n_units, st);
+    InlineOps ops{};
+    ops.op[0] = op;
+    ops.op[0].blob_cost = 1;                                             // one op: blobs are all alike
+    return launch(ctx, ops, a, op.n_units, st);
 }
 
 }  // namespace fq

@@ -50,8 +50,9 @@ struct GemvOp {
     int zero_adjust;             // subtracted from every zero point (mid-point fill of a nested child)
     int phase;                   // -1: no ordering
     int n_units;                 // n_chunks * n_rp
-    int rot;                     // rotation of the CTA blocks for this op (evens out remainders)
+    int rot;                     // rotation of the CTA blocks for this op (evens out remainders); inline ops: its first strip counter
     int split;                   // batch 1: consumer items per blob: 1 (both 16-row tiles) or 2 (one tile each)
+    unsigned blob_cost;          // batch 1: cost of a blob (512 bytes x cost of a byte of the variant)
 };
 static_assert(offsetof(GemvOp, blob_read) == 16 && offsetof(GemvOp, partial) == 8, "consumer block of the op descriptor");
 
@@ -136,7 +137,10 @@ size_t gemm_split_part_bytes(int sm_count);
 double gemm_split_us(const Ctx* ctx, int M, int n_out, int k_in);       // estimates of the time of a call
 double gemm_two_pass_us(const Ctx* ctx, int M, int n_out, int k_in);
 struct CtaWork;
-int launch_gemv1_single(Ctx* ctx, const GemvOp& op, cudaStream_t st);                // batch 1
+// batch 1, up to kInlineOps ops that depend on nothing in the same call: they travel as kernel parameters
+constexpr int kInlineOps = 8;
+struct InlineOps { GemvOp op[kInlineOps]; };
+int launch_gemv1_inline(Ctx* ctx, const InlineOps& ops, int n_ops, cudaStream_t st);
 // table_dev: [GemvOp x n_ops][int phase_total x max(n_phases,1)][uint2 strips x sm_count x n_ops]
 int launch_gemv1_stack(Ctx* ctx, const StackHeader& hdr, const char* table_dev, cudaStream_t st);
 int gemv1_max_phases();

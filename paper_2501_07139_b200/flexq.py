@@ -123,6 +123,8 @@ def fq_meta_bytes(n_out: int, k_in: int, group: int = 128) -> int:
 
 
 def _stream() -> int:
+    if torch.cuda.is_initialized():                      # (without building a Stream object: a call is a few microseconds in all)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return torch.cuda.current_stream().cuda_stream
 
 
