@@ -242,7 +242,8 @@ int fq_gemv_batched(fq_ctx* ctx, int layer, const uint16_t* x_dev, int batch, ui
  *       without gaps; an op of phase p does not read its x before every op of phase p-1 has
  *       written its y (weights of later ops are prefetched meanwhile).
  * Batch 1: at most 512 ops and 1024 phases per call (FQ_ERR_SHAPE otherwise).
- * The call builds a table (ops, and which strips every thread block computes) and uploads it from a
+ * A list of up to 8 ops at batch 1 without phases travels as kernel parameters.  Otherwise the call
+ * builds a table (ops, and which strips every thread block computes) and uploads it from a
  * pinned buffer; a call with the same arguments under the same configuration reuses the uploaded
  * table and only launches the kernel.  The workspace was sized by fq_pack_layer for lists that use
  * every layer at most once; a list that repeats layers may grow it (device allocation + sync). */
@@ -254,21 +255,20 @@ int fq_gemv_stack(fq_ctx* ctx, int n_ops, const int* layers_host,
  * token sequences):  Y[m][n] = sum_k X[m][k] * w^[n][k].
  *   X_dev bf16 [M][ldx >= k_in], Y_dev bf16 [M][ldy >= n_out], row-major, 16-byte aligned,
  *   ldx and ldy multiples of 8, 1 <= M <= 2^20.
- * One fused kernel: X tiles arrive by TMA, the stored blobs are dequantised inside the kernel
- * (w^ = (q - z) * s exactly in fp32, rounded once to bf16) into the shared-memory operand tiles of
- * the tensor cores (tcgen05, fp32 accumulation in TMEM), Y is rounded once to bf16.  Enqueues one
- * kernel on `stream` and encodes one tensor map on the host.  Shapes whose 256 x 256 output tiles would
- * leave the last wave of thread blocks mostly empty are cut into equal runs of (tile, K stage) work
- * instead; a tile shared by two blocks is then the fp32 sum of two partial accumulations (summation
- * order differs from the whole-tile case in the last bit), passed through a 38 MB workspace that the
- * context allocates the first time such a shape is used.  One fq_gemm at a time per context. */
+ * w^ = (q - z) * s exactly in fp32, rounded once to bf16; tensor cores (tcgen05, fp32 accumulation in
+ * TMEM); Y is rounded once to bf16.  Runs whichever of two ways is estimated to be the faster for the
+ * shape: one kernel that converts the weights on their way into the tensor cores, or the two passes of
+ * fq_gemm_two_pass, whose workspace (bf16 of the largest layer) the first such call allocates; where
+ * that is not possible (no memory, the stream is being captured) the first way serves every shape.
+ * Thread blocks may share an output tile, which is then the fp32 sum of their partial sums in K order
+ * (the last bit may differ from the other way's), through slots that belong to the context (29 MB).
+ * One fq_gemm at a time per context. */
 int fq_gemm(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int ldx,
             uint16_t* Y_dev, int ldy, void* stream);
 
-/* The same product computed in two passes, kept as the comparison point of the fused kernel: the
- * layer is first dequantised to bf16 into a workspace of n_out*k_in*2 bytes that the context owns
- * (grown with a device allocation when a larger layer is first used), then multiplied by a plain
- * tcgen05 GEMM.  Same arguments, same rounding points, same results up to the fp32 summation order. */
+/* The same product computed in two passes whatever the shape: the layer is first dequantised to bf16 into a workspace of n_out*k_in*2 bytes that the context owns
+ * (grown with a device allocation when a larger layer is first used), then multiplied by a tcgen05
+ * GEMM over pairs of SMs.  Same arguments, same rounding points, same results up to the fp32 summation order. */
 int fq_gemm_two_pass(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int ldx,
                      uint16_t* Y_dev, int ldy, void* stream);
 
