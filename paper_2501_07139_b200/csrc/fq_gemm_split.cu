@@ -345,7 +345,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_x, const SplitArgs a)
         Run run(a);
         Item it;
         for (; ok && run.next(it); local++) {
-            const int mb = it.tile % a.m_blocks, n = it.tile / a.m_blocks * kRows + trow;
+            const int mb = it.tile % a.m_blocks;
             const int tokens = min(a.tile_n, a.M - mb * a.tile_n);      // of the tile
             ok = __all_sync(0xffffffffu, g_wait<128>(tfull, (uint32_t)local & 1u, abort_flag));
             if (!ok) break;

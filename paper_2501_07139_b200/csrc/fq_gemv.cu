@@ -45,7 +45,7 @@ constexpr int kGemvThreads = (kConsumerWarps + 2 + kOutputWarps) * 32;     // 24
 constexpr int kUnitBytes = 17408;                      // bytes of one unit (whole blobs), at most: 2 x 4-bit or 1 x 8-bit blob
 constexpr int kBlobsMax = kXCols / 512;                // k blobs (512 columns) per chunk, at most
 constexpr int kOutSlots = 16;                          // finished units waiting for an output warp (it scans one slot per lane)
-constexpr int kXSlots = 4;                             // activation chunks kept in shared memory
+constexpr int kXSlots = 3;                             // activation chunks kept in shared memory (a fourth costs a stage of the ring: 1 % slower)
 
 // What the producer tells the consumers: once per op a copy of the op descriptor in a ring ...
 constexpr int kOpRing = 16;                            // > stages + 1: an op slot outlives the start of its last unit
