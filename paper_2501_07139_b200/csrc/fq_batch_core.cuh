@@ -8,6 +8,10 @@
 //   codes -> fp16: a byte q in the low mantissa bits under the exponent of 1024 is the fp16 number 1024 + q; codes that sit at
 //   bit p of their byte give 1024 + q * 2^p, and fma(., 2^-p, -(1024 * 2^-p + z)) is q - z exactly.  Which p costs the fewest
 //   shifts is chosen at compile time per k32 step.
+//
+//   The constant is exact for z below 1024, which covers every quantiser of up to eight bits; stored zero points have 16 bits.  Where a
+//   context holds higher ones, their upper bits are taken out of a unit before it is computed (unit_take_high_zeros), in a kernel of
+//   its own: a test, a mask or one more register in the usual one costs 2 - 7 % of the 13B stack at batch 8.
 #pragma once
 #include <cuda_fp16.h>
 
@@ -143,6 +147,39 @@ __device__ __forceinline__ void unit_compute(uint32_t stage, int first, int step
             for (int i = 0; i < 4; i++) tot[i] = fmaf(sc[i >> 1], acc[0][i] + acc[1][i], tot[i]);
         });
     }
+}
+
+// Takes the zero points of a unit (this warp's part of it: nobody else reads those words) down to their low ten bits; tot gets what
+// that leaves out, -s * (upper bits of z) * (sum of the activations) over the groups.  The sums come from MMAs whose weights are all
+// one, in the layout of tot.
+template <int BP>
+__device__ __forceinline__ void unit_take_high_zeros(uint32_t stage, int first, int steps, uint32_t blob_read, uint32_t xs, int lane, int tile,
+                                                     float (&tot)[4])
+{
+    constexpr uint32_t kOnes = 0x3c003c00u;                           // 1.0 twice
+    const int g = lane >> 2, c = lane & 3;
+    uint32_t xa = xs + (uint32_t)((g & (BP - 1)) * kXRowBytes + c * 8 + first * kStepCols * 2);
+#pragma unroll 1
+    for (int i = 2 * first; i < 2 * (first + steps); i++, xa += kGroup * 2) {     // one group at a time
+        const int ssl = i / 2 % kBlobSteps;
+        const uint32_t words = stage + (uint32_t)(i / 2 / kBlobSteps) * blob_read + (uint32_t)((ssl * kBlobTiles + tile) * 128 + g * 16 + (i & 1) * 8);
+        const uint2 m = lds64(words);                                 // rows g, g + 8
+        if (!__any_sync(0xffffffffu, ((m.x | m.y) >> 26) != 0u)) continue;
+        float sums[4] = {0.f, 0.f, 0.f, 0.f};
+        static_for<0, kGroup / 16>([&](auto H) {
+            const uint2 x = lds64<decltype(H)::value * 32>(xa);
+            mma_f16(sums, kOnes, kOnes, kOnes, kOnes, x.x, x.y);
+        });
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            const uint32_t w = e < 2 ? m.x : m.y;
+            const float share = __half2float(__ushort_as_half((unsigned short)(w & 0xffffu))) * (float)((w >> 16) & ~1023u);   // exact: 11 x 6 bits
+            tot[e] = fmaf(-share, sums[e], tot[e]);
+        }
+        if (c == 0) sts64(words, make_uint2(m.x & 0x03ffffffu, m.y & 0x03ffffffu));           // (all lanes have read them: the vote)
+    }
+    __syncwarp();
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the next copy into the stage comes after these stores
 }
 
 template <int BP>

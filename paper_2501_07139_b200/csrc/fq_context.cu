@@ -2,6 +2,7 @@
 // argument checks and dispatch to the kernels.
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include "fq_internal.cuh"
@@ -48,6 +49,40 @@ const Variant* active_variant(const Layer& L, int bits)
 // with half blobs, packed mixed 1.46 -> 1.55 ms, so only the many-field variants are cut).
 constexpr int kSplitBelowBlobsPerCta = 48;
 constexpr int kSplitAboveFields = 2;
+
+// Words of page-locked host memory in which the device leaves notes, one per context.  The page is allocated once for the process;
+// contexts beyond the first kNotes that live at a time, and all if there is no such memory, do without.
+class Notes {
+public:
+    unsigned* take()
+    {
+        std::lock_guard<std::mutex> lock(mutex_);
+        if (!tried_) {
+            tried_ = true;
+            void* p = nullptr;
+            if (cudaHostAlloc(&p, kNotes * sizeof(unsigned), cudaHostAllocPortable) == cudaSuccess) words_ = static_cast<unsigned*>(p);
+            else cudaGetLastError();
+        }
+        for (int i = 0; words_ && i < kNotes; i++)
+            if (!used_[i]) {
+                used_[i] = true;
+                words_[i] = 0u;
+                return words_ + i;
+            }
+        return nullptr;
+    }
+    void give_back(unsigned* word)                       // (nothing on the device may still write it)
+    {
+        std::lock_guard<std::mutex> lock(mutex_);
+        if (word) used_[word - words_] = false;
+    }
+private:
+    static constexpr int kNotes = 1024;
+    std::mutex mutex_;
+    bool tried_ = false, used_[kNotes] = {};
+    unsigned* words_ = nullptr;
+};
+Notes g_notes;
 
 // Relative cost of a byte, x64, per variant (0..6 packed 2..8 bits, 7..13 nested 2..8 bits).
 unsigned deal_weight(int variant)
@@ -219,6 +254,7 @@ int fq_create(fq_ctx** out, int device, int n_layers)
         delete ctx;
         return FQ_ERR_CUDA;
     }
+    ctx->note = g_notes.take();
     *out = ctx;
     return FQ_OK;
 }
@@ -237,6 +273,7 @@ int fq_destroy(fq_ctx* ctx)
             if (ctx->stage_done[i]) cudaEventDestroy(ctx->stage_done[i]);
         }
         if (ctx->gemm_ws) cudaFree(ctx->gemm_ws);
+        g_notes.give_back(ctx->note);
         for (void* p : ctx->owned) cudaFree(p);
         for (Layer& L : ctx->layers)
             for (Variant& v : L.var)
@@ -308,9 +345,10 @@ int fq_pack_layer(fq_ctx* ctx, int layer, int n_out, int k_in, int bits, int gro
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return FQ_ERR_CUDA;
     const FieldList fl = fmt == FQ_FMT_PLANES ? plane_fields(8) : packed_fields(bits);
-    const int rc = launch_pack(codes_dev, scales_dev, zeros_dev, n_out, k_in, bits, fl, store_out_dev,
+    const int rc = launch_pack(codes_dev, scales_dev, zeros_dev, n_out, k_in, bits, fl, store_out_dev, high_zeros_word(ctx),
                                (cudaStream_t)stream);
     if (rc != FQ_OK) return rc;
+    ctx->stored++;
     const bool first_variant = !L.registered;
     L.registered = true;
     L.n_out = n_out; L.k_in = k_in; L.fmt = fmt;
@@ -456,11 +494,13 @@ int fq_transition_swap(fq_ctx* ctx, const uint8_t* to_bits_host, int n_layers, i
         if (!nv.present) {
             void* p = nullptr;
             if (cudaMallocAsync(&p, nbytes, st) != cudaSuccess) { ctx->config_epoch++; return FQ_ERR_CUDA; }
-            if (cudaMemcpyAsync(p, nv.host, nbytes, cudaMemcpyHostToDevice, st) != cudaSuccess) {
+            if (cudaMemcpyAsync(p, nv.host, nbytes, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+                launch_find_high_zeros(p, L.n_out, L.k_in, b1, high_zeros_word(ctx), st) != FQ_OK) {
                 cudaFreeAsync(p, st);
                 ctx->config_epoch++;
                 return FQ_ERR_CUDA;
             }
+            ctx->stored++;
             nv.store = p; nv.present = true; nv.swap_owned = true;
             rep.bytes_loaded += nbytes;
             resident_extra += nbytes;
@@ -570,16 +610,19 @@ int fq_load(fq_ctx* ctx, const char* path)
                 if (!get(stage.data(), n)) rc = FQ_ERR_IO;
                 else if (cudaMemcpy(static_cast<char*>(dev) + off, stage.data(), n, cudaMemcpyHostToDevice) != cudaSuccess) rc = FQ_ERR_CUDA;
             }
+            if (rc == FQ_OK) rc = launch_find_high_zeros(dev, L.n_out, L.k_in, b, high_zeros_word(ctx), nullptr);
             L.var[b].present = true;
             L.var[b].store = dev;
         }
     }
+    if (rc == FQ_OK && cudaStreamSynchronize(nullptr) != cudaSuccess) rc = FQ_ERR_CUDA;
     if (rc != FQ_OK) {                                   // a failing call changes nothing
         for (void* p : bufs) cudaFree(p);
         return rc;
     }
     for (uint32_t i = 0; i < head[0]; i++) ctx->layers[i] = loaded[i];
     ctx->owned.insert(ctx->owned.end(), bufs.begin(), bufs.end());
+    ctx->stored++;
     ctx->config_epoch++;
     ctx->stack_valid = false;
     return FQ_OK;

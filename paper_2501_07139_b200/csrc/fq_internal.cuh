@@ -69,7 +69,7 @@ struct Ctx {
     // workspace shared by all calls on this context
     char* ws = nullptr;          // device
     size_t ws_bytes = 0;
-    int* status_dev = nullptr;   // device status word
+    int* status_dev = nullptr;   // device status word, and behind it the word of high_zeros_word()
     // stack-call staging
     char* stack_dev = nullptr;   // device copy of the op table
     size_t stack_dev_bytes = 0;
@@ -79,6 +79,8 @@ struct Ctx {
     char* fused_ws = nullptr;            // prefill: counters, then two fp32 tile slots per SM (part of the allocation of status_dev)
     std::vector<void*> owned;    // device buffers allocated by fq_load, freed by fq_destroy
     uint64_t config_epoch = 0;
+    unsigned stored = 1;         // counts the calls that store weights
+    unsigned* note = nullptr;    // host word that the device can write (or null): see zeros_are_low in fq_gemv.cu
     unsigned launch_epoch = 0;   // tag of the split-K partials of the latest decode launch (never 0)
     // the op list that is currently uploaded: every argument word of the call that built it
     std::vector<uint64_t> stack_sig;
@@ -93,6 +95,9 @@ struct Ctx {
     unsigned long long wait_limit_ns = 2000000000ull;   // limit of every device-side wait
 };
 
+// Device word that is not 0 once a zero point above 1023 has been stored by any call on the context (it is never cleared).
+inline unsigned* high_zeros_word(const Ctx* ctx) { return reinterpret_cast<unsigned*>(ctx->status_dev) + 1; }
+
 // Bytes of device workspace for `n_ops` ops whose split-K needs are summed by the caller.
 int ensure_workspace(Ctx* ctx, size_t bytes);
 
@@ -100,7 +105,9 @@ int ensure_workspace(Ctx* ctx, size_t bytes);
 int launch_quantize(const float* w, int n_out, int k_in, int bits, uint8_t* codes, uint16_t* scales,
                     uint16_t* zeros, cudaStream_t st);
 int launch_pack(const uint8_t* codes, const uint16_t* scales, const uint16_t* zeros, int n_out, int k_in,
-                int stored_bits, const FieldList& fl, void* store, cudaStream_t st);
+                int stored_bits, const FieldList& fl, void* store, unsigned* high_zeros, cudaStream_t st);
+// Looks through a stored variant that came from elsewhere (a file, host memory) for what launch_pack notes in high_zeros.
+int launch_find_high_zeros(const void* store, int n_out, int k_in, int stored_bits, unsigned* high_zeros, cudaStream_t st);
 int launch_export_packed(const void* store, int n_out, int k_in, int bits, const FieldList& fl,
                          uint32_t* out, cudaStream_t st);
 int launch_export_planes(const void* store, int n_out, int k_in, int bits, const FieldList& fl,

@@ -182,6 +182,7 @@ struct StoreArgs {
     int stored_bits;               // bits of the stored variant (size of its blobs)
     FieldList fl;                  // fields that are written
     bool wide;                     // codes are 16-byte aligned (rows are multiples of 128 bytes)
+    unsigned* high_zeros;          // set where a zero point is above 1023
 };
 
 constexpr int kPackThreads = kBlobSteps * kBlobTiles * 32;
@@ -240,6 +241,7 @@ __global__ void __launch_bounds__(kPackThreads) pack_kernel(const __grid_constan
             const float z = __half2float(__ushort_as_half(a.zeros[n * a.groups + g]));
             const unsigned zi = (unsigned)fminf(fmaxf(rintf(z), 0.f), 65535.f);
             v = (unsigned)a.scales[n * a.groups + g] | (zi << 16);
+            if (zi > 1023u) *a.high_zeros = 1u;
         }
         reinterpret_cast<uint32_t*>(blob)[t] = v;
         static_assert(kBlobMetaBytes == 4 * kPackThreads, "one scale/zero word per thread");
@@ -279,9 +281,10 @@ static unsigned grid_for(long long total)
 }
 
 int launch_pack(const uint8_t* codes, const uint16_t* scales, const uint16_t* zeros, int n_out, int k_in,
-                int stored_bits, const FieldList& fl, void* store, cudaStream_t st)
+                int stored_bits, const FieldList& fl, void* store, unsigned* high_zeros, cudaStream_t st)
 {
     StoreArgs a{};
+    a.high_zeros = high_zeros;
     a.codes = codes; a.scales = scales; a.zeros = zeros; a.store = (uint8_t*)store;
     a.n_out = n_out; a.k_in = k_in; a.n_kb = k_blobs(k_in); a.groups = k_in / kGroup;
     a.stored_bits = stored_bits; a.fl = fl;
@@ -289,6 +292,24 @@ int launch_pack(const uint8_t* codes, const uint16_t* scales, const uint16_t* ze
     const long long blobs = (long long)row_pairs(n_out) * a.n_kb;
     if (blobs > 0x7fffffffll) return FQ_ERR_SHAPE;
     pack_kernel<<<(unsigned)blobs, kPackThreads, 0, st>>>(a);
+    FQ_CUDA_OK(cudaGetLastError());
+    return FQ_OK;
+}
+
+// Scale/zero words are the first kBlobMetaBytes of every blob.
+__global__ void __launch_bounds__(256) find_high_zeros_kernel(const uint8_t* store, long long blobs, int blob_stride, unsigned* high_zeros)
+{
+    constexpr int kWords = kBlobMetaBytes / 16;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < blobs * kWords; i += (long long)gridDim.x * blockDim.x) {
+        const uint4 m = *reinterpret_cast<const uint4*>(store + i / kWords * blob_stride + i % kWords * 16);
+        if (((m.x | m.y | m.z | m.w) >> 26) != 0u) *high_zeros = 1u;
+    }
+}
+
+int launch_find_high_zeros(const void* store, int n_out, int k_in, int stored_bits, unsigned* high_zeros, cudaStream_t st)
+{
+    const long long blobs = (long long)row_pairs(n_out) * k_blobs(k_in);
+    find_high_zeros_kernel<<<grid_for(blobs * (kBlobMetaBytes / 16)), 256, 0, st>>>((const uint8_t*)store, blobs, blob_bytes(stored_bits), high_zeros);
     FQ_CUDA_OK(cudaGetLastError());
     return FQ_OK;
 }

@@ -104,6 +104,10 @@ __device__ __forceinline__ void sts128(uint32_t a, uint4 v)
 {
     asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
+__device__ __forceinline__ void sts64(uint32_t a, uint2 v)
+{
+    asm volatile("st.shared.v2.u32 [%0], {%1,%2};" ::"r"(a), "r"(v.x), "r"(v.y) : "memory");
+}
 // L2 eviction policies: weights are streamed once per pass (evict first), activations, outputs and the
 // small tables are re-read soon (evict last), so that the stream does not flush them out of the L2.
 __device__ __forceinline__ unsigned long long l2_policy_evict_first()
