@@ -451,9 +451,11 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                     const int row = d.rp * (kUnitRowTiles * kTileRows) + lane;
                     __half* y = reinterpret_cast<__half*>(d.y);
                     if (row < d.n_out) {
+                        // sums of numbers stay finite: an infinite one comes from an activation that is none, and such a one makes
+                        // every output of its batch entry NaN (as the batch-1 kernel does, and fq_gemv promises)
 #pragma unroll
                         for (int b = 0; b < BP; b++)
-                            if (b < d.batch) y[(long long)b * d.n_out + row] = __float2half_rn(sum[b]);
+                            if (b < d.batch) y[(long long)b * d.n_out + row] = __float2half_rn(fmaf(sum[b], 0.f, sum[b]));
                     }
                     done |= 1u << s;
                 }

@@ -1,10 +1,11 @@
-"""Values of the batch decode kernel at the edges of what the calls accept: zero points of any size."""
+"""Values of the batch decode kernel at the edges of what the calls accept: zero points of any size, activations
+that are no numbers."""
 import numpy as np
 import pytest
 import torch
 
 from oracle import fq_oracle as O
-from fq_testlib import bits_of, f64_of, make_layer, to_dev, x_fp16
+from fq_testlib import GEMV_TOL, bits_of, f64_of, make_layer, to_dev, x_fp16
 
 pytestmark = pytest.mark.gpu
 
@@ -96,3 +97,30 @@ def test_zero_points_that_come_later(tmp_path):
         check(swapped, 0, want)
     for f in (fq, loaded, swapped):
         f.fq_destroy()
+
+@pytest.mark.parametrize("bad", [float("inf"), float("-inf"), float("nan")])
+@pytest.mark.parametrize("batch", [1, 2, 4, 5, 8])
+def test_an_activation_that_is_no_number(batch, bad):
+    """One infinite or NaN activation makes every output of its batch entry NaN and leaves the other entries alone, wherever it
+    stands: in the last columns of a layer that ends inside a blob, and in a layer that is too wide for the batch-1 kernel, where one
+    entry takes the same way.  A second op follows in the same launch: nothing of it is touched."""
+    import paper_2501_07139_b200 as P
+    k = 16384 if batch == 1 else 1408
+    fq = P.FlexQ(2)
+    layers = [make_layer(135, 0, 70, k, 4), make_layer(135, 1, 33, k, 8)]
+    for i, (l, bits) in enumerate(zip(layers, (4, 8))):
+        fq.fq_pack_layer(i, *to_dev(*l), bits, P.FQ_FMT_PACKED)
+    xs = [x_fp16(135, i, batch, k).cuda() for i in range(2)]
+    entry = batch - 1
+    for at in (3, k - 1):
+        x = xs[0].clone()
+        x[entry, at] = bad
+        ys = [torch.zeros((batch, n), dtype=torch.float16, device="cuda") for n in (70, 33)]
+        fq.fq_gemv_stack([0, 1], [x, xs[1]], ys, [0, 1], batch)
+        assert fq.fq_status() == 0
+        assert torch.isnan(ys[0][entry].float()).all()
+        want = [O.gemv(*l, bits, bits_of(v)) for l, bits, v in zip(layers, (4, 8), xs)]
+        for b in range(batch):
+            assert b == entry or O.rel_l2(f64_of(ys[0])[b], want[0][b]) <= GEMV_TOL
+            assert O.rel_l2(f64_of(ys[1])[b], want[1][b]) <= GEMV_TOL
+    fq.fq_destroy()
