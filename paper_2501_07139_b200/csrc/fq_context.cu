@@ -194,6 +194,23 @@ static bool allocate_status(Ctx* ctx)
     return cudaMemset(p, 0, kHead + (ctx->fused_ws ? counts : 0)) == cudaSuccess;
 }
 
+// Is the work that is enqueued on `st` recorded into a graph?
+static bool is_capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
+// Lets go of device memory that has been replaced: at fq_destroy if a graph may hold its address, else as soon as nothing uses it.
+static void release_workspace(Ctx* ctx, void* p, bool captured)
+{
+    if (!p) return;
+    if (captured || cudaDeviceSynchronize() != cudaSuccess) ctx->owned.push_back(p);
+    else cudaFree(p);
+}
+
 int ensure_workspace(Ctx* ctx, size_t bytes)
 {
     if (bytes <= ctx->ws_bytes) return FQ_OK;
@@ -904,30 +921,36 @@ int fq_gemv_stack(fq_ctx* ctx, int n_ops, const int* layers_host, const uint16_t
                       : launch_gemv_stack(ctx, ctx->stack_hdr, ctx->stack_dev, batch, st);
 }
 
-static bool may_allocate(cudaStream_t st)
+// Room for the bf16 copy of one layer; the first call asks for that of the largest layer of the context.  A graph may hold the
+// address of the old room (a call was captured that used it): that one is kept until fq_destroy, which happens at most once per
+// capture.  The new room is there before the old one goes.  A size that was not to be had is not asked for again (unless there
+// is no other way: `retry`) before the configuration changes, which is when memory comes free.
+static bool dequant_workspace(fq_ctx* ctx, cudaStream_t st, size_t need, bool retry)
 {
-    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone) return true;
-    cudaGetLastError();
-    return false;
-}
-
-// Room for the bf16 copy of one layer; the first call asks for that of the largest layer of the context.
-static bool dequant_workspace(fq_ctx* ctx, cudaStream_t st, size_t need)
-{
-    if (need <= ctx->gemm_ws_bytes) return true;
-    if (!may_allocate(st) || cudaDeviceSynchronize() != cudaSuccess) return false;
-    size_t most = need;
-    for (const Layer& L : ctx->layers)
-        if (L.registered && (size_t)L.n_out * L.k_in * 2 > most) most = (size_t)L.n_out * L.k_in * 2;
-    if (ctx->gemm_ws) cudaFree(ctx->gemm_ws);
-    ctx->gemm_ws = nullptr; ctx->gemm_ws_bytes = 0;
-    for (const size_t bytes : {most, need}) {
-        if (cudaMalloc(&ctx->gemm_ws, bytes) == cudaSuccess) { ctx->gemm_ws_bytes = bytes; return true; }
-        cudaGetLastError();
-        ctx->gemm_ws = nullptr;
+    const bool captured = is_capturing(st);
+    if (need > ctx->gemm_ws_bytes) {
+        if (captured || (!retry && ctx->gemm_ws_refused_at == ctx->config_epoch && need >= ctx->gemm_ws_refused)) return false;
+        size_t most = need;
+        for (const Layer& L : ctx->layers)
+            if (L.registered && (size_t)L.n_out * L.k_in * 2 > most) most = (size_t)L.n_out * L.k_in * 2;
+        void* room = nullptr;
+        size_t got = 0;
+        for (const size_t bytes : {most, need}) {
+            if (cudaMalloc(&room, bytes) == cudaSuccess) { got = bytes; break; }
+            cudaGetLastError();
+        }
+        if (!got) {
+            ctx->gemm_ws_refused = need;
+            ctx->gemm_ws_refused_at = ctx->config_epoch;
+            return false;
+        }
+        release_workspace(ctx, ctx->gemm_ws, ctx->gemm_ws_captured);
+        ctx->gemm_ws = static_cast<char*>(room);
+        ctx->gemm_ws_bytes = got;
+        ctx->gemm_ws_captured = false;
     }
-    return false;
+    ctx->gemm_ws_captured = ctx->gemm_ws_captured || captured;
+    return true;
 }
 
 static int gemm_common(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int ldx, uint16_t* Y_dev, int ldy, void* stream,
@@ -952,7 +975,7 @@ static int gemm_common(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int
     // every tile of up to 192 tokens, or once for all tokens in a pass of their own.  Both estimates are fits to measured times
     // (within about 15 %); the second way needs room for a bf16 copy of the layer.
     const bool two_pass = !fused || gemm_two_pass_us(ctx, M, L.n_out, L.k_in) < gemm_split_us(ctx, M, L.n_out, L.k_in);
-    if (two_pass && dequant_workspace(ctx, st, (size_t)L.n_out * L.k_in * 2))
+    if (two_pass && dequant_workspace(ctx, st, (size_t)L.n_out * L.k_in * 2, !fused))
         return launch_gemm(ctx, v->store, stride, fl, zero_adjust, L.n_out, L.k_in, X_dev, M, ldx, Y_dev, ldy, ctx->gemm_ws, st);
     if (!fused) return FQ_ERR_CUDA;
     // counters and slots for the sums of tiles that several CTAs share; without them the tiles stay whole

@@ -76,8 +76,11 @@ struct Ctx {
     // prefill: dequantised bf16 copy of the layer being multiplied
     char* gemm_ws = nullptr;
     size_t gemm_ws_bytes = 0;
+    bool gemm_ws_captured = false;       // a captured graph holds the address of gemm_ws
+    size_t gemm_ws_refused = 0;          // size that could not be had, under this configuration
+    uint64_t gemm_ws_refused_at = ~0ull;
     char* fused_ws = nullptr;            // prefill: counters, then two fp32 tile slots per SM (part of the allocation of status_dev)
-    std::vector<void*> owned;    // device buffers allocated by fq_load, freed by fq_destroy
+    std::vector<void*> owned;    // device buffers freed by fq_destroy: those of fq_load, workspaces that graphs may hold
     uint64_t config_epoch = 0;
     unsigned stored = 1;         // counts the calls that store weights
     unsigned* note = nullptr;    // host word that the device can write (or null): see zeros_are_low in fq_gemv.cu
