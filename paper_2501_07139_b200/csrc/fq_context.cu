@@ -216,11 +216,11 @@ int ensure_workspace(Ctx* ctx, size_t bytes)
     if (bytes <= ctx->ws_bytes) return FQ_OK;
     const size_t want = (size_t)round_up((int64_t)(bytes + bytes / 2), 1 << 20);
     char* p = nullptr;
-    FQ_CUDA_OK(cudaDeviceSynchronize());
     FQ_CUDA_OK(cudaMalloc(&p, want));
     if (cudaMemset(p, 0, want) != cudaSuccess) { cudaFree(p); return FQ_ERR_CUDA; }
     FQ_CUDA_OK(cudaDeviceSynchronize());
-    if (ctx->ws) cudaFree(ctx->ws);
+    release_workspace(ctx, ctx->ws, ctx->ws_used);             // (a size half as much again each time: what is kept is bounded)
+    if (ctx->ws_used) ctx->ws_kept.push_back(ctx->ws);
     ctx->ws = p;
     ctx->ws_bytes = want;
     ctx->stack_valid = false;          // cached op tables point into the old workspace
@@ -678,6 +678,7 @@ int fq_status(fq_ctx* ctx)
         // counters may have been left half-way: start from a clean workspace
         FQ_CUDA_OK(cudaMemset(ctx->status_dev, 0, sizeof(int)));
         FQ_CUDA_OK(cudaMemset(ctx->ws, 0, ctx->ws_bytes));
+        for (char* ws : ctx->ws_kept) FQ_CUDA_OK(cudaMemset(ws, 0, kPartialBase));      // (their counters)
         if (ctx->fused_ws) FQ_CUDA_OK(cudaMemset(ctx->fused_ws, 0, gemm_split_flag_bytes(ctx->sm_count)));
         FQ_CUDA_OK(cudaDeviceSynchronize());
     }
@@ -698,6 +699,7 @@ int fq_gemv_batched(fq_ctx* ctx, int layer, const uint16_t* x_dev, int batch, ui
     rc = ensure_workspace(ctx, kPartialBase + pb + 256);
     if (rc != FQ_OK) return rc;
     op.partial = reinterpret_cast<unsigned long long*>(ctx->ws + kPartialBase);
+    ctx->ws_used = true;
     if (!one) return launch_gemv_single(ctx, op, (cudaStream_t)stream);
     InlineOps ops;
     ops.op[0] = op;
@@ -770,6 +772,7 @@ int fq_gemv_stack(fq_ctx* ctx, int n_ops, const int* layers_host, const uint16_t
                 poff += (size_t)round_up((int64_t)op_partial_bytes(ops.op[i], true, 1), 256);
                 ops.op[i].split = (ops.op[i].n_fields > kSplitAboveFields && blobs < (long long)kSplitBelowBlobsPerCta * grid) ? 2 : 1;
             }
+            ctx->ws_used = true;
             return launch_gemv1_inline(ctx, ops, n_ops, st);
         }
     }
@@ -904,10 +907,10 @@ int fq_gemv_stack(fq_ctx* ctx, int n_ops, const int* layers_host, const uint16_t
                 }
         }
         if (ctx->stack_dev_bytes < table_bytes) {
-            FQ_CUDA_OK(cudaDeviceSynchronize());
-            if (ctx->stack_dev) cudaFree(ctx->stack_dev);
-            ctx->stack_dev = nullptr; ctx->stack_dev_bytes = 0;
-            FQ_CUDA_OK(cudaMalloc(&ctx->stack_dev, 2 * table_bytes));
+            char* p = nullptr;
+            FQ_CUDA_OK(cudaMalloc(&p, 2 * table_bytes));
+            release_workspace(ctx, ctx->stack_dev, true);
+            ctx->stack_dev = p;
             ctx->stack_dev_bytes = 2 * table_bytes;
         }
         FQ_CUDA_OK(cudaMemcpyAsync(ctx->stack_dev, host, table_bytes, cudaMemcpyHostToDevice, st));
@@ -917,6 +920,7 @@ int fq_gemv_stack(fq_ctx* ctx, int n_ops, const int* layers_host, const uint16_t
         ctx->stack_sig.swap(sig);
         ctx->stack_valid = true;
     }
+    ctx->ws_used = true;
     return one ? launch_gemv1_stack(ctx, ctx->stack_hdr, ctx->stack_dev, st)
                       : launch_gemv_stack(ctx, ctx->stack_hdr, ctx->stack_dev, batch, st);
 }

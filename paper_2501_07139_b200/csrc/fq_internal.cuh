@@ -69,6 +69,8 @@ struct Ctx {
     // workspace shared by all calls on this context
     char* ws = nullptr;          // device
     size_t ws_bytes = 0;
+    bool ws_used = false;        // a launch has used a workspace: a graph may hold its address (asking costs 0.1 us a call)
+    std::vector<char*> ws_kept;  // replaced workspaces that graphs may hold (freed with `owned`)
     int* status_dev = nullptr;   // device status word, and behind it the word of high_zeros_word()
     // stack-call staging
     char* stack_dev = nullptr;   // device copy of the op table
