@@ -24,8 +24,8 @@
 // A whole stack of layers runs as one launch.  Every op's units are dealt to the CTAs in
 // contiguous, K-chunk-major blocks (a CTA needs the activations of one or two chunks only);
 // the producer runs ahead across op boundaries because weights do not depend on activations.
-// Every wait has a time limit; when one runs out the kernel records FQ_ERR_TIMEOUT, stops
-// computing, drains its copies and returns.
+// Every wait has a time limit (fq_set_wait_limit_ns); when one runs out the kernel records FQ_ERR_TIMEOUT, stops
+// computing, stays until its copies have landed and returns.
 #include <cuda_fp16.h>
 
 #include "fq_batch_core.cuh"
@@ -136,7 +136,15 @@ struct StackArgs {
     const unsigned* high_zeros;            // not 0: some stored zero point is above 1023
     unsigned* note;                        // host memory (or null): the first CTA notes there what it found ...
     unsigned stored;                       // ... and as of which state of the context
+    unsigned long long wait_ns;            // limit of every wait
 };
+
+// A wait ran out: stops every role of the CTA.
+__device__ __forceinline__ void give_up(int* status, volatile int* flags)
+{
+    atomicCAS(status, 0, FQ_ERR_TIMEOUT);
+    flags[0] = 1; flags[1] = 1;
+}
 
 // Warp-cooperative fetch of op descriptors with one op of look-ahead: the words of op i+1 travel
 // while op i is processed.
@@ -255,9 +263,8 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                             if (wraps > 0 && !mbar_try_wait(empty, (wraps - 1u) & 1u)) {
                                 // the ring is full: the usual case when the consumers wait for activations
                                 if (flags[1]) ok = 0;
-                                else if (!mbar_wait(empty, (wraps - 1u) & 1u)) {
-                                    atomicCAS(sa.status, 0, FQ_ERR_TIMEOUT);
-                                    flags[0] = 1; flags[1] = 1;
+                                else if (!mbar_wait(empty, (wraps - 1u) & 1u, sa.wait_ns)) {
+                                    give_up(sa.status, flags);
                                     ok = 0;
                                 }
                             }
@@ -277,7 +284,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                         // transaction stays pending, the status word ends every wait
                         if (!FQ_IN_BOUNDS(rp >= 0 && rp < n_rp && kb0 >= 0 && kb0 + nb <= n_kb && bytes <= (uint32_t)S::kStageBytes,
                                           sa.status)) {
-                            if (lane == 0) { flags[0] = 1; flags[1] = 1; }
+                            if (lane == 0) give_up(sa.status, flags);
                             stop = true;
                             break;
                         }
@@ -302,6 +309,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
             fetch.store(&opbuf[(oi + 1) & 1], lane);
             __syncwarp();
         }
+        if (stop) let_copies_land();
         if (lane == 0 && !stop) out_total[0] = oseq;                // the output warps may leave after this many
     } else if (warp == kActWarp) {
         // ================================================================== activations
@@ -335,9 +343,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                 int go = 1;                                            // 0: stop, 1: fetch, 2: publish without fetching
                 if (lane == 0) {
                     // the slot is free when every unit of the segment that used it before is done
-                    if (!smem_wait([&] { return x_pending[slot] == 0 || flags[1]; })) {
-                        atomicCAS(sa.status, 0, FQ_ERR_TIMEOUT); flags[0] = 1; flags[1] = 1;
-                    }
+                    if (!smem_wait([&] { return x_pending[slot] == 0 || flags[1]; }, sa.wait_ns)) give_up(sa.status, flags);
                     // the activations are the previous phase's outputs
                     if (!flags[0] && op.phase > 0 && phase_known < op.phase - 1) {
                         const unsigned long long need = (unsigned long long)sa.phase_total[op.phase - 1];
@@ -345,7 +351,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                         unsigned it = 0;
                         while (ld_acquire_u64(sa.phase_done + (op.phase - 1)) < need) {
                             if ((++it & 63u) == 0u &&
-                                (global_ns() - t0 > kWaitLimitNs || *reinterpret_cast<volatile int*>(sa.status) != 0 ||
+                                (global_ns() - t0 > sa.wait_ns || *reinterpret_cast<volatile int*>(sa.status) != 0 ||
                                  flags[0])) { atomicCAS(sa.status, 0, FQ_ERR_TIMEOUT); flags[0] = 1; break; }
                         }
                     }
@@ -382,10 +388,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                              (uint32_t)have * 2u, bar);
             }
         }
-        // copies that are still in flight land before the CTA may exit (their units wait for them unless the kernel is aborting)
-        if (lane == 0 && flags[1])
-            for (int i = max(0, seg + 1 - kXSlots); i <= seg; i++)
-                if (x_ready[i % kXSlots] == i + 1) mbar_wait(xbars + 8 * (i % kXSlots), (unsigned)(i / kXSlots) & 1u, 1000000ull);
+        if (stop) let_copies_land();
     } else if (warp >= kOutputWarp) {
         // ================================================================== output warps
         // Finishes row pairs.  The unit whose K chunk is (row pair mod chunks) adds up its row pair: its own
@@ -481,8 +484,8 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                 else if ((++idle_it & 127u) == 0u) {
                     const unsigned long long now = global_ns();
                     if (last_progress == 0ull) last_progress = now;
-                    else if (now - last_progress > kWaitLimitNs) {
-                        atomicCAS(sa.status, 0, FQ_ERR_TIMEOUT); flags[0] = 1; flags[1] = 1;
+                    else if (now - last_progress > sa.wait_ns) {
+                        give_up(sa.status, flags);
                         leave = 1;
                     }
                 }
@@ -519,13 +522,10 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
             // a stage's uses are consumed strictly in order: wait for the release of the previous
             // use before trusting the parity of the full barrier
             bool ok = true;
-            if (use > 0) ok = smem_wait([&] { return released[stage] >= use * S::kWarpsPerUnit || flags[1]; });
-            if (ok) ok = mbar_wait(full, use & 1u);
-            if (!ok || flags[1]) {
-                if (lane == 0 && !ok) { atomicCAS(sa.status, 0, FQ_ERR_TIMEOUT); flags[0] = 1; flags[1] = 1; }
-                stop = true;
-                break;
-            }
+            if (use > 0) ok = smem_wait([&] { return released[stage] >= use * S::kWarpsPerUnit || flags[1]; }, sa.wait_ns);
+            if (ok) ok = mbar_wait(full, use & 1u, sa.wait_ns);
+            if (!ok) give_up(sa.status, flags);
+            if (!__all_sync(0xffffffffu, flags[1] == 0)) { stop = true; break; }      // (the lanes leave together, whatever the clocks of their waits said)
             struct { int ch, rp, cnt, seg, blob_read, variant, batch, op_slot, oseq, n_chunks;
                      unsigned long long* partial; } d;
             {
@@ -544,12 +544,8 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
             const int oslot = d.oseq % kOutSlots;
             if (d.oseq >= 0) {
                 const unsigned ogen = (unsigned)(d.oseq / kOutSlots);
-                if (!smem_wait([&] { return out_gen[oslot] == ogen || flags[1]; })) {
-                    if (lane == 0) { atomicCAS(sa.status, 0, FQ_ERR_TIMEOUT); flags[0] = 1; flags[1] = 1; }
-                    stop = true;
-                    break;
-                }
-                if (flags[1]) { stop = true; break; }
+                if (!smem_wait([&] { return out_gen[oslot] == ogen || flags[1]; }, sa.wait_ns)) give_up(sa.status, flags);
+                if (!__all_sync(0xffffffffu, flags[1] == 0)) { stop = true; break; }
                 if (tile == 0 && half == 0 && lane == 0) {
                     const GemvOp& od = *reinterpret_cast<const GemvOp*>(opring + d.op_slot * S::kOpBytes);
                     OutDesc& q = odesc[oslot];
@@ -562,13 +558,11 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
             // dependency phase); a warp that is several publications ahead would read a stale parity, so only a barrier that
             // belongs to this segment counts
             const unsigned xpar = (unsigned)(d.seg / kXSlots) & 1u;
-            if (x_ready[slot] != d.seg + 1 && !flags[1]) mbar_wait(xbars + 8 * slot, xpar);
-            if (!smem_wait([&] { return x_ready[slot] == d.seg + 1 || flags[1]; }) || (!flags[1] && !mbar_wait(xbars + 8 * slot, xpar))) {
-                if (lane == 0) { atomicCAS(sa.status, 0, FQ_ERR_TIMEOUT); flags[0] = 1; }
-            }
+            if (x_ready[slot] != d.seg + 1 && !flags[1]) mbar_wait(xbars + 8 * slot, xpar, sa.wait_ns);
+            if (!smem_wait([&] { return x_ready[slot] == d.seg + 1 || flags[1]; }, sa.wait_ns) || (!flags[1] && !mbar_wait(xbars + 8 * slot, xpar, sa.wait_ns)))
+                give_up(sa.status, flags);
             __threadfence_block();
-            __syncwarp();
-            const bool live = !flags[0];
+            const bool live = __all_sync(0xffffffffu, flags[0] == 0);
 
             float tot[4] = {0.f, 0.f, 0.f, 0.f};
             if constexpr (HIGH)
@@ -593,9 +587,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
             const int lr = tile * kTileRows + g;
             // the two halves of the columns: whoever delivers the second one adds the first (the order does not change the sum)
             if constexpr (S::kHalves) {
-                if (!smem_wait([&] { return delivered[1] >= turn || flags[1]; })) {        // the previous unit's have been taken
-                    if (lane == 0) { atomicCAS(sa.status, 0, FQ_ERR_TIMEOUT); flags[0] = 1; flags[1] = 1; }
-                }
+                if (!smem_wait([&] { return delivered[1] >= turn || flags[1]; }, sa.wait_ns)) give_up(sa.status, flags);        // the previous unit's have been taken
                 if (__any_sync(0xffffffffu, flags[1] != 0)) { stop = true; break; }
                 turn++;
                 float* mine = halves + half * S::kOutFloats;
@@ -640,6 +632,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                 st_relaxed_u64x2(pu + 8 * BP, tag | __float_as_uint(tot[2]), tag | __float_as_uint(tot[3]));
             }
         }
+        if (stop) let_copies_land();
     }
 
     __syncthreads();
@@ -688,6 +681,7 @@ static int launch_batch(Ctx* ctx, const GemvOp& single, StackArgs& sa, int batch
     sa.high_zeros = high_zeros_word(ctx);
     sa.note = ctx->note;
     sa.stored = ctx->stored;
+    sa.wait_ns = ctx->wait_limit_ns;
     if (zeros_are_low(ctx))
         return batch_pad(batch) == 4 ? launch_impl<4, false>(ctx, single, sa, total_units, st) : launch_impl<8, false>(ctx, single, sa, total_units, st);
     return batch_pad(batch) == 4 ? launch_impl<4, true>(ctx, single, sa, total_units, st) : launch_impl<8, true>(ctx, single, sa, total_units, st);

@@ -63,6 +63,12 @@ __device__ __forceinline__ bool smem_wait(Pred pred, unsigned long long limit_ns
         if (global_ns() - t0 > limit_ns) return false;
     }
 }
+// For a warp that leaves because a wait ran out: copies that nobody waits for any more may still be on their way into this CTA's
+// shared memory, which must not go before they are there.  That takes microseconds; the warp stays much longer.
+__device__ __forceinline__ void let_copies_land()
+{
+    for (const unsigned long long t0 = global_ns(); global_ns() - t0 < 200000ull;) __nanosleep(1000);
+}
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar)
 {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
