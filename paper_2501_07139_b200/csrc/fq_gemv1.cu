@@ -673,6 +673,7 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
                 }
                 if (!ok) {
                     if (lane == 0 && !ctl[S::cAbort]) raise_timeout(a, ctl);
+                    let_copies_land();
                     break;
                 }
             }
@@ -687,6 +688,7 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
             if (ok) ok = wait_mbar(bars + 256 + 8 * xslot, ((e.z - 1u) / kXSlots) & 1u, ctl, a.wait_ns);
             if (!__all_sync(0xffffffffu, ok)) {
                 if (lane == 0 && !ctl[S::cAbort]) raise_timeout(a, ctl);
+                let_copies_land();
                 break;
             }
             __threadfence_block();
@@ -804,7 +806,7 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
                 __threadfence_block();
                 ctl[S::cStripBusy + sslot] = 0u;                             // the producer may reuse the slot
             }
-            if (!live) break;
+            if (!live) { let_copies_land(); break; }
             if (finish && phase >= 0) {
                 __threadfence();                                             // y before the phase counter
                 __syncwarp();
