@@ -133,13 +133,14 @@ __device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n) : "memory");
 }
 // Brings the descriptors of the ops a few steps ahead into L1: the table is read once per op by three roles,
-// and a miss would cost each of them a trip to DRAM (the weights keep flushing the L2).
-__device__ __forceinline__ void prefetch_ops(const GemvOp* ops, int oi, int n_ops, int lane)
+// and a miss would cost each of them a trip to DRAM (the weights keep flushing the L2).  For a table in global memory only: ops
+// that came as kernel parameters are not in it.
+__device__ __forceinline__ void prefetch_ops(const GemvOp* ops, int oi, int n_ops, int lane, int* status)
 {
     const int ahead = oi + 2 + (lane >> 1);                        // lanes 0..7: ops oi+2 .. oi+5, two lines each
     if (lane < 8 && ahead < n_ops) {
         const char* p = reinterpret_cast<const char*>(ops + ahead) + (lane & 1) * 64;
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+        if (FQ_IN_BOUNDS(__isGlobal(p), status)) asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
     }
 }
 // The strips of one op for one CTA: rp_first .. rp_last; the first starts at blob c_first, the last ends
@@ -544,7 +545,7 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
                 it_nkb = 0;
                 do { it_oi++; } while (it_oi < a.n_ops && range[it_oi].x == kRangeEmpty);
                 if (it_oi >= a.n_ops) return false;
-                prefetch_ops(ops, it_oi, a.n_ops, lane);
+                if (a.table) prefetch_ops(ops, it_oi, a.n_ops, lane, a.status);
                 const GemvOp& op = ops[it_oi];
                 const StripOrder so(range[it_oi], op.n_kb);
                 it_nkb = op.n_kb; it_kin = op.k_in; it_phase = op.phase; it_split = op.split == 2 ? 2 : 1;
