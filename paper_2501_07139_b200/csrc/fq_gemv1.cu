@@ -57,6 +57,11 @@ constexpr int kMaxKb = 28;                             // blobs per strip, at mo
 constexpr int kQD = 8;                                 // entries per consumer queue
 constexpr int kArrivedMax = 8192;                      // counters of shared strips (the area of the phase counters, not used at the same time)
 constexpr int kMaxPhasesDev = 1024;
+// Bytes that a CTA asks into the L2 before the previous kernel is done: two stages, what the ring is filled with first.  More
+// gets in the way of the copies.  Microseconds without / 64 KB / 256 KB / everything: eight 11008 x 4096 matrices at 4 bits 33.2 / 32.0 /
+// 32.0 / 41.0, 16384 x 14336 at 8 bits 42.1 / 41.0 / 38.6 / 46.4, 4096 x 11008 at 4 bits 9.4 / 8.8 / 9.0 / 9.1, the calls of eight 7B
+// blocks 351 / 341 / 367 / 377.
+constexpr int kAskBytes = 65536;
 constexpr int kMaxOpsDev = 512;                        // ops of one launch (their per-CTA ranges sit in shared memory)
 
 // What the producer tells a consumer warp about one item (one 16-byte store, one 16-byte load).
@@ -359,18 +364,23 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
     }
     __syncthreads();
     if (!a.table && warp < kCW) {
-        // launched while the previous kernel of the stream drains: ask for this CTA's blobs to be brought into the L2 meanwhile
-        for (int oi = 0; oi < a.n_ops; oi++) {
+        // launched while the previous kernel of the stream drains: ask for this CTA's first blobs to be brought into the L2 meanwhile
+        int before = 0;                                                    // bytes of the ops and blobs in front
+        for (int oi = 0; oi < a.n_ops && before < kAskBytes; oi++) {
             const GemvOp& op = ops[oi];
             const StripOrder so(range[oi], op.n_kb);
             for (int si = warp; si < so.n_strips; si += kCW) {
                 const int rp = so.strip(si);
                 int c0, c1;
                 so.chunks(rp, c0, c1);
-                if (c0 + lane < c1 && FQ_IN_BOUNDS(rp < op.n_rp && c1 <= op.n_kb, a.status))
+                const int at = (si > 0 ? si * op.n_kb - so.c_first : 0) + lane;      // number of the blob in this CTA's part of the op
+                if (c0 + lane < c1 && before + (long long)at * op.blob_read < kAskBytes &&
+                    FQ_IN_BOUNDS(rp < op.n_rp && c1 <= op.n_kb, a.status))
                     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
                                  ::"l"(op.store + ((long long)rp * op.n_kb + c0 + lane) * op.blob_stride), "r"(op.blob_read) : "memory");
             }
+            if (so.n_strips > 0)
+                before = (int)min((long long)kAskBytes, before + ((long long)(so.n_strips - 1) * op.n_kb + so.c_last - so.c_first) * op.blob_read);
         }
     }
     // nothing above reads or writes what the previous kernel may still be working on
