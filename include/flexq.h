@@ -258,10 +258,12 @@ int fq_gemv_stack(fq_ctx* ctx, int n_ops, const int* layers_host,
  * w^ = (q - z) * s exactly in fp32, rounded once to bf16; tensor cores (tcgen05, fp32 accumulation in
  * TMEM); Y is rounded once to bf16.  Runs whichever of two ways is estimated to be the faster for the
  * shape: one kernel that converts the weights on their way into the tensor cores, or the two passes of
- * fq_gemm_two_pass, whose workspace (bf16 of the largest layer) the first such call allocates; where
- * that is not possible (no memory, the stream is being captured) the first way serves every shape.
- * Thread blocks may share an output tile, which is then the fp32 sum of their partial sums in K order
- * (the last bit may differ from the other way's), through slots that belong to the context (29 MB).
+ * fq_gemm_two_pass.  In the first way thread blocks may share an output tile, which is then the fp32 sum of
+ * their partial sums in K order (the last bit may differ from the other way's), through slots that belong to
+ * the context (24 MB).  The second way converts a layer larger than that in parts, through the same memory,
+ * on the first such call; the second such call allocates room for the bf16 copy of the largest layer, which later
+ * calls use and fq_destroy frees.  Where it cannot be had (no memory, the stream is being captured) the
+ * conversion stays in parts.  The results are the same bits.
  * One fq_gemm at a time per context. */
 int fq_gemm(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int ldx,
             uint16_t* Y_dev, int ldy, void* stream);

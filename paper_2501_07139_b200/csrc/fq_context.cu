@@ -957,6 +957,18 @@ static bool dequant_workspace(fq_ctx* ctx, cudaStream_t st, size_t need, bool re
     return true;
 }
 
+// How many outputs of a layer to convert at a time when their bf16 copies may take `bytes`: all, or equal parts in whole tiles
+// where that costs no further part.  0: not even the rows of one blob fit.
+static int slice_rows(int n_out, int k_in, size_t bytes)
+{
+    constexpr int kStrip = kBlobTiles * kTileRows, kTile = 256;
+    const long long fit = (long long)(bytes / ((size_t)k_in * 2)) / kStrip * kStrip;
+    if (fit >= n_out) return n_out;
+    if (fit < kStrip) return 0;
+    const long long parts = (n_out + fit - 1) / fit, even = round_up((n_out + parts - 1) / parts, kTile);
+    return (int)(even <= fit ? even : fit);
+}
+
 static int gemm_common(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int ldx, uint16_t* Y_dev, int ldy, void* stream,
                        bool fused)
 {
@@ -976,17 +988,34 @@ static int gemm_common(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int
     const cudaStream_t st = (cudaStream_t)stream;
     const FieldList fl = active_fields(L, bits);
     // Two ways to the same product, whichever the shape makes the faster one: converting the weights inside the GEMM, once for
-    // every tile of up to 192 tokens, or once for all tokens in a pass of their own.  Both estimates are fits to measured times
+    // every tile of up to 160 tokens, or once for all tokens in a pass of their own.  Both estimates are fits to measured times
     // (within about 15 %); the second way needs room for a bf16 copy of the layer.
     const bool two_pass = !fused || gemm_two_pass_us(ctx, M, L.n_out, L.k_in) < gemm_split_us(ctx, M, L.n_out, L.k_in);
-    if (two_pass && dequant_workspace(ctx, st, (size_t)L.n_out * L.k_in * 2, !fused))
-        return launch_gemm(ctx, v->store, stride, fl, zero_adjust, L.n_out, L.k_in, X_dev, M, ldx, Y_dev, ldy, ctx->gemm_ws, st);
-    if (!fused) return FQ_ERR_CUDA;
+    float* slots = ctx->fused_ws ? reinterpret_cast<float*>(ctx->fused_ws + gemm_split_flag_bytes(ctx->sm_count)) : nullptr;
+    if (two_pass) {
+        const size_t need = (size_t)L.n_out * L.k_in * 2;
+        const int fit = slots ? slice_rows(L.n_out, L.k_in, gemm_split_part_bytes(ctx->sm_count)) : 0;
+        if (fused && fit > 0 && need > ctx->gemm_ws_bytes) {
+            // The copy goes through the slots of the other way, some outputs at a time: the same sums (an output does not know
+            // which others are computed beside it) and up to 15 % slower.  Allocating takes 0.35 ms, as long as a call at 8192 tokens
+            // and 4096 x 4096, so the first call does without and the second asks for the room once its work is on its way.
+            for (int n0 = 0; n0 < L.n_out; n0 += fit) {
+                const int rc = launch_gemm(ctx, static_cast<const uint8_t*>(v->store) + (long long)(n0 / (kBlobTiles * kTileRows)) * k_blobs(L.k_in) * stride,
+                                           stride, fl, zero_adjust, L.n_out - n0 < fit ? L.n_out - n0 : fit, L.k_in, X_dev, M, ldx,
+                                           Y_dev + n0, ldy, slots, st);
+                if (rc != FQ_OK) return rc;
+            }
+            if (fit < L.n_out && ++ctx->gemm_sliced >= 2) dequant_workspace(ctx, st, need, false);
+            return FQ_OK;
+        }
+        if (dequant_workspace(ctx, st, need, !fused))
+            return launch_gemm(ctx, v->store, stride, fl, zero_adjust, L.n_out, L.k_in, X_dev, M, ldx, Y_dev, ldy, ctx->gemm_ws, st);
+        if (!fused) return FQ_ERR_CUDA;
+    }
     // counters and slots for the sums of tiles that several CTAs share; without them the tiles stay whole
     unsigned* arrived = reinterpret_cast<unsigned*>(ctx->fused_ws);
-    float* parts = ctx->fused_ws ? reinterpret_cast<float*>(ctx->fused_ws + gemm_split_flag_bytes(ctx->sm_count)) : nullptr;
     const int read = L.fmt == FQ_FMT_PLANES ? blob_bytes(plane_read_bits(bits)) : stride;
-    return launch_gemm_split(ctx, v->store, stride, read, fl, zero_adjust, L.n_out, L.k_in, X_dev, M, ldx, Y_dev, ldy, parts, arrived, st);
+    return launch_gemm_split(ctx, v->store, stride, read, fl, zero_adjust, L.n_out, L.k_in, X_dev, M, ldx, Y_dev, ldy, slots, arrived, st);
 }
 
 int fq_gemm(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int ldx, uint16_t* Y_dev, int ldy, void* stream)

@@ -81,6 +81,7 @@ struct Ctx {
     bool gemm_ws_captured = false;       // a captured graph holds the address of gemm_ws
     size_t gemm_ws_refused = 0;          // size that could not be had, under this configuration
     uint64_t gemm_ws_refused_at = ~0ull;
+    int gemm_sliced = 0;                 // calls that did without a larger gemm_ws
     char* fused_ws = nullptr;            // prefill: counters, then two fp32 tile slots per SM (part of the allocation of status_dev)
     std::vector<void*> owned;    // device buffers freed by fq_destroy: those of fq_load, workspaces that graphs may hold
     uint64_t config_epoch = 0;
