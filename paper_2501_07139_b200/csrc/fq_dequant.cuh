@@ -124,15 +124,26 @@ __device__ __forceinline__ void merge_group_codes(const uint4 (&raw)[group_loads
 
 // Four codes of one row (one A register) -> four bf16 weights w^ = (q - z) * s, each rounded once.
 //   Codes up to 255: a byte q under the exponent byte 0x64 is the fp16 number 1024 + q; subtracting zz = 1024 + z
-//   in fp16 is exact (integers below 2048), the product with the fp16 scale is exact in fp32 (9 x 11 bits).
-__device__ __forceinline__ uint2 codes_to_bf16(uint32_t q4, __half2 zz, float s)
+//   in fp16 is exact for the low ten bits of z (integers below 2048), the product with the fp16 scale is exact in fp32 (11 x 11
+//   bits), and c = -(upper bits of z) * s (exact: 6 x 11 bits) is added in the same instruction.
+struct WideZero {
+    __half2 zz;
+    float c;
+    //   meta : the stored scale/zero word        adjust : subtracted from z (the mid-point fill of a nested child)
+    __device__ __forceinline__ WideZero(uint32_t meta, int adjust, float s)
+    {
+        zz = __half2half2(__int2half_rn((int)((meta >> 16) & 1023u) + 1024 - adjust));
+        c = -(float)((meta >> 16) & ~1023u) * s;
+    }
+};
+__device__ __forceinline__ uint2 codes_to_bf16(uint32_t q4, const WideZero& z, float s)
 {
     const uint32_t p02 = (q4 & 0x00ff00ffu) | 0x64006400u;          // columns 0 and 2
     const uint32_t p13 = __byte_perm(q4, 0x64646464u, 0x4341);      // columns 1 and 3
-    const float2 d02 = __half22float2(__hsub2(*reinterpret_cast<const __half2*>(&p02), zz));
-    const float2 d13 = __half22float2(__hsub2(*reinterpret_cast<const __half2*>(&p13), zz));
-    const __nv_bfloat162 lo = __floats2bfloat162_rn(d02.x * s, d13.x * s);
-    const __nv_bfloat162 hi = __floats2bfloat162_rn(d02.y * s, d13.y * s);
+    const float2 d02 = __half22float2(__hsub2(*reinterpret_cast<const __half2*>(&p02), z.zz));
+    const float2 d13 = __half22float2(__hsub2(*reinterpret_cast<const __half2*>(&p13), z.zz));
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(fmaf(d02.x, s, z.c), fmaf(d13.x, s, z.c));
+    const __nv_bfloat162 hi = __floats2bfloat162_rn(fmaf(d02.y, s, z.c), fmaf(d13.y, s, z.c));
     uint2 o;
     o.x = *reinterpret_cast<const uint32_t*>(&lo);
     o.y = *reinterpret_cast<const uint32_t*>(&hi);

@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(256) dequant_kernel(const DequantArgs a)
                 const long long n = (long long)rp * 32 + tl * kTileRows + g + 8 * hr;
                 if (n >= a.n_out) continue;
                 const float s = __half2float(__ushort_as_half((unsigned short)(mm[hr] & 0xffffu)));
-                const __half2 zz = __half2half2(__int2half_rn(1024 + (int)(mm[hr] >> 16) - a.zero_adjust));
+                const WideZero zz(mm[hr], a.zero_adjust, s);
                 const float cc = -(float)(128 + (int)(mm[hr] >> 16)) * s;
                 __nv_bfloat16* row = a.out + n * a.k_in + ks * 64 + 4 * c;
 #pragma unroll

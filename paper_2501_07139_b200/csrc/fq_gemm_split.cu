@@ -462,15 +462,14 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_x, const SplitArgs a)
                 for (int tl = 0; tl < kBlobTiles; tl++) {
                     align_group_words<VARIANT>(raw[tl], grp);
                     const uint32_t mm[2] = {meta[tl].x, meta[tl].y};
-                    __half2 zz[2];
                     float sc[2], cc[2];
 #pragma unroll
                     for (int hr = 0; hr < 2; hr++) {
                         sc[hr] = have ? __half2float(__ushort_as_half((unsigned short)(mm[hr] & 0xffffu))) : 0.f;   // rows past N: zeros
-                        zz[hr] = __half2half2(__int2half_rn(1024 + (int)(mm[hr] >> 16) - a.zero_adjust));
                         cc[hr] = -(float)((kHalved ? 256 - a.zero_adjust : 128) + (int)(mm[hr] >> 16)) * sc[hr];
                         if (kHalved) sc[hr] *= 2.f;
                     }
+                    const WideZero zz[2] = {{mm[0], a.zero_adjust, sc[0]}, {mm[1], a.zero_adjust, sc[1]}};
                     unrolled<0, 2>([&](auto H) {                               // 64 columns at a time
                         constexpr int h = decltype(H)::value;
                         uint32_t w[16];
