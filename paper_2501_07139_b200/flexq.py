@@ -122,9 +122,14 @@ def fq_meta_bytes(n_out: int, k_in: int, group: int = 128) -> int:
     return int(lib().fq_meta_bytes(n_out, k_in, group))
 
 
+# torch's own short way to the stream's handle, where there is one: without building a Stream object, a call is a few microseconds in all
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream() -> int:
-    if torch.cuda.is_initialized():                      # (without building a Stream object: a call is a few microseconds in all)
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if _raw_stream and _device and torch.cuda.is_initialized():
+        return _raw_stream(_device())
     return torch.cuda.current_stream().cuda_stream
 
 
