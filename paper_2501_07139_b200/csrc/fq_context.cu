@@ -120,12 +120,7 @@ int fill_op(const Ctx* ctx, int layer, const uint16_t* x, uint16_t* y, int batch
     if (!v) return FQ_ERR_NO_VARIANT;
     const FieldList fl = active_fields(L, bits);
     std::memset(&op, 0, sizeof op);
-    for (int i = 0; i < fl.n; i++) {
-        op.field_width[i] = fl.width[i];
-        op.field_shift[i] = fl.shift[i];
-    }
     op.n_fields = fl.n;
-    op.bits = bits;
     op.variant = variant_index(L.fmt == FQ_FMT_PLANES, bits);
     op.store = static_cast<const uint8_t*>(v->store);
     op.blob_stride = blob_bytes(L.fmt == FQ_FMT_PLANES ? 8 : bits);
@@ -134,15 +129,12 @@ int fill_op(const Ctx* ctx, int layer, const uint16_t* x, uint16_t* y, int batch
     op.y = y;
     op.n_out = L.n_out;
     op.k_in = L.k_in;
-    op.n_ss = supersteps(L.k_in);
     op.n_kb = k_blobs(L.k_in);
     op.n_rp = row_pairs(L.n_out);
     op.chunk_blobs = one ? gemv1_chunk_blobs(op.blob_read)
                                 : gemv_chunk_blobs(L.fmt == FQ_FMT_PLANES ? plane_read_bits(bits) : bits);
     op.n_chunks = (op.n_kb + op.chunk_blobs - 1) / op.chunk_blobs;
     op.batch = batch;
-    // nested child: codes are the parent's top bits; the dropped bits are filled with their mid-point
-    op.zero_adjust = (L.fmt == FQ_FMT_PLANES && bits < 8) ? (1 << (7 - bits)) : 0;
     // what is dealt to the CTAs: batch 1 the blobs of every strip, batch 2..8 the K chunks of every row pair
     op.n_units = (one ? op.n_kb : op.n_chunks) * op.n_rp;
     if ((long long)op.n_units * 1024 >= (1ll << 31)) return FQ_ERR_SHAPE;              // 32-bit unit arithmetic on the device
@@ -177,7 +169,7 @@ size_t layer_partial_bytes(int n_out, int k_in)
 
 namespace fq {
 
-// Status word, and behind it the prefill's counters and slots (29 MB): an allocation costs about 0.4 ms whatever its size, and
+// Status word, and behind it the prefill's counters and slots (24 MB): an allocation costs about 0.4 ms whatever its size, and
 // the first prompt of a context should not pay for one.  Without that much memory prefill keeps its tiles whole.
 static bool allocate_status(Ctx* ctx)
 {
@@ -983,6 +975,7 @@ static int gemm_common(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int
     if (!v) return FQ_ERR_NO_VARIANT;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return FQ_ERR_CUDA;
+    // nested child: codes are the parent's top bits; the dropped bits are filled with their mid-point
     const int zero_adjust = (L.fmt == FQ_FMT_PLANES && bits < 8) ? (1 << (7 - bits)) : 0;
     const int stride = blob_bytes(L.fmt == FQ_FMT_PLANES ? 8 : bits);
     const cudaStream_t st = (cudaStream_t)stream;

@@ -211,7 +211,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
 
     if (warp == kProducerWarp) {
         // ================================================================== producer (one warp)
-        // Lane 0 owns the barriers; lanes 0 .. 2*n_fields+1 each issue one bulk copy per unit.
+        // Lane 0 owns the barriers and issues a unit's copy; of a nested child a lane per blob issues that blob's.
         GemvOp* opbuf = reinterpret_cast<GemvOp*>(smem + S::oOpBuf);
         uint8_t* opring = smem + S::oOpRing;
         OpFetch fetch;

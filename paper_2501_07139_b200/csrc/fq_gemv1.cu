@@ -1,8 +1,8 @@
 // Decode path, batch 1: fused dequantize-GEMV over tiled field arrays, one persistent CTA per SM.
 //
 // Work split.  An op (one matrix) is cut into STRIPS of 32 output rows x the whole K, a strip into blobs of
-// 512 columns.  Blobs are numbered strip-major and dealt to the CTAs in equal contiguous blocks (cta_work in
-// fq_internal.cuh), so every CTA streams the same number of bytes and almost every strip is computed by ONE
+// 512 columns.  Blobs are numbered strip-major and dealt to the CTAs in contiguous blocks of equal cost (by the host
+// for a table of ops, by inline_work for ops that came as parameters), so almost every strip is computed by ONE
 // CTA from end to end: its K reduction stays in shared memory and the CTA writes y itself.  Only a strip
 // that a block boundary cuts is shared by two (rarely three) CTAs: the CTA that owns the strip's FIRST blob
 // finishes it, the others publish the sums of their blobs as tagged 64-bit words (fp32 value, launch tag)
@@ -11,8 +11,9 @@
 // its blobs of a strip in "units" of up to six (what one ring stage holds).  y[row] is always the sum of the per-blob sums in
 // blob order, whoever computed them, so results do not depend on how the op was dealt.
 //
-// (In a launch without dependency phases a shared strip is added up by whoever publishes its last blob sum instead, so that no
-// CTA waits for another; such launches need not be cooperative and overlap the previous kernel of the stream.)
+// (Ops that came as kernel parameters, up to eight without dependencies: a shared strip is added up by whoever publishes its last
+// blob sum instead, so that no CTA waits for another; such launches need not be cooperative and overlap the previous kernel of the
+// stream.  Longer lists, fq_gemv_static and ops of more than kArrivedMax strips wait as above.)
 //
 // Roles of a CTA:
 //   producer warp   : walks the op list, streams units into a ring of shared-memory stages with bulk
@@ -149,7 +150,7 @@ __device__ __forceinline__ void prefetch_ops(const GemvOp* ops, int oi, int n_op
     }
 }
 // The strips of one op for one CTA: rp_first .. rp_last; the first starts at blob c_first, the last ends
-// before blob c_last (see cta_work).  Packed into two words per (CTA, op) by the host for a stack call.
+// before blob c_last (see CtaWork).  Packed into two words per (CTA, op) by the host for a stack call.
 constexpr uint32_t kRangeEmpty = 0xffffffffu;
 FQ_HD uint2 pack_range(const CtaWork& w, int n_kb)
 {

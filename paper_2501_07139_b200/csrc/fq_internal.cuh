@@ -40,14 +40,10 @@ struct GemvOp {
     uint16_t* y;                 // fp16 [batch][n_out]
     int blob_stride;             // bytes from one blob to the next (size of the stored variant's blobs)
     int n_fields;
-    uint8_t field_width[kMaxFields];
-    uint8_t field_shift[kMaxFields];
-    int bits;                    // code bytes per tile superstep = 512 * bits
     int n_out, k_in;
-    int n_ss, n_kb;              // supersteps, k blobs
+    int n_kb;                    // k blobs
     int n_rp;                    // row pairs = units per K chunk
     int chunk_blobs;             // k blobs per K chunk (the last chunk may be shorter)
-    int zero_adjust;             // subtracted from every zero point (mid-point fill of a nested child)
     int phase;                   // -1: no ordering
     int n_units;                 // n_chunks * n_rp
     int rot;                     // rotation of the CTA blocks for this op (evens out remainders); inline ops: its first strip counter
@@ -167,7 +163,7 @@ int launch_gemv_stack(Ctx* ctx, const StackHeader& hdr, const char* table_dev, i
 // Units of an op (n_units units, block rotation rot) that CTA `cta` of `grid` processes: [lo, hi).
 void gemv_cta_range(int n_units, int rot, int cta, int grid, int& lo, int& hi);
 
-// ---- how a decode op is dealt to the CTAs of the persistent grid (shared by host and device code)
+// ---- how a decode op is dealt to the CTAs of the persistent grid
 // The pieces of an op (batch 1: the blobs of its 32-row strips; batch 2..8: K chunks of row pairs) are numbered
 // strip-major, u = rp * pieces_per_strip + i, and dealt in contiguous blocks; the block boundaries rotate from
 // op to op so that the remainders even out.
@@ -194,14 +190,6 @@ struct CtaWork {
         return rp_last - rp_first + 1 - (lo - rp_first * n_chunks > 0 ? 1 : 0);
     }
 };
-FQ_HD CtaWork cta_work(int n_units, int n_chunks, int rot, int cta, int grid)
-{
-    CtaWork w;
-    cta_range(n_units, rot, cta, grid, w.lo, w.hi);
-    w.rp_first = w.lo / n_chunks;
-    w.rp_last = w.hi > w.lo ? (w.hi - 1) / n_chunks : w.rp_first;
-    return w;
-}
 
 int launch_gemm(Ctx* ctx, const void* store, int blob_stride, const FieldList& fl, int zero_adjust, int n_out, int k_in,
                 const uint16_t* X, int M, int ldx, uint16_t* Y, int ldy, void* w_scratch, cudaStream_t st);

@@ -134,18 +134,4 @@ FQ_HD FieldPos field_pos(int f, int r, int kk)
     return q;
 }
 
-// Inverse: field slot q (0 .. 32/f - 1; q = byte * P + t) of word `word` of lane `lane` of chunk
-// `chunk` belongs to which (row, column) of the tile, and at which bit it sits.
-FQ_HD void field_owner(int f, int chunk, int lane, int word, int q, int& r, int& kk, int& bit)
-{
-    const int P = 8 / f;
-    const int byte = q / P, t = q % P;
-    const int g = lane >> 2, c = lane & 3;
-    const int half = word >> 1, hi_row = word & 1;
-    const int j = chunk * P + t;
-    r = g + 8 * hi_row;
-    kk = j * 32 + half * 16 + c * 4 + byte;
-    bit = byte * 8 + t * f;
-}
-
 }  // namespace fq

@@ -71,7 +71,7 @@ static __device__ __forceinline__ void umma_commit(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = 128, N = 256.
+// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, of m x n outputs.
 static __device__ __forceinline__ uint32_t umma_idesc_bf16(int m, int n)
 {
     uint32_t d = 0;
