@@ -183,12 +183,13 @@ def prefill_pass(P, device, blocks, steps, warmup, tokens=PREFILL_TOKENS):
     ms = timed(one_pass)
     ms_two = timed(one_pass_two)
     status = fq.fq_status()
+    launches = sum(2 if fq.fq_gemm_plan(i, m)["two_pass"] else 1 for i in range(L))
     fq.fq_destroy()
     if status != 0:
         raise RuntimeError(f"device status {status} after the prefill pass")
     flop = sum(2.0 * m * sh.n_out * sh.k_in for sh in shapes)
     return {"ms_per_pass": ms, "tflops": flop / (ms * 1e-3) / 1e12, "flop_per_pass": flop, "tokens": m,
-            "matrices": L, "average_bits": S.average_bits(bits, shapes), "gpu_launches_per_pass": 2 * L,
+            "matrices": L, "average_bits": S.average_bits(bits, shapes), "gpu_launches_per_pass": launches,
             "two_pass": {"ms_per_pass": ms_two, "tflops": flop / (ms_two * 1e-3) / 1e12, "gpu_launches_per_pass": 2 * L}}
 
 

@@ -87,7 +87,8 @@ int fq_quantize_layer(const float* w_dev, int n_out, int k_in, int bits, int gro
  *           ceil(b / 2) fields of every blob (a child of odd width ignores the low bit of its last
  *           field) and every b in [2,8] becomes selectable.
  *   codes_dev   uint8 [n_out][k_in], one code per byte; read, not retained.
- *   scales_dev, zeros_dev   fp16 [n_out][k_in/128]; read, not retained.
+ *   scales_dev, zeros_dev   fp16 [n_out][k_in/128]; read, not retained.  Zero points are integers of any size
+ *           that fp16 holds; a context that holds one above 1023 decodes batch 2..8 a little slower.
  *   store_out_dev fq_store_bytes() bytes, 256-byte aligned; written and RETAINED.
  * The first variant packed for a layer becomes its active one. */
 int fq_pack_layer(fq_ctx* ctx, int layer, int n_out, int k_in, int bits, int group, int fmt,
@@ -204,7 +205,7 @@ int fq_sqdiff(const uint16_t* a_bf16_dev, const uint16_t* b_bf16_dev, size_t n, 
  *   Layers with k_in <= 14336 run in the batch-1 kernel (the activations of one 32-row strip stay in shared
  *   memory); wider layers run in the batch kernel, slower per byte but without a limit on k_in.
  * Enqueues one kernel on `stream`; neither allocates (the scratch was reserved by fq_pack_layer) nor
- * synchronises.  An activation group that holds an infinity or a NaN makes every output NaN. */
+ * synchronises.  An activation that is an infinity or a NaN makes every output NaN. */
 int fq_gemv(fq_ctx* ctx, int layer, const uint16_t* x_dev, uint16_t* y_dev, void* stream);
 
 /* Same result as fq_gemv, for callers that must not allocate device memory.  (The paper has no
@@ -232,7 +233,8 @@ int fq_gemv(fq_ctx* ctx, int layer, const uint16_t* x_dev, uint16_t* y_dev, void
 int fq_gemv_static(fq_ctx* ctx, int layer, const uint16_t* x_dev, uint16_t* y_dev, void* stream);
 
 /* Decode at batch 1..8:  Y[b][n] = sum_k X[b][k] * w^[n][k].
- *   x_dev fp16 [batch][k_in], y_dev fp16 [batch][n_out], densely packed rows. */
+ *   x_dev fp16 [batch][k_in], y_dev fp16 [batch][n_out], densely packed rows.
+ * An activation that is an infinity or a NaN makes every output of its batch entry NaN. */
 int fq_gemv_batched(fq_ctx* ctx, int layer, const uint16_t* x_dev, int batch, uint16_t* y_dev, void* stream);
 
 /* Decode through a whole stack of layers in ONE persistent launch; op i computes
@@ -246,7 +248,10 @@ int fq_gemv_batched(fq_ctx* ctx, int layer, const uint16_t* x_dev, int batch, ui
  * builds a table (ops, and which strips every thread block computes) and uploads it from a
  * pinned buffer; a call with the same arguments under the same configuration reuses the uploaded
  * table and only launches the kernel.  The workspace was sized by fq_pack_layer for lists that use
- * every layer at most once; a list that repeats layers may grow it (device allocation + sync). */
+ * every layer at most once; a list that repeats layers may grow it (device allocation + sync).
+ * Stream capture: fq_gemv and fq_gemv_batched at batch 1 (k_in <= 14336), lists that travel as kernel parameters, and
+ * fq_gemm can be replayed.  The other decode launches tell their own sums by a launch number, which a replay
+ * repeats: capture them only for a graph that is launched once. */
 int fq_gemv_stack(fq_ctx* ctx, int n_ops, const int* layers_host,
                   const uint16_t* const* x_dev_host, uint16_t* const* y_dev_host,
                   const int* phases_host, int batch, void* stream);
@@ -275,6 +280,16 @@ int fq_gemm_two_pass(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int l
                      uint16_t* Y_dev, int ldy, void* stream);
 
 /* Test / reporting support ------------------------------------------------------------ */
+
+/* How fq_gemm runs M tokens through `layer`.  Host only. */
+typedef struct fq_gemm_plan_report {
+    int two_pass;               /* 1: as fq_gemm_two_pass, 0: one kernel, described by the rest      */
+    int shared;                 /* output tiles are shared between thread blocks                     */
+    int blocks;                 /* thread blocks; if shared, each takes an equal run of the (tile, 128 columns of K) pairs */
+    int tile_tokens;            /* a tile is this many tokens x 128 outputs                          */
+    long long tiles;
+} fq_gemm_plan_report;
+int fq_gemm_plan(const fq_ctx* ctx, int layer, int M, fq_gemm_plan_report* report_host);
 
 /* Writes the canonical form of what is stored for `layer` at width `bits`:
  *   PACKED: uint32 [n_out][k_in*bits/32], per row a little-endian bitstream, code k in bits

@@ -961,6 +961,14 @@ static int slice_rows(int n_out, int k_in, size_t bytes)
     return (int)(even <= fit ? even : fit);
 }
 
+// Two ways to the same product, whichever the shape makes the faster one: converting the weights inside the GEMM, once for every
+// tile of up to 160 tokens, or once for all tokens in a pass of their own.  Both estimates are fits to measured times (within
+// about 15 %); the second way needs room for a bf16 copy of the layer.
+static bool two_pass_is_faster(const fq_ctx* ctx, const Layer& L, int M)
+{
+    return gemm_two_pass_us(ctx, M, L.n_out, L.k_in) < gemm_split_us(ctx, M, L.n_out, L.k_in);
+}
+
 static int gemm_common(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int ldx, uint16_t* Y_dev, int ldy, void* stream,
                        bool fused)
 {
@@ -980,10 +988,7 @@ static int gemm_common(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int
     const int stride = blob_bytes(L.fmt == FQ_FMT_PLANES ? 8 : bits);
     const cudaStream_t st = (cudaStream_t)stream;
     const FieldList fl = active_fields(L, bits);
-    // Two ways to the same product, whichever the shape makes the faster one: converting the weights inside the GEMM, once for
-    // every tile of up to 160 tokens, or once for all tokens in a pass of their own.  Both estimates are fits to measured times
-    // (within about 15 %); the second way needs room for a bf16 copy of the layer.
-    const bool two_pass = !fused || gemm_two_pass_us(ctx, M, L.n_out, L.k_in) < gemm_split_us(ctx, M, L.n_out, L.k_in);
+    const bool two_pass = !fused || two_pass_is_faster(ctx, L, M);
     float* slots = ctx->fused_ws ? reinterpret_cast<float*>(ctx->fused_ws + gemm_split_flag_bytes(ctx->sm_count)) : nullptr;
     if (two_pass) {
         const size_t need = (size_t)L.n_out * L.k_in * 2;
@@ -1009,6 +1014,18 @@ static int gemm_common(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int
     unsigned* arrived = reinterpret_cast<unsigned*>(ctx->fused_ws);
     const int read = L.fmt == FQ_FMT_PLANES ? blob_bytes(plane_read_bits(bits)) : stride;
     return launch_gemm_split(ctx, v->store, stride, read, fl, zero_adjust, L.n_out, L.k_in, X_dev, M, ldx, Y_dev, ldy, slots, arrived, st);
+}
+
+int fq_gemm_plan(const fq_ctx* ctx, int layer, int M, fq_gemm_plan_report* report_host)
+{
+    if (!ctx || !report_host || layer < 0 || layer >= (int)ctx->layers.size()) return FQ_ERR_ARG;
+    const Layer& L = ctx->layers[layer];
+    if (!L.registered) return FQ_ERR_NOT_PACKED;
+    if (M < 1 || M > (1 << 20)) return FQ_ERR_SHAPE;
+    *report_host = fq_gemm_plan_report{};
+    report_host->two_pass = two_pass_is_faster(ctx, L, M);
+    if (!report_host->two_pass) gemm_split_plan(ctx, M, L.n_out, L.k_in, report_host);
+    return FQ_OK;
 }
 
 int fq_gemm(fq_ctx* ctx, int layer, const uint16_t* X_dev, int M, int ldx, uint16_t* Y_dev, int ldy, void* stream)

@@ -572,6 +572,15 @@ double gemm_split_us(const Ctx* ctx, int M, int n_out, int k_in)
     return Plan(ctx->sm_count, M, n_out, k_in).us * (1.0 + 0.3 * (M < 2048 ? M : 2048) / 2048.0);
 }
 
+void gemm_split_plan(const Ctx* ctx, int M, int n_out, int k_in, fq_gemm_plan_report* out)
+{
+    const Plan plan(ctx->sm_count, M, n_out, k_in);
+    out->shared = ctx->fused_ws && plan.share;
+    out->tile_tokens = split_tile_n(M);
+    out->tiles = plan.tiles;
+    out->blocks = (int)(out->shared ? plan.runs : (plan.tiles < ctx->sm_count ? plan.tiles : ctx->sm_count));
+}
+
 size_t gemm_split_flag_bytes(int sm_count) { return (size_t)round_up((int64_t)sm_count * sizeof(unsigned), 256); }
 size_t gemm_split_part_bytes(int sm_count) { return (size_t)sm_count * 2 * kRows * kTokens * sizeof(float); }
 

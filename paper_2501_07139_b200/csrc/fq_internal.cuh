@@ -143,6 +143,7 @@ int launch_gemm_split(Ctx* ctx, const void* store, int blob_stride, int blob_rea
                       cudaStream_t st);
 size_t gemm_split_flag_bytes(int sm_count);
 size_t gemm_split_part_bytes(int sm_count);
+void gemm_split_plan(const Ctx* ctx, int M, int n_out, int k_in, fq_gemm_plan_report* out);
 double gemm_split_us(const Ctx* ctx, int M, int n_out, int k_in);       // estimates of the time of a call
 double gemm_two_pass_us(const Ctx* ctx, int M, int n_out, int k_in);
 struct CtaWork;

@@ -27,7 +27,7 @@ EXPORTS = [
     "fq_create", "fq_destroy", "fq_store_bytes", "fq_quantize_layer", "fq_pack_layer",
     "fq_set_config", "fq_gemv", "fq_gemv_batched", "fq_gemv_stack", "fq_gemm", "fq_export_layer",
     "fq_export_meta", "fq_storage_bytes", "fq_active_bits", "fq_status", "fq_strerror", "fq_gemv_static", "fq_transition", "fq_save", "fq_load", "fq_search_chain", "fq_prune_chain", "fq_sqdiff",
-    "fq_set_wait_limit_ns", "fq_code_bytes", "fq_meta_bytes", "fq_stream_read", "fq_gemm_two_pass",
+    "fq_set_wait_limit_ns", "fq_code_bytes", "fq_meta_bytes", "fq_stream_read", "fq_gemm_two_pass", "fq_gemm_plan",
     "fq_host_variant", "fq_transition_swap",
 ]
 
@@ -41,6 +41,10 @@ class SwapReport(C.Structure):
     _fields_ = [("bytes_loaded", C.c_uint64), ("bytes_freed", C.c_uint64), ("peak_extra_bytes", C.c_uint64),
                 ("resident_bytes", C.c_uint64), ("footprint_from", C.c_uint64), ("footprint_to", C.c_uint64),
                 ("layers_changed", C.c_int), ("one_way", C.c_int)]
+
+
+class GemmPlan(C.Structure):
+    _fields_ = [("two_pass", C.c_int), ("shared", C.c_int), ("blocks", C.c_int), ("tile_tokens", C.c_int), ("tiles", C.c_longlong)]
 
 
 class FlexQError(RuntimeError):
@@ -84,6 +88,7 @@ def lib():
     L.fq_gemv_stack.argtypes = [vp, i, vp, vp, vp, vp, i, vp]
     L.fq_gemm.argtypes = [vp, i, vp, i, i, vp, i, vp]
     L.fq_gemm_two_pass.argtypes = [vp, i, vp, i, i, vp, i, vp]
+    L.fq_gemm_plan.argtypes = [vp, i, i, C.POINTER(GemmPlan)]
     L.fq_export_layer.argtypes = [vp, i, i, vp, vp]
     L.fq_export_meta.argtypes = [vp, i, i, vp, vp, vp]
     L.fq_storage_bytes.argtypes = [vp]
@@ -347,6 +352,12 @@ class FlexQ:
         return Y
 
     # -- export (tests / reporting) ----------------------------------------------------------
+    def fq_gemm_plan(self, layer: int, tokens: int) -> dict:
+        """How `fq_gemm` runs that many tokens through a layer."""
+        r = GemmPlan()
+        _check(lib().fq_gemm_plan(self._h, layer, tokens, C.byref(r)), "fq_gemm_plan")
+        return {f: getattr(r, f) for f, _ in GemmPlan._fields_}
+
     def fq_export_layer(self, layer: int, bits: int, n_out: int, k_in: int) -> torch.Tensor:
         out = torch.empty(n_out * k_in * bits // 32, dtype=torch.int32, device=self.device)
         _check(lib().fq_export_layer(self._h, layer, bits, out.data_ptr(), _stream()), "fq_export_layer")

@@ -1,5 +1,5 @@
-"""GPU parity of the prefill path against the fp64 CPU oracle: the fused kernel behind fq_gemm (blobs
-dequantised inside the tcgen05 GEMM) and its two-pass comparison point fq_gemm_two_pass."""
+"""GPU parity of the prefill path against the fp64 CPU oracle: fq_gemm ("fused" below, although it takes the two-pass way for
+long prompts) and fq_gemm_two_pass."""
 import numpy as np
 import pytest
 import torch
@@ -36,7 +36,7 @@ def _ref(codes, s, z, bits, fmt, x):
 @pytest.mark.parametrize("fmt_bits", [(0, 2), (0, 3), (0, 4), (0, 5), (0, 6), (0, 7), (0, 8), (1, 3), (1, 6), (1, 8)])
 def test_gemm_small_every_element(P, which, fmt_bits):
     fmt, bits = fmt_bits
-    n, k, m = 300, 384, 200                      # ragged against the 128 x 256 x 64 tiles
+    n, k, m = 300, 384, 200                      # ragged against every tile
     stored = 8 if fmt == 1 else bits
     codes, s, z = make_layer(110, bits, n, k, stored)
     fq = P.FlexQ(1)
@@ -75,16 +75,16 @@ def test_gemm_token_counts(P, which, m):
 
 @pytest.mark.parametrize("bits", [3, 4])
 def test_gemm_more_tiles_than_sms(P, which, bits):
-    """9 x 17 = 153 output tiles of 256 x 256 on 148 SMs: the fused kernel cuts the (tile, K stage) sequence into equal
-    runs, so tiles are shared between two CTAs (partial sums through the workspace); sampled rows against the oracle,
-    and the two kernels against each other (a shared tile adds two fp32 partial sums, so the last bf16 bit may differ)."""
+    """153 output tiles of 256 x 256 on 74 pairs of SMs, ragged in both directions; sampled rows against the oracle.  fq_gemm takes
+    the two-pass way at this size, so the calls that are compared run the same kernels, one of them in the memory of the
+    first long prompts; test_gpu_prefill_plan.py compares the two ways."""
     n, k, m = 17 * 256 - 40, 640, 9 * 256 - 3
     codes, s, z = make_layer(115, bits, n, k, bits)
     fq = P.FlexQ(1)
     fq.fq_pack_layer(0, *to_dev(codes, s, z), bits, P.FQ_FMT_PACKED)
     x = x_bf16(115, bits, m, k).cuda()
     y = torch.full((m, n), float("nan"), dtype=torch.bfloat16, device="cuda")
-    for _ in range(2):                                   # twice: the partial-sum flags of the first launch are stale in the second
+    for _ in range(2):                                   # twice: the second one finds what the first one left
         _gemm(fq, which, 0, x, y)
     assert fq.fq_status() == 0
     other = torch.empty_like(y)

@@ -49,7 +49,8 @@ def test_token_counts_and_ragged_outputs(m, shape):
 
 @pytest.mark.parametrize("fmt_bits", [(0, 2), (0, 3), (0, 5), (0, 7), (0, 8), (1, 2), (1, 3), (1, 5), (1, 8)])
 def test_every_field_list_with_shared_tiles(fmt_bits):
-    """Two row tiles and 34 K stages: up to 17 CTAs share a tile, runs begin and end inside blobs."""
+    """Two row tiles and 34 K stages: 17 CTAs share a tile, runs begin and end inside blobs (none in two tiles: those are
+    test_gpu_prefill_plan.py's)."""
     import paper_2501_07139_b200 as P
     fmt, bits = fmt_bits
     n, k, m = 200, 34 * 128, 37
@@ -60,8 +61,9 @@ def test_every_field_list_with_shared_tiles(fmt_bits):
 
 def test_shared_tiles_do_not_depend_on_timing():
     import paper_2501_07139_b200 as P
-    n, k, m = 1408, 1152, 77
+    n, k, m = 640, 9984, 77
     fq, ref = _layer(P, 122, n, k, 4, P.FQ_FMT_PACKED)
+    assert fq.fq_gemm_plan(0, m)["shared"] and not fq.fq_gemm_plan(0, m)["two_pass"]
     x = x_bf16(122, 0, m, k).cuda()
     first = _check(fq, ref, x, n).clone()
     y = torch.empty((m, n), dtype=torch.bfloat16, device="cuda")
