@@ -14,6 +14,7 @@
 #include <cuda_fp16.h>
 
 #include "fq_layout.cuh"
+#include "fq_merge.cuh"
 #include "fq_ptx.cuh"
 
 namespace fq {
@@ -99,6 +100,60 @@ __device__ __forceinline__ void field_step(uint32_t fa, const uint4 (&bx)[4], in
     }
 }
 
+// The same for all fields of a nested child of three or more bits at once: its fields are merged first (fq_merge.cuh), so that one MMA
+// and one pass over the sums serve all of them instead of one each.  Two fields give 4-bit codes, two steps to a word, which are taken
+// apart like a stored 4-bit field; three and four give bytes.  v gets the sums in units of the parent's code.  The loop alone, 16
+// warps with everything in shared memory, weights a clock and SM at 4 / 6 / 8 bits: 60 / 40 / 32 one field at a time, 72 / 50 / 40 merged.
+//   fa : shared address of this lane's 16-byte chunk of field 0 of the tile, this superstep
+template <int VARIANT>
+__device__ __forceinline__ void nested_step(uint32_t fa, const uint4 (&bx)[4], int c, int m1, int (&v)[2][2])
+{
+    constexpr FieldList FL = variant_fields(VARIANT);
+    constexpr int N = FL.n, KEEP = FL.keep[N - 1];
+    static_for<0, 2>([&](auto GI) {                            // a field's chunk holds the four k32 steps of a group
+        constexpr int grp = decltype(GI)::value;
+        uint4 raw[N];
+        static_for<0, N>([&](auto FI) {
+            constexpr int fi = decltype(FI)::value;
+            raw[fi] = lds128<kBlobSteps * kBlobTiles * 512 * 2 * fi + grp * 512>(fa);
+        });
+        uint32_t a[4][4];                                      // [step][A register]
+        static_for<0, 4>([&](auto RI) {
+            constexpr int r = decltype(RI)::value;
+            uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+            for (int i = 0; i < N; i++) w[i] = r == 0 ? raw[i].x : r == 1 ? raw[i].y : r == 2 ? raw[i].z : raw[i].w;
+            if constexpr (N == 2) {
+                constexpr uint32_t m = KEEP == 2 ? 0x0f0f0f0fu : 0x0e0e0e0eu;
+                uint32_t even, odd;
+                merge_nibbles(w[0], w[1], even, odd);
+                a[0][r] = even & m; a[1][r] = odd & m;
+                if constexpr (KEEP == 2) {                     // high nibbles = word - low nibbles, as multiply-adds
+                    a[2][r] = (uint32_t)((int)a[0][r] * m1 + (int)even);
+                    a[3][r] = (uint32_t)((int)a[1][r] * m1 + (int)odd);
+                } else {
+                    a[2][r] = even & (m << 4); a[3][r] = odd & (m << 4);
+                }
+            } else {
+                uint32_t step[4];
+                merge_bytes<N, KEEP>(w, step);
+#pragma unroll
+                for (int t = 0; t < 4; t++) a[t][r] = step[t];
+            }
+        });
+        int acc[4];
+        static_for<0, 4>([&](auto TI) {
+            constexpr int t = decltype(TI)::value;
+            const uint32_t b0 = grp == 0 ? bx[t].x : bx[t].z, b1 = grp == 0 ? bx[t].y : bx[t].w;
+            if constexpr (t == 0) mma_u8s8_first(acc, a[t][0], a[t][1], a[t][2], a[t][3], b0, b1);
+            else mma_u8s8(acc, a[t][0], a[t][1], a[t][2], a[t][3], b0, b1);
+        });
+        const int up = N == 2 ? 4 - 4 * (c >> 1) : 0;          // 4-bit codes: steps 2 and 3 are in the high nibbles
+        v[grp][0] = (acc[1] * 256 + acc[0]) << up;
+        v[grp][1] = (acc[3] * 256 + acc[2]) << up;
+    });
+}
+
 // The fields of one (superstep, tile), unrolled at compile time from the variant's field list.
 template <int VARIANT, int FI, int PREFIX, int SS, int TILE>
 struct FieldLoop {
@@ -165,6 +220,7 @@ __device__ __forceinline__ void blob_compute(uint32_t blob, const uint32_t (&xd)
     // is the same as lowering every zero point by that amount
     constexpr int kAdjust = (VARIANT >= 7 && VARIANT < 13) ? 1 << (7 - (VARIANT - 5)) : 0;
     constexpr bool kUnrolled = variant_fields(VARIANT).n <= 2;
+    constexpr bool kMerged = VARIANT >= 7 && variant_fields(VARIANT).n >= 2;          // (nested_step)
     const int g = lane >> 2, c = lane & 3;
     const uint32_t fbase = blob + kBlobMetaBytes + lane * 16;
     const uint32_t mbase = blob + g * 16;
@@ -183,7 +239,8 @@ __device__ __forceinline__ void blob_compute(uint32_t blob, const uint32_t (&xd)
                 if (tsel == 2 - tile) return;                    // (warp-uniform) this tile belongs to another item
                 const uint4 mw = lds128<(ss * kBlobTiles + tile) * 128>(mbase);
                 int v[2][2];
-                FieldLoop<VARIANT, 0, 0, ss, tile>::run(fbase, bx, c, m1, v);
+                if constexpr (kMerged) nested_step<VARIANT>(fbase + (ss * kBlobTiles + tile) * 1024, bx, c, m1, v);
+                else FieldLoop<VARIANT, 0, 0, ss, tile>::run(fbase, bx, c, m1, v);
                 group_epilogue<kAdjust>(mw, v, nx, sc, tot[tile]);
             });
         });
@@ -201,7 +258,8 @@ __device__ __forceinline__ void blob_compute(uint32_t blob, const uint32_t (&xd)
                 const int st = ss * kBlobTiles + tile;
                 const uint4 mw = lds128(mbase + st * 128);
                 int v[2][2];
-                FieldLoopRt<VARIANT, 0, 0>::run(fbase, st, bx, c, m1, v);
+                if constexpr (kMerged) nested_step<VARIANT>(fbase + st * 1024, bx, c, m1, v);
+                else FieldLoopRt<VARIANT, 0, 0>::run(fbase, st, bx, c, m1, v);
                 float t2[2] = {0.f, 0.f};
                 group_epilogue<kAdjust>(mw, v, nx, sc, t2);
                 if (tile == 0) { tt[0][0] += t2[0]; tt[0][1] += t2[1]; }
