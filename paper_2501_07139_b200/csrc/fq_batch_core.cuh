@@ -10,7 +10,7 @@
 //   shifts is chosen at compile time per k32 step.
 //
 //   The constant is exact for z below 1024, which covers every quantiser of up to eight bits; stored zero points have 16 bits.  Where a
-//   context holds higher ones, their upper bits are taken out of a unit before it is computed (unit_take_high_zeros), in a kernel of
+//   context holds higher ones, their upper bits are taken out of a blob before it is computed (blob_take_high_zeros), in a kernel of
 //   its own: a test, a mask or one more register in the usual one costs 2 - 7 % of the 13B stack at batch 8.
 #pragma once
 #include <cuda_fp16.h>
@@ -18,6 +18,7 @@
 #include <cstdint>
 
 #include "fq_layout.cuh"
+#include "fq_merge.cuh"
 #include "fq_ptx.cuh"
 
 namespace fq {
@@ -26,7 +27,7 @@ namespace fq {
 FQ_HDC int batch_pad(int batch) { return batch <= 4 ? 4 : 8; }
 // Activations in shared memory: the rows as they are in global memory, kXRowPad bytes more than a chunk of `kXCols` columns
 // apart: the 8-byte loads of half a warp (four rows, four column runs) then hit every bank once.
-constexpr int kXCols = 1024;
+constexpr int kXCols = kBlobSteps * kStepCols;
 constexpr int kXRowPad = 32;
 constexpr int kXRowBytes = kXCols * 2 + kXRowPad;
 
@@ -110,20 +111,18 @@ __device__ __forceinline__ void group_mma(const uint32_t (&fa)[kMaxFields], uint
     });
 }
 
-// Supersteps first .. first + steps - 1 of a unit, one 16-row tile: tot[0..1] row g, tot[2..3] row g + 8, batch entries 2c, 2c + 1.
-//   stage : shared address of the unit's first blob        xs : of the activation slot
+// A blob, one 16-row tile: tot[0..1] row g, tot[2..3] row g + 8, batch entries 2c, 2c + 1.
+//   blob : its shared address        xs : of the activation slot
 template <int VARIANT, int BP>
-__device__ __forceinline__ void unit_compute(uint32_t stage, int first, int steps, uint32_t blob_read, uint32_t xs, int lane, int tile, float (&tot)[4])
+__device__ __forceinline__ void blob_compute(uint32_t blob, uint32_t xs, int lane, int tile, float (&tot)[4])
 {
     constexpr FieldList FL = variant_fields(VARIANT);
     const int g = lane >> 2, c = lane & 3;
     // batch entries beyond the padding read a valid entry's activations; nobody uses what they add up to
-    uint32_t xa = xs + (uint32_t)((g & (BP - 1)) * kXRowBytes + c * 8 + first * kStepCols * 2);
+    uint32_t xa = xs + (uint32_t)((g & (BP - 1)) * kXRowBytes + c * 8);
 #pragma unroll 1                                                     // (keeps the specialised loops small)
-    for (int s = first; s < first + steps; s++, xa += kStepCols * 2) {
-        const int ssl = s % kBlobSteps;
-        const uint32_t blob = stage + (uint32_t)(s / kBlobSteps) * blob_read;
-        const int st_tile = ssl * kBlobTiles + tile;
+    for (int ss = 0; ss < kBlobSteps; ss++, xa += kStepCols * 2) {
+        const int st_tile = ss * kBlobTiles + tile;
         uint32_t fa[kMaxFields];
         static_for<0, FL.n>([&](auto FI) {
             constexpr int fi = decltype(FI)::value;
@@ -149,20 +148,18 @@ __device__ __forceinline__ void unit_compute(uint32_t stage, int first, int step
     }
 }
 
-// Takes the zero points of a unit (this warp's part of it: nobody else reads those words) down to their low ten bits; tot gets what
+// Takes the zero points of a blob's row tile (nobody else reads those words) down to their low ten bits; tot gets what
 // that leaves out, -s * (upper bits of z) * (sum of the activations) over the groups.  The sums come from MMAs whose weights are all
 // one, in the layout of tot.
 template <int BP>
-__device__ __forceinline__ void unit_take_high_zeros(uint32_t stage, int first, int steps, uint32_t blob_read, uint32_t xs, int lane, int tile,
-                                                     float (&tot)[4])
+__device__ __forceinline__ void blob_take_high_zeros(uint32_t blob, uint32_t xs, int lane, int tile, float (&tot)[4])
 {
     constexpr uint32_t kOnes = 0x3c003c00u;                           // 1.0 twice
     const int g = lane >> 2, c = lane & 3;
-    uint32_t xa = xs + (uint32_t)((g & (BP - 1)) * kXRowBytes + c * 8 + first * kStepCols * 2);
+    uint32_t xa = xs + (uint32_t)((g & (BP - 1)) * kXRowBytes + c * 8);
 #pragma unroll 1
-    for (int i = 2 * first; i < 2 * (first + steps); i++, xa += kGroup * 2) {     // one group at a time
-        const int ssl = i / 2 % kBlobSteps;
-        const uint32_t words = stage + (uint32_t)(i / 2 / kBlobSteps) * blob_read + (uint32_t)((ssl * kBlobTiles + tile) * 128 + g * 16 + (i & 1) * 8);
+    for (int i = 0; i < 2 * kBlobSteps; i++, xa += kGroup * 2) {      // one group at a time
+        const uint32_t words = blob + (uint32_t)((i / 2 * kBlobTiles + tile) * 128 + g * 16 + (i & 1) * 8);
         const uint2 m = lds64(words);                                 // rows g, g + 8
         if (!__any_sync(0xffffffffu, ((m.x | m.y) >> 26) != 0u)) continue;
         float sums[4] = {0.f, 0.f, 0.f, 0.f};
@@ -179,14 +176,13 @@ __device__ __forceinline__ void unit_take_high_zeros(uint32_t stage, int first, 
         if (c == 0) sts64(words, make_uint2(m.x & 0x03ffffffu, m.y & 0x03ffffffu));           // (all lanes have read them: the vote)
     }
     __syncwarp();
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the next copy into the stage comes after these stores
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the next copy into this place comes after these stores
 }
 
 template <int BP>
-__device__ __forceinline__ void unit_dispatch(int variant, uint32_t stage, int first, int steps, uint32_t blob_read, uint32_t xs, int lane, int tile,
-                                              float (&tot)[4])
+__device__ __forceinline__ void blob_dispatch(int variant, uint32_t blob, uint32_t xs, int lane, int tile, float (&tot)[4])
 {
-#define FQ_VARIANT_CASE(V) case V: unit_compute<V, BP>(stage, first, steps, blob_read, xs, lane, tile, tot); break;
+#define FQ_VARIANT_CASE(V) case V: blob_compute<V, BP>(blob, xs, lane, tile, tot); break;
     switch (variant) {
         FQ_VARIANT_CASE(0) FQ_VARIANT_CASE(1) FQ_VARIANT_CASE(2) FQ_VARIANT_CASE(3) FQ_VARIANT_CASE(4)
         FQ_VARIANT_CASE(5) FQ_VARIANT_CASE(6) FQ_VARIANT_CASE(7) FQ_VARIANT_CASE(8) FQ_VARIANT_CASE(9)

@@ -131,13 +131,14 @@ int fill_op(const Ctx* ctx, int layer, const uint16_t* x, uint16_t* y, int batch
     op.k_in = L.k_in;
     op.n_kb = k_blobs(L.k_in);
     op.n_rp = row_pairs(L.n_out);
-    op.chunk_blobs = one ? gemv1_chunk_blobs(op.blob_read)
-                                : gemv_chunk_blobs(L.fmt == FQ_FMT_PLANES ? plane_read_bits(bits) : bits);
-    op.n_chunks = (op.n_kb + op.chunk_blobs - 1) / op.chunk_blobs;
+    op.chunk_blobs = one ? gemv1_chunk_blobs(op.blob_read) : 1;
+    op.n_chunks = op.n_kb;                                       // batch 2..8: a chunk of K is a blob
     op.batch = batch;
     // what is dealt to the CTAs: batch 1 the blobs of every strip, batch 2..8 the K chunks of every row pair
-    op.n_units = (one ? op.n_kb : op.n_chunks) * op.n_rp;
-    if ((long long)op.n_units * 1024 >= (1ll << 31)) return FQ_ERR_SHAPE;              // 32-bit unit arithmetic on the device
+    op.n_units = op.n_kb * op.n_rp;
+    // 32-bit unit arithmetic on the device (batch 2..8: blobs of up to four bits have always counted in pairs)
+    const int pair = !one && op.blob_read <= blob_bytes(4) ? 2 : 1;
+    if ((long long)((op.n_kb + pair - 1) / pair) * op.n_rp * 1024 >= (1ll << 31)) return FQ_ERR_SHAPE;
     if (one && (batch != 1 || L.k_in > gemv1_max_k())) return FQ_ERR_SHAPE;                   // a strip's activations stay in shared memory
     op.phase = -1;
     op.rot = 0;
@@ -152,7 +153,6 @@ int fill_op(const Ctx* ctx, int layer, const uint16_t* x, uint16_t* y, int batch
 size_t op_partial_bytes(const GemvOp& op, bool one, int max_batch)
 {
     if (one) return op.n_kb <= 1 ? 0 : (size_t)op.n_rp * op.n_kb * 32 * sizeof(unsigned long long);
-    if (op.n_chunks <= 1) return 0;
     return (size_t)op.n_rp * op.n_chunks * gemv_partial_bytes_per_unit(max_batch);
 }
 

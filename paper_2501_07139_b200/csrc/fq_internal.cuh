@@ -43,7 +43,7 @@ struct GemvOp {
     int n_out, k_in;
     int n_kb;                    // k blobs
     int n_rp;                    // row pairs = units per K chunk
-    int chunk_blobs;             // k blobs per K chunk (the last chunk may be shorter)
+    int chunk_blobs;             // batch 1: k blobs that one stage of the ring holds, at most
     int phase;                   // -1: no ordering
     int n_units;                 // n_chunks * n_rp
     int rot;                     // rotation of the CTA blocks for this op (evens out remainders); inline ops: its first strip counter
@@ -133,8 +133,6 @@ int current_sm_count();
 
 int launch_stream_read(const void* src, size_t bytes, unsigned* sink, int sm_count, cudaStream_t st);
 
-// Chunking policy of the decode kernel: k blobs (512 columns) per K chunk.
-int gemv_chunk_blobs(int bits);
 size_t gemv_partial_bytes_per_unit(int batch);
 int launch_gemv_single(Ctx* ctx, const GemvOp& op, cudaStream_t st);                 // batch 2..8
 // parts == nullptr: whole tiles only; else tiles may be shared between CTAs through these slots
