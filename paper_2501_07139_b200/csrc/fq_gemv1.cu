@@ -239,68 +239,62 @@ __device__ CtaWork inline_work(const GemvOp* ops, int oi, int n_ops, int cta, in
 }
 
 // ------------------------------------------------------------------------------- activation pre-processing
+__device__ __forceinline__ uint32_t max_u16x2(uint32_t x, uint32_t y)
+{
+    uint32_t r;
+    asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(y));
+    return r;
+}
 // One blob (two supersteps of 256 columns, 8 per lane each) of fp16 activations -> fixed point per group of
 // 128 columns: x_int = rint(x * 2^(13 - E)) with 2^E <= max|x| < 2^(E+1), stored as two signed byte digits in
 // B-fragment order, plus per group the integer sum and the factor 2^(E - 13).  A group that holds an
 // infinity or a NaN gets the factor NaN, so that every row sum that touches it comes out NaN.  The two
 // supersteps are independent chains of shuffles and conversions: written side by side so that their
 // latencies overlap.
+// This loop competes with the consumers for issue slots: packed maxima, one fma per value instead of a multiplication and a
+// conversion, and byte sums (dp4a) take two thirds of the instructions of doing each of these element by element (four 7B blocks in
+// order, 4 bits 162.7 -> 161.3 us, nested 6 bits 229.4 -> 228).
 __device__ __forceinline__ void convert_blob(const uint4 (&raw)[2], uint8_t* xdig, uint8_t* xgrp, int lane)
 {
-    float f[2][8], amax[2];
-    bool bad[2];
+    // the largest magnitude of a group, as the bits of a half: an infinity or a NaN (0x7c00 and above) is larger than any
+    // number.  Both supersteps in one word: low half the first.
+    uint32_t top[2];
 #pragma unroll
-    for (int ss = 0; ss < 2; ss++) {
-        const __half2* h2 = reinterpret_cast<const __half2*>(&raw[ss]);
+    for (int ss = 0; ss < 2; ss++)
+        top[ss] = max_u16x2(max_u16x2(raw[ss].x & 0x7fff7fffu, raw[ss].y & 0x7fff7fffu), max_u16x2(raw[ss].z & 0x7fff7fffu, raw[ss].w & 0x7fff7fffu));
+    uint32_t amax = max_u16x2(__byte_perm(top[0], top[1], 0x5410), __byte_perm(top[0], top[1], 0x7632));
 #pragma unroll
-        for (int i = 0; i < 4; i++) {
-            const float2 t2 = __half22float2(h2[i]);
-            f[ss][2 * i] = t2.x; f[ss][2 * i + 1] = t2.y;
-        }
-        float m01 = fmaxf(fabsf(f[ss][0]), fabsf(f[ss][1])), m23 = fmaxf(fabsf(f[ss][2]), fabsf(f[ss][3]));
-        float m45 = fmaxf(fabsf(f[ss][4]), fabsf(f[ss][5])), m67 = fmaxf(fabsf(f[ss][6]), fabsf(f[ss][7]));
-        amax[ss] = fmaxf(fmaxf(m01, m23), fmaxf(m45, m67));
-        // an infinity or a NaN: |x| <= 65504 fails for both (fmaxf drops a NaN, so test the elements)
-        bool ok = true;
-#pragma unroll
-        for (int i = 0; i < 8; i++) ok = ok && (fabsf(f[ss][i]) <= 65504.f);
-        bad[ss] = !ok;
-    }
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) {
-        amax[0] = fmaxf(amax[0], __shfl_xor_sync(0xffffffffu, amax[0], o));
-        amax[1] = fmaxf(amax[1], __shfl_xor_sync(0xffffffffu, amax[1], o));
-    }
-    const unsigned badmask0 = __ballot_sync(0xffffffffu, bad[0]), badmask1 = __ballot_sync(0xffffffffu, bad[1]);
-    bad[0] = ((badmask0 >> (lane & 16)) & 0xffffu) != 0u;       // anywhere in this lane's group of 16 lanes
-    bad[1] = ((badmask1 >> (lane & 16)) & 0xffffu) != 0u;
-    int xi[2][8], sum[2];
+    for (int o = 8; o > 0; o >>= 1) amax = max_u16x2(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    uint32_t xi[2][8];                                               // x_int in the low 16 bits
     float back[2];
 #pragma unroll
     for (int ss = 0; ss < 2; ss++) {
-        const int eb = (__float_as_int(amax[ss]) >> 23) & 0xff;  // biased exponent of the group maximum
-        const bool fin = amax[ss] > 0.f && !bad[ss];
+        const uint32_t m = ss ? amax >> 16 : amax & 0xffffu;
+        const bool bad = m >= 0x7c00u, fin = m > 0u && !bad;
+        const int eb = __float_as_int(__half2float(__ushort_as_half((unsigned short)m))) >> 23;      // biased exponent of the group maximum
         const float mult = fin ? __int_as_float((267 - eb) << 23) : 0.f;
-        back[ss] = bad[ss] ? __int_as_float(0x7fc00000) : (fin ? __int_as_float((eb - 13) << 23) : 0.f);
+        back[ss] = bad ? __int_as_float(0x7fc00000) : (fin ? __int_as_float((eb - 13) << 23) : 0.f);
+        const uint32_t keep = bad ? 0u : ~0u;                        // (nothing of such a group counts but the factor)
+        const uint32_t w[4] = {raw[ss].x & keep, raw[ss].y & keep, raw[ss].z & keep, raw[ss].w & keep};
 #pragma unroll
-        for (int i = 0; i < 8; i++) xi[ss][i] = bad[ss] ? 0 : __float2int_rn(f[ss][i] * mult);
-        sum[ss] = ((xi[ss][0] + xi[ss][1]) + (xi[ss][2] + xi[ss][3])) + ((xi[ss][4] + xi[ss][5]) + (xi[ss][6] + xi[ss][7]));
-    }
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) {
-        sum[0] += __shfl_xor_sync(0xffffffffu, sum[0], o);
-        sum[1] += __shfl_xor_sync(0xffffffffu, sum[1], o);
+        for (int i = 0; i < 4; i++) {
+            // 1.5 * 2^23 + x * mult, rounded once to an integer (ties to even): the low bits are the integer
+            const float2 t2 = __half22float2(*reinterpret_cast<const __half2*>(&w[i]));
+            xi[ss][2 * i] = __float_as_uint(fmaf(t2.x, mult, 12582912.f));
+            xi[ss][2 * i + 1] = __float_as_uint(fmaf(t2.y, mult, 12582912.f));
+        }
     }
     // lane l holds columns 8l .. 8l+7 of a superstep: k32 step j = l >> 2, half (l >> 1) & 1, column blocks c0, c0 + 1
     const int j = lane >> 2, half = (lane >> 1) & 1, c0 = 2 * (lane & 1);
+    int sum[2];
 #pragma unroll
     for (int ss = 0; ss < 2; ss++) {
         // signed digits base 256 of four values at a time: low byte as is, high byte + carry
         uint32_t lo4[2], hi4[2];
 #pragma unroll
         for (int r = 0; r < 2; r++) {
-            const uint32_t p01 = __byte_perm((uint32_t)xi[ss][4 * r + 0], (uint32_t)xi[ss][4 * r + 1], 0x5410);
-            const uint32_t p23 = __byte_perm((uint32_t)xi[ss][4 * r + 2], (uint32_t)xi[ss][4 * r + 3], 0x5410);
+            const uint32_t p01 = __byte_perm(xi[ss][4 * r], xi[ss][4 * r + 1], 0x5410);
+            const uint32_t p23 = __byte_perm(xi[ss][4 * r + 2], xi[ss][4 * r + 3], 0x5410);
             const uint32_t h01 = (((p01 >> 8) & 0x00ff00ffu) + ((p01 >> 7) & 0x00010001u)) & 0x00ff00ffu;
             const uint32_t h23 = (((p23 >> 8) & 0x00ff00ffu) + ((p23 >> 7) & 0x00010001u)) & 0x00ff00ffu;
             lo4[r] = __byte_perm(p01, p23, 0x6420);
@@ -311,12 +305,23 @@ __device__ __forceinline__ void convert_blob(const uint4 (&raw)[2], uint8_t* xdi
         *reinterpret_cast<uint32_t*>(cell + 16) = lo4[1];
         *reinterpret_cast<uint32_t*>(cell + 64) = hi4[0];
         *reinterpret_cast<uint32_t*>(cell + 64 + 16) = hi4[1];
-        if ((lane & 15) == 0) {
+        sum[ss] = __dp4a((int)lo4[0], 0x01010101, __dp4a((int)lo4[1], 0x01010101, 0)) +
+                  256 * __dp4a((int)hi4[0], 0x01010101, __dp4a((int)hi4[1], 0x01010101, 0));
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+        sum[0] += __shfl_xor_sync(0xffffffffu, sum[0], o);
+        sum[1] += __shfl_xor_sync(0xffffffffu, sum[1], o);
+    }
+    if ((lane & 15) == 0) {
+#pragma unroll
+        for (int ss = 0; ss < 2; ss++) {
             reinterpret_cast<int*>(xgrp)[ss * 2 + (lane >> 4)] = sum[ss];
             reinterpret_cast<float*>(xgrp + 16)[ss * 2 + (lane >> 4)] = back[ss];
         }
     }
 }
+
 
 // ------------------------------------------------------------------------------- the kernel
 __global__ void __launch_bounds__(kThreads, 1)
