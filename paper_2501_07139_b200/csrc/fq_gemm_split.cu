@@ -402,12 +402,12 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_x, const SplitArgs a)
                         out[(t0 / 4 + e) * kRows] = make_float4(__uint_as_float(v[4 * e]), __uint_as_float(v[4 * e + 1]),
                                                                 __uint_as_float(v[4 * e + 2]), __uint_as_float(v[4 * e + 3]));
                 }
-                __threadfence();
+                fence_gpu();
                 __syncwarp();
                 if (lane == 0 && atomicAdd(const_cast<int*>(&due[2 + (local > 0)]), 1) == 3) {    // the fourth epilogue warp
-                    __threadfence();
+                    fence_cta();                                        // (the other three warps' sums, too)
                     const Sharers sh(run, it.tile);
-                    if (atomicAdd(a.arrived + sh.c0, 1u) == (unsigned)(sh.c1 - sh.c0)) {
+                    if (atom_add_acq_rel(a.arrived + sh.c0, 1u) == (unsigned)(sh.c1 - sh.c0)) {
                         a.arrived[sh.c0] = 0u;
                         due[local > 0] = 1;
                     }
@@ -419,7 +419,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_x, const SplitArgs a)
             if (lane == 0) mbar_arrive(tempty);
         }
         if (a.parts) {
-            if (lane == 0) { __threadfence(); mbar_arrive(sums_due); }
+            if (lane == 0) mbar_arrive(sums_due);
             if (ok) ok = __all_sync(0xffffffffu, g_wait(sums_due, 0u, abort_flag));
             if (ok) add_shared_tiles(a, due, quarter, 0, lane);
         }

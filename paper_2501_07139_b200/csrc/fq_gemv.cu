@@ -312,12 +312,12 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                         const int b = i / ((cols - have) / 8), k = have + i % ((cols - have) / 8) * 8;
                         sts128(xs + (uint32_t)(b * kXRowBytes + k * 2), make_uint4(0u, 0u, 0u, 0u));
                     }
-                __threadfence_block();
+                fence_cta();
                 __syncwarp();
                 if (lane == 0) {
                     // all that can be done before the phase opens; from here on the consumers sleep on the slot's barrier
                     x_pending[slot] = units * kWarpsPerUnit;
-                    __threadfence_block();
+                    fence_cta();
                     x_ready[slot] = seg + 1;
                     // the activations are the previous phase's outputs
                     if (!flags[0] && op.phase > 0 && phase_known < op.phase - 1) {
@@ -331,7 +331,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                         }
                     }
                     // other SMs' plain stores (y of the previous phase) and this SM's reads of the slot before the copies below
-                    __threadfence_block();
+                    fence_cta();
                     asm volatile("fence.proxy.async;" ::: "memory");
                     go = flags[1] ? 0 : (flags[0] ? 2 : 1);
                     if (go == 1) mbar_expect_tx(bar, (uint32_t)(op.batch * have * 2));
@@ -366,7 +366,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
         auto count = [&] {                                               // all of them are: the last of the warps to say so counts them
             if (uncounted > 0 && phase >= 0) {
                 __syncwarp();
-                __threadfence();                                         // y before the phase counter
+                fence_gpu();                                         // y before the phase counter
                 if (lane == 0 && atomicAdd(const_cast<unsigned*>(&finished[phase & 3]), 1u) == kOutputWarps - 1u) {
                     finished[phase & 3] = 0u;
                     red_add_relaxed_u64(sa.phase_done + phase, (unsigned long long)uncounted);
@@ -492,7 +492,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                 if (x_ready[slot] != d.seg + 1 && !flags[1]) mbar_wait(xbars + 8 * slot, xpar, sa.wait_ns);
                 if (!smem_wait([&] { return x_ready[slot] == d.seg + 1 || flags[1]; }, sa.wait_ns) || (!flags[1] && !mbar_wait(xbars + 8 * slot, xpar, sa.wait_ns)))
                     give_up(sa.status, flags);
-                __threadfence_block();
+                fence_cta();
                 seg_seen = d.seg;
             }
             const bool live = __all_sync(0xffffffffu, flags[0] == 0);
@@ -524,12 +524,12 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
 
     __syncthreads();
     if (threadIdx.x == 0 && sa.n_phases > 0) {
-        __threadfence();
+        fence_gpu();
         const unsigned old = atomicAdd(sa.exit_count, 1u);
         if (old == gridDim.x - 1) {                    // last CTA out: counters back to zero
             for (int p = 0; p < sa.n_phases; p++) sa.phase_done[p] = 0ull;
             *sa.exit_count = 0u;
-            __threadfence();
+            fence_gpu();
         }
     }
 }

@@ -464,7 +464,7 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
                     else d = make_uint4((uint32_t)(cur.rot + rp), 0u, 0u, 0u);
                     if (lane < 4) sts128(sdesc_a + (uint32_t)sslot * 64u + (uint32_t)lane * 16u, d);
                     if (lane == 0) ctl[S::cStripBusy + sslot] = 1u;
-                    __threadfence_block();                           // the descriptor before any item that refers to it
+                    fence_cta();                           // the descriptor before any item that refers to it
                     __syncwarp();
                 }
                 const uint8_t* src = store + ((long long)rp * n_kb + kb_lo) * blob_stride;
@@ -601,7 +601,7 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
                             }
                             if (ok) ctl[S::cPhaseKnown] = (unsigned)(p + 1);
                         }
-                        __threadfence_block();
+                        fence_cta();
                         ctl[S::cPollLock] = 0u;
                         break;
                     }
@@ -637,12 +637,11 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
                 const uint4 raw[2] = {r0, r1};
                 convert_blob(raw, xdig, xgrp, lane);
             }
-            __threadfence_block();
+            fence_cta();
             __syncwarp();
             if (lane == 0) {
                 ctl[S::cXCnt + slot] = (unsigned)it.uses;
                 ctl[S::cXTag + slot] = it.xs + 1u;
-                __threadfence_block();
                 mbar_arrive(bars + 256 + 8 * slot);                        // wakes the consumers that sleep on this slot
             }
             return true;
@@ -708,7 +707,6 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
                 let_copies_land();
                 break;
             }
-            __threadfence_block();
             const uint32_t xdig = sbase + S::oXDig + (uint32_t)xslot * kXBlobDigitBytes;
             uint32_t xd[4];
 #pragma unroll
@@ -742,14 +740,14 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
                     else st_relaxed_u64(dpart + kb * 32 + lr, tag | __float_as_uint(v));   // finished elsewhere
                 }
             }
-            __threadfence_block();
+            fence_cta();
             __syncwarp();
             int last = 0;
             if (lane == 0) last = atomicAdd(const_cast<unsigned*>(&ctl[S::cStripCnt + sslot]), 1u) + 1u == (unsigned)expect;
             last = __shfl_sync(0xffffffffu, last, 0);
             if (!last) continue;
             // ---- this warp delivered the strip's last item
-            __threadfence_block();
+            fence_cta();
             bool live = true;
             if (finish) {
                 // lane = row of the strip; blob sums in blob order: this CTA's from shared memory, then the blobs
@@ -796,13 +794,13 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
                 // a shared strip of a launch without dependencies: whoever publishes the last blob sum adds all of them up, in
                 // blob order.  Nobody waits for a CTA that may not be running yet.
                 const int mine = d.kb_hi - d.kb_lo, n_kb = d.n_kb;
-                __threadfence();                                             // the sums of this CTA's items before the count
+                fence_gpu();                                             // the sums of this CTA's items before the count
                 __syncwarp();
                 unsigned before = 0;
                 if (lane == 0 && FQ_IN_BOUNDS(d.counter >= 0 && d.counter < kArrivedMax, a.status)) before = atomicAdd(a.arrived + d.counter, (unsigned)mine);
                 before = __shfl_sync(0xffffffffu, before, 0);
                 if ((int)before + mine == n_kb) {
-                    __threadfence();
+                    fence_gpu();
                     float sum = 0.f;
                     for (int q0 = 0; q0 < n_kb; q0 += 8) {
                         unsigned long long wv[8];
@@ -820,12 +818,12 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
             __syncwarp();
             if (lane == 0) {
                 ctl[S::cStripCnt + sslot] = 0u;
-                __threadfence_block();
+                fence_cta();
                 ctl[S::cStripBusy + sslot] = 0u;                             // the producer may reuse the slot
             }
             if (!live) { let_copies_land(); break; }
             if (finish && phase >= 0) {
-                __threadfence();                                             // y before the phase counter
+                fence_gpu();                                             // y before the phase counter
                 __syncwarp();
                 if (lane == 0) {
                     const unsigned done = atomicAdd(const_cast<unsigned*>(&ctl[S::cFinCnt + (phase & 7)]), 1u) + 1u;
@@ -840,12 +838,12 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
 
     __syncthreads();
     if (threadIdx.x == 0 && a.n_phases > 0) {
-        __threadfence();
+        fence_gpu();
         const unsigned old = atomicAdd(a.exit_count, 1u);
         if (old == gridDim.x - 1) {                    // last CTA out: counters back to zero
             for (int p = 0; p < a.n_phases; p++) a.phase_done[p] = 0ull;
             *a.exit_count = 0u;
-            __threadfence();
+            fence_gpu();
         }
     }
 }
