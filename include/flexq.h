@@ -90,8 +90,9 @@ int fq_quantize_layer(const float* w_dev, int n_out, int k_in, int bits, int gro
  *   scales_dev, zeros_dev   fp16 [n_out][k_in/128]; read, not retained.  Zero points are integers of any size
  *           that fp16 holds; a context that holds one above 1023 decodes batch 2..8 a little slower.
  *   store_out_dev fq_store_bytes() bytes, 256-byte aligned; written and RETAINED.
- *     (Calls read it while the stream's previous kernel ends, so a kernel of the caller's that lets its
- *     successors begin early must not be the one that writes it.)
+ *     (fq_gemm may read it while the stream's previous kernel ends, unless a call of this library has stored weights or
+ *     changed the configuration since the stream's last fq_gemm.  Whoever changes these bytes with a kernel of their own
+ *     therefore calls fq_set_config, with the same widths if need be, between that and the next fq_gemm.)
  * The first variant packed for a layer becomes its active one. */
 int fq_pack_layer(fq_ctx* ctx, int layer, int n_out, int k_in, int bits, int group, int fmt,
                   const uint8_t* codes_dev, const uint16_t* scales_dev, const uint16_t* zeros_dev,

@@ -186,8 +186,7 @@ static bool allocate_status(Ctx* ctx)
     return cudaMemset(p, 0, kHead + (ctx->fused_ws ? counts : 0)) == cudaSuccess;
 }
 
-// Is the work that is enqueued on `st` recorded into a graph?
-static bool is_capturing(cudaStream_t st)
+bool is_capturing(cudaStream_t st)
 {
     cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;
@@ -358,6 +357,7 @@ int fq_pack_layer(fq_ctx* ctx, int layer, int n_out, int k_in, int bits, int gro
                                (cudaStream_t)stream);
     if (rc != FQ_OK) return rc;
     ctx->stored++;
+    ctx->stores_in_graphs = ctx->stores_in_graphs || is_capturing((cudaStream_t)stream);
     const bool first_variant = !L.registered;
     L.registered = true;
     L.n_out = n_out; L.k_in = k_in; L.fmt = fmt;
@@ -510,6 +510,7 @@ int fq_transition_swap(fq_ctx* ctx, const uint8_t* to_bits_host, int n_layers, i
                 return FQ_ERR_CUDA;
             }
             ctx->stored++;
+            ctx->stores_in_graphs = ctx->stores_in_graphs || is_capturing(st);
             nv.store = p; nv.present = true; nv.swap_owned = true;
             rep.bytes_loaded += nbytes;
             resident_extra += nbytes;

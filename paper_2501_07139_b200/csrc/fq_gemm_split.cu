@@ -268,11 +268,12 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_x, const SplitArgs a)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = *tmem_ptr;
-    // Everything above may run while the previous kernel of the stream finishes, and so may the dequantisation: the stored blobs are
-    // written by kernels and copies that end before their successors begin (flexq.h), so the first four stages of weights are in TMEM
-    // when X may be read.  X, Y and the workspace may be the previous kernel's: the other warps wait, and a dequantisation warp comes to
-    // the workspace and to Y (add_shared_tiles) only after the epilogue's arrivals.  A call, us, all warps waiting -> these not:
-    // 4096 x 4096 at 77 tokens 16.2 -> 15.0, at 160 20.3 -> 18.9; 11008 x 4096 at 77 18.7 -> 17.7, at 300 36.6 -> 35.1.
+    // Everything above may run while the previous kernel of the stream finishes, and so may the dequantisation of the first four
+    // stages: whatever wrote the stored blobs has come before an earlier launch of this kernel, or this launch does not overlap at all
+    // (launch_gemm_split), so that weights are in TMEM when X may be read.  X, Y and the workspace may be the previous kernel's: the other
+    // warps wait, and a dequantisation warp comes to the workspace and to Y (add_shared_tiles) only after the epilogue's arrivals.  A
+    // call, us, all warps waiting -> these not: 4096 x 4096 at 77 tokens 16.2 -> 15.0, at 160 20.3 -> 18.9; 11008 x 4096 at 77 18.7 -> 17.7,
+    // at 300 36.6 -> 35.1.
     if (warp < 6) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -519,20 +520,21 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_x, const SplitArgs a)
     }
 }
 
+//   overlap : start while the previous kernel of the stream drains
 template <int VARIANT>
-int launch_variant(Ctx* ctx, const CUtensorMap& map_x, const SplitArgs& a, int grid, cudaStream_t st)
+int launch_variant(Ctx* ctx, const CUtensorMap& map_x, const SplitArgs& a, int grid, bool overlap, cudaStream_t st)
 {
     static bool configured[64] = {};
     if (ctx->device < 64 && !configured[ctx->device]) {
         FQ_CUDA_OK(cudaFuncSetAttribute(gemm_split_kernel<VARIANT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SplitSmem::kTotal));
         configured[ctx->device] = true;
     }
-    cudaLaunchAttribute overlap{};                  // start while the previous kernel of the stream drains (see the kernel)
-    overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    overlap.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute early{};
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = SplitSmem::kTotal;
-    cfg.stream = st; cfg.attrs = &overlap; cfg.numAttrs = 1;
+    cfg.stream = st; cfg.attrs = &early; cfg.numAttrs = overlap ? 1u : 0u;
     FQ_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_split_kernel<VARIANT>, map_x, a));
     return FQ_OK;
 }
@@ -613,13 +615,25 @@ int launch_gemm_split(Ctx* ctx, const void* store, int blob_stride, int blob_rea
         a.parts = parts; a.arrived = arrived;
         a.run_base = (unsigned)(plan.pairs / grid); a.run_extra = (unsigned)(plan.pairs % grid);
     }
+    // An overlapping launch reads stored weights while the stream's previous kernel may still be running, and where that one wrote
+    // them (fq_pack_layer) nothing makes them visible before griddepcontrol.wait.  So the first launch on a stream after anything that
+    // stores weights or changes the configuration comes after all of the stream's work, without overlap: what was stored before it is
+    // in place for every later launch there.  A launch that is only captured orders nothing, and a captured call that stores weights
+    // runs whenever its graph does: contexts with such calls do without overlap.
+    const bool overlap = !ctx->stores_in_graphs && ctx->gemm_after_stores_at == ctx->config_epoch && ctx->gemm_after_stores_on == st;
+    int launched = FQ_ERR_ARG;
     switch (variant) {
-#define FQ_CASE(V) case V: return launch_variant<V>(ctx, map_x, a, (int)grid, st);
+#define FQ_CASE(V) case V: launched = launch_variant<V>(ctx, map_x, a, (int)grid, overlap, st); break;
         FQ_CASE(0) FQ_CASE(1) FQ_CASE(2) FQ_CASE(3) FQ_CASE(4) FQ_CASE(5) FQ_CASE(6)
         FQ_CASE(7) FQ_CASE(8) FQ_CASE(9) FQ_CASE(10) FQ_CASE(11) FQ_CASE(12) FQ_CASE(13)
 #undef FQ_CASE
-        default: return FQ_ERR_ARG;
+        default: break;
     }
+    if (launched == FQ_OK && !overlap && !is_capturing(st)) {
+        ctx->gemm_after_stores_at = ctx->config_epoch;
+        ctx->gemm_after_stores_on = st;
+    }
+    return launched;
 }
 
 }  // namespace fq

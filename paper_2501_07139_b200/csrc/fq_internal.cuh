@@ -78,6 +78,10 @@ struct Ctx {
     size_t gemm_ws_refused = 0;          // size that could not be had, under this configuration
     uint64_t gemm_ws_refused_at = ~0ull;
     int gemm_sliced = 0;                 // calls that did without a larger gemm_ws
+    // prefill: everything that wrote stored weights came before a launch on this stream, as of this configuration (see launch_gemm_split)
+    cudaStream_t gemm_after_stores_on = nullptr;
+    uint64_t gemm_after_stores_at = ~0ull;
+    bool stores_in_graphs = false;       // a captured call stores weights: nobody here sees when its graph runs
     char* fused_ws = nullptr;            // prefill: counters, then two fp32 tile slots per SM (part of the allocation of status_dev)
     std::vector<void*> owned;    // device buffers freed by fq_destroy: those of fq_load, workspaces that graphs may hold
     uint64_t config_epoch = 0;
@@ -100,6 +104,8 @@ struct Ctx {
 // Device word that is not 0 once a zero point above 1023 has been stored by any call on the context (it is never cleared).
 inline unsigned* high_zeros_word(const Ctx* ctx) { return reinterpret_cast<unsigned*>(ctx->status_dev) + 1; }
 
+// Is the work that is enqueued on `st` recorded into a graph?
+bool is_capturing(cudaStream_t st);
 // Bytes of device workspace for `n_ops` ops whose split-K needs are summed by the caller.
 int ensure_workspace(Ctx* ctx, size_t bytes);
 
