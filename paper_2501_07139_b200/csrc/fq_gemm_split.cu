@@ -271,9 +271,8 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_x, const SplitArgs a)
     // Everything above may run while the previous kernel of the stream finishes, and so may the dequantisation of the first four
     // stages: whatever wrote the stored blobs has come before an earlier launch of this kernel, or this launch does not overlap at all
     // (launch_gemm_split), so that weights are in TMEM when X may be read.  X, Y and the workspace may be the previous kernel's: the other
-    // warps wait, and a dequantisation warp comes to the workspace and to Y (add_shared_tiles) only after the epilogue's arrivals.  A
-    // call, us, all warps waiting -> these not: 4096 x 4096 at 77 tokens 16.2 -> 15.0, at 160 20.3 -> 18.9; 11008 x 4096 at 77 18.7 -> 17.7,
-    // at 300 36.6 -> 35.1.
+    // warps wait here, the dequantisation warps after their first stage.  A call, us, all warps waiting here -> these not:
+    // 4096 x 4096 at 77 tokens 16.2 -> 15.0, at 160 20.3 -> 18.9; 11008 x 4096 at 77 18.7 -> 17.7, at 300 36.6 -> 35.1.
     if (warp < 6) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -460,7 +459,9 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_x, const SplitArgs a)
 #pragma unroll
                 for (int tl = 0; tl < kBlobTiles; tl++)
                     meta[tl] = __ldg(reinterpret_cast<const uint2*>(blob + blob_meta_off(ssl, tl) + blob_meta_word(grp, g)));
-                // ---- the stage's columns of TMEM must be free (the MMAs that read their previous contents are done)
+                // ---- the stage's columns of TMEM must be free (the MMAs that read their previous contents are done).  The MMAs begin
+                // when the previous kernel has ended, however long that takes: only then does a wait for them have a limit
+                if (wraps == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
                 const bool is_free = wraps == 0 || g_wait(empty0 + 8 * stage, (wraps - 1u) & 1u, abort_flag);
                 if (!__all_sync(0xffffffffu, is_free)) { ok = false; break; }      // (the lanes must leave together)
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -500,6 +501,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_x, const SplitArgs a)
                 if (lane == 0) mbar_arrive(full0 + 8 * stage);
             }
         }
+        if (wraps <= 1) asm volatile("griddepcontrol.wait;" ::: "memory");
         if (a.parts) {
             if (ok) ok = __all_sync(0xffffffffu, g_wait<64>(sums_due, 0u, abort_flag));
             if (ok) add_shared_tiles(a, due, dw, 1 + grp_id, lane);
