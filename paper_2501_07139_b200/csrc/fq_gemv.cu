@@ -366,10 +366,13 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
         auto count = [&] {                                               // all of them are: the last of the warps to say so counts them
             if (uncounted > 0 && phase >= 0) {
                 __syncwarp();
-                fence_gpu();                                         // y before the phase counter
-                if (lane == 0 && atomicAdd(const_cast<unsigned*>(&finished[phase & 3]), 1u) == kOutputWarps - 1u) {
-                    finished[phase & 3] = 0u;
-                    red_add_relaxed_u64(sa.phase_done + phase, (unsigned long long)uncounted);
+                if (lane == 0) {
+                    fence_cta();                                     // this warp's y before its count
+                    if (atomicAdd(const_cast<unsigned*>(&finished[phase & 3]), 1u) == kOutputWarps - 1u) {
+                        finished[phase & 3] = 0u;
+                        fence_gpu();                                 // all four warps' y before the phase counter
+                        red_add_relaxed_u64(sa.phase_done + phase, (unsigned long long)uncounted);
+                    }
                 }
             }
             uncounted = 0;
@@ -527,6 +530,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
         fence_gpu();
         const unsigned old = atomicAdd(sa.exit_count, 1u);
         if (old == gridDim.x - 1) {                    // last CTA out: counters back to zero
+            fence_gpu();
             for (int p = 0; p < sa.n_phases; p++) sa.phase_done[p] = 0ull;
             *sa.exit_count = 0u;
             fence_gpu();
