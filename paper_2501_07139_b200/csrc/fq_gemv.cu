@@ -338,6 +338,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                     else mbar_arrive(bar);
                 }
                 go = __shfl_sync(0xffffffffu, go, 0);
+                __syncwarp();                                          // what lane 0 has seen comes before the other lanes' copies (a shuffle orders nothing)
                 if (op.phase > 0) phase_known = op.phase - 1;          // (meaningless after an abort; unused then)
                 if (go == 0) { stop = true; break; }
                 if (go == 1 && lane < op.batch && FQ_IN_BOUNDS(k0 + have <= op.k_in && have <= kXCols, sa.status))
