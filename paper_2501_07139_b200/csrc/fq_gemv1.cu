@@ -578,6 +578,11 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
         };
         // Is the phase that produces this op's activations complete?  (phases are opened in order)
         auto phase_open = [&](int phase) -> bool { return phase <= 0 || (int)ctl[S::cPhaseKnown] >= phase; };
+        // ... and once lane 0 has seen that it is: the previous phase's outputs before this warp's loads
+        auto phase_seen = [&](int phase) {
+            if (phase > 0 && lane == 0) fence_cta();
+            __syncwarp();
+        };
         // Waits -- bounded -- until it is.  One warp of the CTA at a time polls the counters in global memory,
         // always the earliest phase that is not known to be complete (a warp whose next blob belongs to a
         // later phase must not keep a warp that still has to convert an earlier phase's activations from
@@ -599,7 +604,10 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
                                     ok = 0; break;
                                 }
                             }
-                            if (ok) ctl[S::cPhaseKnown] = (unsigned)(p + 1);
+                            if (ok) {
+                                fence_cta();                                     // (what this warp has acquired goes with the word)
+                                ctl[S::cPhaseKnown] = (unsigned)(p + 1);
+                            }
                         }
                         fence_cta();
                         ctl[S::cPollLock] = 0u;
@@ -610,6 +618,7 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
                 }
                 if (!ok && !ctl[S::cAbort]) raise_timeout(a, ctl);
             }
+            phase_seen(phase);
             return __shfl_sync(0xffffffffu, ok, 0) != 0;
         };
         auto load = [&](const Item& it, uint4& r0, uint4& r1) {
@@ -637,9 +646,9 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
                 const uint4 raw[2] = {r0, r1};
                 convert_blob(raw, xdig, xgrp, lane);
             }
-            fence_cta();
             __syncwarp();
             if (lane == 0) {
+                fence_cta();
                 ctl[S::cXCnt + slot] = (unsigned)it.uses;
                 ctl[S::cXTag + slot] = it.xs + 1u;
                 mbar_arrive(bars + 256 + 8 * slot);                        // wakes the consumers that sleep on this slot
@@ -656,7 +665,7 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
         while (va) {
             const bool vb = advance(B);
             bool issued = false;
-            if (vb && __shfl_sync(0xffffffffu, phase_open(B.phase) ? 1 : 0, 0)) { load(B, rb0, rb1); issued = true; }
+            if (vb && __shfl_sync(0xffffffffu, phase_open(B.phase) ? 1 : 0, 0)) { phase_seen(B.phase); load(B, rb0, rb1); issued = true; }
             if (!process(A, ra0, ra1)) break;
             if (vb && !issued) {
                 if (!phase_wait(B.phase)) break;
@@ -740,14 +749,17 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
                     else st_relaxed_u64(dpart + kb * 32 + lr, tag | __float_as_uint(v));   // finished elsewhere
                 }
             }
-            fence_cta();
             __syncwarp();
             int last = 0;
-            if (lane == 0) last = atomicAdd(const_cast<unsigned*>(&ctl[S::cStripCnt + sslot]), 1u) + 1u == (unsigned)expect;
+            if (lane == 0) {
+                fence_cta();                                                 // the sums before the count, the count before others' sums
+                last = atomicAdd(const_cast<unsigned*>(&ctl[S::cStripCnt + sslot]), 1u) + 1u == (unsigned)expect;
+                if (last) fence_cta();
+            }
             last = __shfl_sync(0xffffffffu, last, 0);
             if (!last) continue;
             // ---- this warp delivered the strip's last item
-            fence_cta();
+            __syncwarp();
             bool live = true;
             if (finish) {
                 // lane = row of the strip; blob sums in blob order: this CTA's from shared memory, then the blobs
@@ -794,13 +806,12 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
                 // a shared strip of a launch without dependencies: whoever publishes the last blob sum adds all of them up, in
                 // blob order.  Nobody waits for a CTA that may not be running yet.
                 const int mine = d.kb_hi - d.kb_lo, n_kb = d.n_kb;
-                fence_gpu();                                             // the sums of this CTA's items before the count
-                __syncwarp();
                 unsigned before = 0;
-                if (lane == 0 && FQ_IN_BOUNDS(d.counter >= 0 && d.counter < kArrivedMax, a.status)) before = atomicAdd(a.arrived + d.counter, (unsigned)mine);
+                if (lane == 0 && FQ_IN_BOUNDS(d.counter >= 0 && d.counter < kArrivedMax, a.status))
+                    before = atom_add_acq_rel(a.arrived + d.counter, (unsigned)mine);   // the sums of this CTA's items before, the others' after
                 before = __shfl_sync(0xffffffffu, before, 0);
                 if ((int)before + mine == n_kb) {
-                    fence_gpu();
+                    __syncwarp();
                     float sum = 0.f;
                     for (int q0 = 0; q0 < n_kb; q0 += 8) {
                         unsigned long long wv[8];
@@ -823,12 +834,13 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
             }
             if (!live) { let_copies_land(); break; }
             if (finish && phase >= 0) {
-                fence_gpu();                                             // y before the phase counter
                 __syncwarp();
                 if (lane == 0) {
+                    fence_cta();                                             // this warp's y before its count
                     const unsigned done = atomicAdd(const_cast<unsigned*>(&ctl[S::cFinCnt + (phase & 7)]), 1u) + 1u;
                     if (done == (unsigned)fin_total[phase]) {
                         ctl[S::cFinCnt + (phase & 7)] = 0u;
+                        fence_gpu();                                         // all warps' y before the phase counter
                         if (FQ_IN_BOUNDS(phase < a.n_phases, a.status)) red_add_relaxed_u64(a.phase_done + phase, 1ull);
                     }
                 }
@@ -841,6 +853,7 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
         fence_gpu();
         const unsigned old = atomicAdd(a.exit_count, 1u);
         if (old == gridDim.x - 1) {                    // last CTA out: counters back to zero
+            fence_gpu();
             for (int p = 0; p < a.n_phases; p++) a.phase_done[p] = 0ull;
             *a.exit_count = 0u;
             fence_gpu();
