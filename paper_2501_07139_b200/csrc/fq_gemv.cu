@@ -224,6 +224,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                             break;
                         }
                         unsigned long long t0 = 0ull;
+                        unsigned moved = tail + issued;              // (both only grow)
                         for (unsigned it = 0;; it++) {
                             // units that have been consumed since, in order
                             const unsigned old = tail + (unsigned)lane;
@@ -245,7 +246,9 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                             const unsigned left = __ballot_sync(0xffffffffu, todo);
                             issued = first + (unsigned)(n - __popc(left));
                             if (!left) break;
-                            // the ring is full, the usual case when the consumers wait for activations: sleep on the oldest unit's barrier
+                            // the ring is full, the usual case when the consumers wait for activations: sleep on the oldest unit's barrier.
+                            // What has a limit is the time without any progress
+                            if (tail + issued != moved) { moved = tail + issued; t0 = 0ull; }
                             int leave = 0;
                             if (lane == 0 && !mbar_try_wait(bars + 8 * (kPlaces + tail % kPlaces), (tail / kPlaces) & 1u) && (it & 15u) == 15u) {
                                 const unsigned long long now = global_ns();
