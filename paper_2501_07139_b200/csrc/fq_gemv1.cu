@@ -707,10 +707,16 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
             const int kb = (int)((e.y >> 10) & 31u), sslot = (int)((e.y >> 15) & 7u), variant = (int)((e.y >> 18) & 15u);
             const int tsel = (int)((e.y >> 22) & 3u);                        // 0: both tiles, 1 / 2: tile 0 / 1 only
             // ---- its weights and its activations
+            const bool held = ctl[S::cXTag + xslot] == e.z;                  // the slot holds (or is about to publish) this blob
             bool ok = wait_mbar(bars + 8 * stage, (uint32_t)parity, ctl, a.wait_ns);
             // (a hardware wake-up: at the start of a dependency phase every consumer sleeps here and must not
             // take issue slots from the pre-processing warps; the slot's barrier completes once per publication)
-            if (ok) ok = wait_mbar(bars + 256 + 8 * xslot, ((e.z - 1u) / kXSlots) & 1u, ctl, a.wait_ns);
+            const uint32_t xbar = bars + 256 + 8 * xslot, xparity = ((e.z - 1u) / kXSlots) & 1u;
+            if (ok) ok = wait_mbar(xbar, xparity, ctl, a.wait_ns);
+            // A warp whose item is that far ahead of the activation warps that the slot's blob before this one is not published yet
+            // has read the parity of the blob before that: only the barrier of a slot that holds this blob counts
+            if (ok && !held)
+                ok = wait_smem([&] { return ctl[S::cXTag + xslot] == e.z; }, ctl, a.wait_ns) && wait_mbar(xbar, xparity, ctl, a.wait_ns);
             if (!__all_sync(0xffffffffu, ok)) {
                 if (lane == 0 && !ctl[S::cAbort]) raise_timeout(a, ctl);
                 let_copies_land();

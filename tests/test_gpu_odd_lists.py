@@ -1,0 +1,40 @@
+"""Lists at batch 1 whose shares of a thread block are unusual: a blob or two of a matrix, hundreds of strips of a phase."""
+import pytest
+import torch
+
+import paper_2501_07139_b200 as P
+from fq_testlib import x_fp16
+
+pytestmark = pytest.mark.gpu
+
+
+def random_layer(fq, i, n, k, bits):
+    g = torch.Generator(device="cuda").manual_seed(1000 * i + bits)
+    w = torch.randn((n, k), device="cuda", generator=g)
+    fq.fq_pack_layer(i, *P.fq_quantize_layer(w, bits), bits, P.FQ_FMT_PACKED)
+
+
+# rows and columns of the layers, ops of the list, ops to a phase (0: no phases).  14336 columns are 28 blobs, as many as activation slots:
+# a block that has the last blob of one op and the first ones of the next needs the same slots twice within its first items.
+#   64 x one strip      : twelve blobs a block, of one op or two
+#   3 x 99 strips       : two strips and a blob or two of a third one a block and phase
+#   widths in turn      : slots of the next phase's activations come before those of this one are taken
+LISTS = [([(32, 14336)] * 4, 64, 0), ([(3168, 14336)] * 3, 12, 3), ([(3168, 14336), (96, 512), (4800, 2048)], 24, 3), ([(640, 14336), (64, 128)], 40, 1)]
+
+
+@pytest.mark.parametrize("shapes,n_ops,per_phase", LISTS)
+def test_a_blob_or_two_of_a_matrix(shapes, n_ops, per_phase):
+    fq = P.FlexQ(len(shapes))
+    for i, (n, k) in enumerate(shapes):
+        random_layer(fq, i, n, k, 2)
+    order = [j % len(shapes) for j in range(n_ops)]
+    xs = [x_fp16(184, j, 1, shapes[i][1]).cuda() for j, i in enumerate(order)]
+    want = [fq.fq_gemv(i, x, torch.empty((1, shapes[i][0]), dtype=torch.float16, device="cuda")) for i, x in zip(order, xs)]
+    phases = [j // per_phase for j in range(n_ops)] if per_phase else None
+    for _ in range(20):
+        ys = [torch.full_like(w, 7.0) for w in want]
+        fq.fq_gemv_stack(order, xs, ys, phases)
+        torch.cuda.synchronize()
+        assert all(torch.equal(y, w) for y, w in zip(ys, want))
+    assert fq.fq_status() == 0
+    fq.fq_destroy()
