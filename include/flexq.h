@@ -246,7 +246,8 @@ int fq_gemv_batched(fq_ctx* ctx, int layer, const uint16_t* x_dev, int batch, ui
  *   phases_host (may be NULL = no ordering): non-decreasing int [n_ops], starting at 0 and
  *       without gaps; an op of phase p does not read its x before every op of phase p-1 has
  *       written its y (weights of later ops are prefetched meanwhile).
- * Batch 1: at most 512 ops and 1024 phases per call (FQ_ERR_SHAPE otherwise).
+ * Batch 1: at most 512 ops and 1024 phases per call, and some 300 million outputs in a phase that another one follows
+ * (FQ_ERR_SHAPE otherwise).
  * A list of up to 8 ops at batch 1 without phases travels as kernel parameters.  Otherwise the call
  * builds a table (ops, and which strips every thread block computes) and uploads it from a
  * pinned buffer; a call with the same arguments under the same configuration reuses the uploaded

@@ -1,5 +1,6 @@
 // C ABI entry points: context, layer registry, configuration / footprint accountant,
 // argument checks and dispatch to the kernels.
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -837,6 +838,7 @@ int fq_gemv_stack(fq_ctx* ctx, int n_ops, const int* layers_host, const uint16_t
             // neighbour.
             uint2* ranges = reinterpret_cast<uint2*>(host + range_off);
             std::vector<int> last_phase(grid, -1);
+            std::vector<long long> finishing(grid);
             for (int g0 = 0, group = 0; g0 < n_ops; group++) {
                 int g1 = g0 + 1;
                 while (g1 < n_ops && (!phases_host || phases_host[g1] == phases_host[g0])) g1++;
@@ -856,6 +858,7 @@ int fq_gemv_stack(fq_ctx* ctx, int n_ops, const int* layers_host, const uint16_t
                 const bool whole_strips = phases_host && strips < 2ll * grid;
                 const int rot = (int)((unsigned)group * 53u % (unsigned)grid);      // spreads the remainders
                 unsigned long long before = 0;
+                std::fill(finishing.begin(), finishing.end(), 0ll);
                 for (int i = g0; i < g1; i++) {
                     const unsigned long long sz = ops[i].blob_cost;
                     const unsigned long long bytes = (unsigned long long)ops[i].n_units * sz;
@@ -875,6 +878,7 @@ int fq_gemv_stack(fq_ctx* ctx, int n_ops, const int* layers_host, const uint16_t
                         w.rp_first = w.lo / ops[i].n_kb;
                         w.rp_last = w.hi > w.lo ? (w.hi - 1) / ops[i].n_kb : w.rp_first;
                         ranges[(size_t)c * n_ops + i] = gemv1_pack_range(w, ops[i].n_kb);
+                        finishing[c] += w.finishing(ops[i].n_kb);
                         if (phases_host && w.finishing(ops[i].n_kb) > 0 && last_phase[c] != phases_host[i]) {
                             last_phase[c] = phases_host[i];
                             phase_total[phases_host[i]]++;
@@ -882,6 +886,8 @@ int fq_gemv_stack(fq_ctx* ctx, int n_ops, const int* layers_host, const uint16_t
                     }
                     before += bytes;
                 }
+                // (nobody waits for the last phase)
+                if (g1 < n_ops && *std::max_element(finishing.begin(), finishing.end()) > gemv1_max_phase_strips()) return FQ_ERR_SHAPE;
                 g0 = g1;
             }
         } else {

@@ -90,7 +90,7 @@ static_assert(sizeof(StripDesc) == 64, "descriptor layout");
 
 struct Smem {
     static constexpr int kFixed = kXSlots * (kXBlobDigitBytes + kXBlobGroupBytes + 8) + 1024 + kStripSlots * kMaxKb * 128 +
-                                  kCW * kQD * 16 + kStripSlots * 64 + kMaxPhasesDev + kMaxOpsDev * 8 + 1024;
+                                  kCW * kQD * 16 + kStripSlots * 64 + kMaxPhasesDev * 2 + kMaxOpsDev * 8 + 1024;
     static constexpr int kStages = (232448 - kFixed) / kStageBytes;
     static constexpr int oStages = 0;
     static constexpr int oXDig = oStages + kStages * kStageBytes;            // [slot][1024]
@@ -100,8 +100,8 @@ struct Smem {
     static constexpr int oQueue = oPart + kStripSlots * kMaxKb * 128;        // uint4 [warp][kQD]
     static constexpr int oStrip = oQueue + kCW * kQD * 16;                   // StripDesc [strip slot]
     static constexpr int oRange = oStrip + kStripSlots * 64;                 // uint2 [op]: this CTA's strips of every op
-    static constexpr int oFinTot = oRange + kMaxOpsDev * 8;                  // u8 [phase]: strips this CTA finishes
-    static constexpr int oBars = oFinTot + kMaxPhasesDev;                    // full[S], empty[S], then one per activation slot
+    static constexpr int oFinTot = oRange + kMaxOpsDev * 8;                  // u16 [phase]: strips this CTA finishes
+    static constexpr int oBars = oFinTot + kMaxPhasesDev * 2;                    // full[S], empty[S], then one per activation slot
     static constexpr int oCtl = oBars + 2 * 16 * 8 + kXSlots * 8;
     // control words (u32 each)
     static constexpr int cXTag = 0;                                          // [kXSlots] activation blob number + 1 held
@@ -334,7 +334,7 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
     const uint32_t sbase = smem_u32(smem);
     const uint32_t bars = sbase + S::oBars;                               // full[s] at 8 s, empty[s] at 128 + 8 s
     volatile unsigned* ctl = reinterpret_cast<volatile unsigned*>(smem + S::oCtl);
-    unsigned char* fin_total = smem + S::oFinTot;
+    unsigned short* fin_total = reinterpret_cast<unsigned short*>(smem + S::oFinTot);
     const uint2* range = reinterpret_cast<const uint2*>(smem + S::oRange);
     const GemvOp* ops = a.table ? a.table : inl.op;
 
@@ -350,7 +350,7 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
     for (int i = threadIdx.x; i < S::kCtlWords; i += blockDim.x) ctl[i] = 0u;
     for (int i = threadIdx.x; i < 256; i += blockDim.x) reinterpret_cast<uint32_t*>(smem + S::oZero)[i] = 0u;
     for (int i = threadIdx.x; i < kCW * kQD * 4; i += blockDim.x) reinterpret_cast<uint32_t*>(smem + S::oQueue)[i] = 0u;
-    for (int i = threadIdx.x; i < kMaxPhasesDev / 4; i += blockDim.x) reinterpret_cast<uint32_t*>(fin_total)[i] = 0u;
+    for (int i = threadIdx.x; i < kMaxPhasesDev / 2; i += blockDim.x) reinterpret_cast<uint32_t*>(fin_total)[i] = 0u;
     // this CTA's strips of every op
     for (int oi = threadIdx.x; oi < a.n_ops; oi += blockDim.x) {
         uint2 r;
@@ -364,8 +364,8 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
         for (int oi = threadIdx.x; oi < a.n_ops; oi += blockDim.x) {
             const int phase = ops[oi].phase;
             const int fin = StripOrder(range[oi], ops[oi].n_kb).finishing();
-            if (fin > 0 && phase >= 0)                              // four 8-bit counters per word
-                atomicAdd(reinterpret_cast<unsigned*>(fin_total) + (phase >> 2), (unsigned)fin << (8 * (phase & 3)));
+            if (fin > 0 && phase >= 0)                              // two 16-bit counters per word (enough: checked on the host)
+                atomicAdd(reinterpret_cast<unsigned*>(fin_total) + (phase >> 1), (unsigned)fin << (16 * (phase & 1)));
         }
     }
     __syncthreads();
@@ -905,6 +905,7 @@ unsigned next_epoch(unsigned& e)
 }  // namespace
 
 int gemv1_max_phases() { return kMaxPhasesDev; }
+int gemv1_max_phase_strips() { return 65535; }
 int gemv1_max_ops() { return kMaxOpsDev; }
 uint2 gemv1_pack_range(const CtaWork& w, int n_chunks) { return pack_range(w, n_chunks); }
 int gemv1_max_k() { return kMaxKb * 512; }

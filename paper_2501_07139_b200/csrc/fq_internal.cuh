@@ -158,6 +158,7 @@ int launch_gemv1_inline(Ctx* ctx, const InlineOps& ops, int n_ops, cudaStream_t 
 // table_dev: [GemvOp x n_ops][int phase_total x max(n_phases,1)][uint2 strips x sm_count x n_ops]
 int launch_gemv1_stack(Ctx* ctx, const StackHeader& hdr, const char* table_dev, cudaStream_t st);
 int gemv1_max_phases();
+int gemv1_max_phase_strips();       // strips of a phase that one CTA finishes
 int gemv1_max_ops();
 int gemv1_max_k();
 int gemv1_chunk_blobs(int blob_read_bytes);

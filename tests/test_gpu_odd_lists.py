@@ -38,3 +38,28 @@ def test_a_blob_or_two_of_a_matrix(shapes, n_ops, per_phase):
         assert all(torch.equal(y, w) for y, w in zip(ys, want))
     assert fq.fq_status() == 0
     fq.fq_destroy()
+
+
+def test_hundreds_of_strips_of_a_phase():
+    """A phase of which every block finishes more than 255 strips; the next one reads its outputs, which are no numbers before."""
+    n, k, ops = 65536, 128, 24                           # 24 x 2048 strips: 332 a block of 148
+    fq = P.FlexQ(2)
+    random_layer(fq, 0, n, k, 2)
+    random_layer(fq, 1, 640, 14336, 4)
+    x = x_fp16(185, 0, 1, k).cuda()
+    want = fq.fq_gemv(0, x, torch.empty((1, n), dtype=torch.float16, device="cuda"))
+    ends = [want[:, -14336:].clone(), want[:, :14336].clone()]
+    after = [fq.fq_gemv(1, e, torch.empty((1, 640), dtype=torch.float16, device="cuda")) for e in ends]
+    torch.cuda.synchronize()
+    assert all(torch.isfinite(a).all() for a in after)
+    ys = [torch.empty_like(want) for _ in range(ops)]
+    last = [torch.empty_like(a) for a in after]
+    for _ in range(10):
+        for y in ys:
+            y.fill_(float("nan"))
+        fq.fq_gemv_stack([0] * ops + [1, 1], [x] * ops + [ys[-1][:, -14336:], ys[0][:, :14336]], ys + last, [0] * ops + [1, 1])
+        torch.cuda.synchronize()
+        assert all(torch.equal(y, want) for y in ys)
+        assert all(torch.equal(a, b) for a, b in zip(last, after))
+    assert fq.fq_status() == 0
+    fq.fq_destroy()
