@@ -150,7 +150,8 @@ __device__ __forceinline__ void prefetch_ops(const GemvOp* ops, int oi, int n_op
     }
 }
 // The strips of one op for one CTA: rp_first .. rp_last; the first starts at blob c_first, the last ends
-// before blob c_last (see CtaWork).  Packed into two words per (CTA, op) by the host for a stack call.
+// before blob c_last (see CtaWork).  Packed into two words per (CTA, op) by the host for a stack call: 24 bits of strip (an op has
+// fewer than 2^21 blobs), eight of blob.
 constexpr uint32_t kRangeEmpty = 0xffffffffu;
 FQ_HD uint2 pack_range(const CtaWork& w, int n_kb)
 {
@@ -158,7 +159,7 @@ FQ_HD uint2 pack_range(const CtaWork& w, int n_kb)
     int f0, f1, l0, l1;
     w.chunks(n_kb, w.rp_first, f0, f1);
     w.chunks(n_kb, w.rp_last, l0, l1);
-    return uint2{(uint32_t)w.rp_first | (uint32_t)f0 << 20, (uint32_t)w.rp_last | (uint32_t)l1 << 20};
+    return uint2{(uint32_t)w.rp_first | (uint32_t)f0 << 24, (uint32_t)w.rp_last | (uint32_t)l1 << 24};
 }
 struct StripOrder {
     int rp_first, rp_last, c_first, c_last, n_kb, n_strips;
@@ -166,8 +167,8 @@ struct StripOrder {
     {
         n_kb = n_kb_;
         if (r.x == kRangeEmpty) { n_strips = 0; rp_first = rp_last = c_first = c_last = 0; return; }
-        rp_first = (int)(r.x & 0xfffffu); c_first = (int)(r.x >> 20);
-        rp_last = (int)(r.y & 0xfffffu); c_last = (int)(r.y >> 20);
+        rp_first = (int)(r.x & 0xffffffu); c_first = (int)(r.x >> 24);
+        rp_last = (int)(r.y & 0xffffffu); c_last = (int)(r.y >> 24);
         n_strips = rp_last - rp_first + 1;
     }
     __device__ __forceinline__ int strip(int i) const { return rp_first + i; }

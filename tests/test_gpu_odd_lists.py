@@ -63,3 +63,24 @@ def test_hundreds_of_strips_of_a_phase():
         assert all(torch.equal(a, b) for a, b in zip(last, after))
     assert fq.fq_status() == 0
     fq.fq_destroy()
+
+
+def test_more_rows_than_twenty_bits_of_strips():
+    """33.5 million outputs are 2^20 strips; the layer has a few more."""
+    n, k, bits = (1 << 25) + 2000, 128, 2
+    fq = P.FlexQ(1)
+    codes = torch.randint(0, 4, (n, k), dtype=torch.uint8, device="cuda", generator=torch.Generator(device="cuda").manual_seed(7))
+    scales = torch.full((n, 1), 2.0 ** -6, dtype=torch.float16, device="cuda")
+    zeros = torch.ones((n, 1), dtype=torch.float16, device="cuda")
+    fq.fq_pack_layer(0, codes, scales, zeros, bits, P.FQ_FMT_PACKED)
+    x = x_fp16(186, 0, 1, k).cuda()
+    ys = [torch.full((1, n), float("nan"), dtype=torch.float16, device="cuda") for _ in range(2)]
+    fq.fq_gemv(0, x, ys[0])
+    fq.fq_gemv_stack([0], [x], ys[1:], [0])
+    assert fq.fq_status() == 0
+    for rows in (slice(0, 70000), slice((1 << 25) - 70000, n)):
+        want = ((codes[rows].double() - 1) * 2.0 ** -6) @ x[0].double()
+        for y in ys:
+            assert float((y[0, rows].double() - want).norm() / want.norm()) <= 1e-3
+    assert torch.equal(ys[0], ys[1])
+    fq.fq_destroy()
