@@ -577,7 +577,8 @@ static int launch_batch(Ctx* ctx, const GemvOp& single, StackArgs& sa, int batch
     sa.note = ctx->note;
     sa.stored = ctx->stored;
     sa.wait_ns = ctx->wait_limit_ns;
-    if (zeros_are_low(ctx))
+    // (a captured launch runs whenever its graph does, and so does a captured call that stores weights: no answer holds for them)
+    if (zeros_are_low(ctx) && !ctx->stores_in_graphs && !is_capturing(st))
         return batch_pad(batch) == 4 ? launch_impl<4, false>(ctx, single, sa, total_units, st) : launch_impl<8, false>(ctx, single, sa, total_units, st);
     return batch_pad(batch) == 4 ? launch_impl<4, true>(ctx, single, sa, total_units, st) : launch_impl<8, true>(ctx, single, sa, total_units, st);
 }

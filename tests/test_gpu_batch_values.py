@@ -98,6 +98,61 @@ def test_zero_points_that_come_later(tmp_path):
     for f in (fq, loaded, swapped):
         f.fq_destroy()
 
+
+def test_zero_points_that_a_graph_stores():
+    """A captured fq_pack_layer stores high zero points after calls have run without any; a captured decode call runs after they were
+    stored eagerly."""
+    import paper_2501_07139_b200 as P
+    n, k, batch, bits = 75, 1152, 4, 8
+    low, (high, w) = make_layer(138, 0, n, k, bits), _high(138, n, k, bits)
+    x = x_fp16(138, 0, batch, k).cuda()
+    want = f64_of(x) @ w.T
+
+    def setup():
+        fq = P.FlexQ(1)
+        store = fq.fq_pack_layer(0, *to_dev(*low), bits, P.FQ_FMT_PACKED)
+        dev = to_dev(*high)
+
+        def pack():
+            assert P.lib().fq_pack_layer(fq._h, 0, n, k, bits, 128, P.FQ_FMT_PACKED, *(t.data_ptr() for t in dev), store.data_ptr(),
+                                         torch.cuda.current_stream().cuda_stream) == 0
+
+        return fq, pack, dev
+
+    def decode(fq, y):
+        fq.fq_gemv_batched(0, x, y)
+
+    y = torch.zeros((batch, n), dtype=torch.float16, device="cuda")
+    fq, pack, keep = setup()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        pack()
+    for _ in range(3):
+        decode(fq, y)
+        assert fq.fq_status() == 0
+    graph.replay()
+    for _ in range(2):
+        decode(fq, y)
+        assert fq.fq_status() == 0
+        assert all(O.rel_l2(f64_of(y)[b], want[b]) <= 5e-4 for b in range(batch))
+    del graph
+    fq.fq_destroy()
+
+    fq, pack, keep = setup()
+    for _ in range(3):
+        decode(fq, y)
+        assert fq.fq_status() == 0
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        decode(fq, y)
+    pack()
+    graph.replay()
+    assert fq.fq_status() == 0
+    assert all(O.rel_l2(f64_of(y)[b], want[b]) <= 5e-4 for b in range(batch))
+    del graph
+    fq.fq_destroy()
+
+
 @pytest.mark.parametrize("bad", [float("inf"), float("-inf"), float("nan")])
 @pytest.mark.parametrize("batch", [1, 2, 4, 5, 8])
 def test_an_activation_that_is_no_number(batch, bad):
