@@ -132,8 +132,7 @@ int fill_op(const Ctx* ctx, int layer, const uint16_t* x, uint16_t* y, int batch
     op.k_in = L.k_in;
     op.n_kb = k_blobs(L.k_in);
     op.n_rp = row_pairs(L.n_out);
-    op.chunk_blobs = one ? gemv1_chunk_blobs(op.blob_read) : 1;
-    op.n_chunks = op.n_kb;                                       // batch 2..8: a chunk of K is a blob
+    op.chunk_blobs = one ? gemv1_chunk_blobs(op.blob_read) : 0;
     op.batch = batch;
     // what is dealt to the CTAs: batch 1 the blobs of every strip, batch 2..8 the K chunks of every row pair
     op.n_units = op.n_kb * op.n_rp;
@@ -154,7 +153,7 @@ int fill_op(const Ctx* ctx, int layer, const uint16_t* x, uint16_t* y, int batch
 size_t op_partial_bytes(const GemvOp& op, bool one, int max_batch)
 {
     if (one) return op.n_kb <= 1 ? 0 : (size_t)op.n_rp * op.n_kb * 32 * sizeof(unsigned long long);
-    return (size_t)op.n_rp * op.n_chunks * gemv_partial_bytes_per_unit(max_batch);
+    return (size_t)op.n_rp * op.n_kb * gemv_partial_bytes_per_unit(max_batch);
 }
 
 // Scratch that a registered layer can need in one launch, whatever its active variant and the batch.

@@ -192,7 +192,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
             int lo, hi;
             cta_range(op.n_units, op.rot, cta, grid, lo, hi);
             if (lo < hi) {
-                const int n_rp = op.n_rp, n_kb = op.n_kb, n_chunks = op.n_chunks, variant = op.variant;
+                const int n_rp = op.n_rp, n_kb = op.n_kb, variant = op.variant;
                 const uint32_t bytes = (uint32_t)op.blob_read;
                 const long long blob_stride = op.blob_stride;
                 const uint8_t* const store = op.store;
@@ -211,7 +211,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                         const unsigned off = wrapped ? ((unsigned)lane - before_wrap) * bytes : head + (unsigned)lane * bytes;
                         const unsigned start = wrapped ? vhead + ((unsigned)S::kRing - head) + off : vhead + (unsigned)lane * bytes;
                         // the chunk whose CTA adds up a row pair rotates with the row pair, so that this work is spread evenly over the CTAs
-                        const bool finishes = lane < n && ch == my_rp % n_chunks;
+                        const bool finishes = lane < n && ch == my_rp % n_kb;
                         const unsigned fin = __ballot_sync(0xffffffffu, finishes);
                         const unsigned unit = issued + (unsigned)lane, place = unit % kPlaces, first = issued;
                         const uint32_t full = bars + 8 * place;
@@ -237,7 +237,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
                             if (todo && start + bytes - low <= (unsigned)S::kRing && unit - tail < (unsigned)kPlaces) {
                                 int4* d = reinterpret_cast<int4*>(smem + S::oDesc + place * (int)sizeof(UnitDesc));
                                 d[0] = make_int4(ch, my_rp, (int)off, seg);
-                                d[1] = make_int4(variant, n_chunks, (int)(uint32_t)(uintptr_t)partial, (int)(uint32_t)((uintptr_t)partial >> 32));
+                                d[1] = make_int4(variant, n_kb, (int)(uint32_t)(uintptr_t)partial, (int)(uint32_t)((uintptr_t)partial >> 32));
                                 *reinterpret_cast<int2*>(d + 2) = make_int2(finishes ? oseq + __popc(fin & ((1u << lane) - 1u)) : -1, (int)start);
                                 mbar_expect_tx(full, bytes);
                                 bulk_g2s(smem_u32(smem + S::oRing) + off, store + ((long long)my_rp * n_kb + ch) * blob_stride, bytes, full);
@@ -391,7 +391,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
             int lo, hi;
             cta_range(op.n_units, op.rot, cta, grid, lo, hi);
             if (lo >= hi) continue;
-            const int n_rp = op.n_rp, n_chunks = op.n_chunks;
+            const int n_rp = op.n_rp, n_chunks = op.n_kb;
             if (op.phase != phase) { count(); phase = op.phase; }
             for (int ch = lo / n_rp; ch <= (hi - 1) / n_rp && !stop; ch++) {
                 const int rp_lo = max(lo - ch * n_rp, 0), rp_hi = min(hi - ch * n_rp, n_rp);
@@ -598,7 +598,7 @@ int launch_gemv_single(Ctx* ctx, const GemvOp& op, cudaStream_t st)
     sa.n_ops = 1;
     sa.n_phases = 0;
     sa.epoch = next_epoch(ctx->launch_epoch);
-    const long long units = (long long)op.n_rp * op.n_chunks;
+    const long long units = (long long)op.n_rp * op.n_kb;
     return launch_batch(ctx, op, sa, op.batch, units, st);
 }
 

@@ -31,26 +31,23 @@ constexpr int kUnitRowTiles = 2;   // a decode unit covers two 16-row tiles (32 
 struct GemvOp {
     const uint8_t* store;        // blobs [row_pair][k_blob]
     unsigned long long* partial; // split-K partial sums, one tagged word per (row pair, chunk, row, batch entry)
-    // read by every consumer warp for every unit: kept together, 16-byte aligned, one vector load
     int blob_read;               // bytes of every blob that this op reads (all of it, or a nested child's prefix)
     int variant;                 // variant_index(format, bits): selects the specialised inner loop
     int batch;
-    int n_chunks;                // K chunks
     const uint16_t* x;           // fp16 [batch][k_in]
     uint16_t* y;                 // fp16 [batch][n_out]
     int blob_stride;             // bytes from one blob to the next (size of the stored variant's blobs)
     int n_fields;
     int n_out, k_in;
-    int n_kb;                    // k blobs
+    int n_kb;                    // k blobs; batch 2..8: K chunks, of a blob each
     int n_rp;                    // row pairs = units per K chunk
     int chunk_blobs;             // batch 1: k blobs that one stage of the ring holds, at most
     int phase;                   // -1: no ordering
-    int n_units;                 // n_chunks * n_rp
+    int n_units;                 // n_kb * n_rp
     int rot;                     // rotation of the CTA blocks for this op (evens out remainders); inline ops: its first strip counter
     int split;                   // batch 1: consumer items per blob: 1 (both 16-row tiles) or 2 (one tile each)
     unsigned blob_cost;          // batch 1: cost of a blob (512 bytes x cost of a byte of the variant)
 };
-static_assert(offsetof(GemvOp, blob_read) == 16 && offsetof(GemvOp, partial) == 8, "consumer block of the op descriptor");
 
 struct StackHeader {
     int n_ops;

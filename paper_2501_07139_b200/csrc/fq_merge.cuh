@@ -22,32 +22,27 @@ __device__ __forceinline__ void merge_nibbles(uint32_t upper, uint32_t lower, ui
     odd = pick<0xccccccccu>(upper, lower >> 2);
 }
 
-// The words of the first N fields -> the parent's bytes of steps 0 .. 3, dropped bits zero (of the last field the upper KEEP bits count).
+// The words of the first N fields, two or more -> the parent's bytes of steps 0 .. 3, dropped bits zero (of the last field the upper KEEP bits count).
 template <int N, int KEEP>
 __device__ __forceinline__ void merge_bytes(const uint32_t (&w)[4], uint32_t (&step)[4])
 {
     constexpr uint32_t kPair = 0xccccccccu, kHigh = 0xf0f0f0f0u;
-    static_assert(N >= 1 && N <= 4 && (KEEP == 1 || KEEP == 2), "fields of a nested child");
-    if constexpr (N == 1) {
-        constexpr uint32_t m = 0xc0c0c0c0u & (KEEP == 2 ? ~0u : 0x80808080u);
-        step[0] = (w[0] << 6) & m; step[1] = (w[0] << 4) & m; step[2] = (w[0] << 2) & m; step[3] = w[0] & m;
+    static_assert(N >= 2 && N <= 4 && (KEEP == 1 || KEEP == 2), "fields of a nested child");
+    uint32_t ue, uo;
+    merge_nibbles(w[0], w[1], ue, uo);
+    if constexpr (N == 2) {
+        constexpr uint32_t m = KEEP == 2 ? kHigh : 0xe0e0e0e0u;
+        step[0] = (ue << 4) & m; step[1] = (uo << 4) & m; step[2] = ue & m; step[3] = uo & m;
     } else {
-        uint32_t ue, uo;
-        merge_nibbles(w[0], w[1], ue, uo);
-        if constexpr (N == 2) {
-            constexpr uint32_t m = KEEP == 2 ? kHigh : 0xe0e0e0e0u;
-            step[0] = (ue << 4) & m; step[1] = (uo << 4) & m; step[2] = ue & m; step[3] = uo & m;
+        uint32_t ve, vo;
+        if constexpr (N == 3) {
+            constexpr uint32_t m = KEEP == 2 ? kPair : 0x88888888u;
+            ve = (w[2] << 2) & m; vo = w[2] & m;
         } else {
-            uint32_t ve, vo;
-            if constexpr (N == 3) {
-                constexpr uint32_t m = KEEP == 2 ? kPair : 0x88888888u;
-                ve = (w[2] << 2) & m; vo = w[2] & m;
-            } else {
-                merge_nibbles(w[2], KEEP == 2 ? w[3] : w[3] & 0xaaaaaaaau, ve, vo);
-            }
-            step[0] = pick<kHigh>(ue << 4, ve); step[2] = pick<kHigh>(ue, ve >> 4);
-            step[1] = pick<kHigh>(uo << 4, vo); step[3] = pick<kHigh>(uo, vo >> 4);
+            merge_nibbles(w[2], KEEP == 2 ? w[3] : w[3] & 0xaaaaaaaau, ve, vo);
         }
+        step[0] = pick<kHigh>(ue << 4, ve); step[2] = pick<kHigh>(ue, ve >> 4);
+        step[1] = pick<kHigh>(uo << 4, vo); step[3] = pick<kHigh>(uo, vo >> 4);
     }
 }
 
