@@ -440,6 +440,19 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
             uint16_t* const y = cur.y;
             unsigned long long* const partial = cur.partial;
             const bool contiguous = cur.blob_read == cur.blob_stride;
+            // Consumers wait for an activation slot's barrier by parity, which tells a use of the slot from the one before it and not from
+            // the one before that.  So an op's items are queued once every blob that its own ones replace in their slots has been
+            // published.  (Such a blob belongs to an earlier op, all of whose items are queued: this wait holds up nobody that it waits for.)
+            if (xseq + (unsigned)n_kb > (unsigned)kXSlots) {
+                const int x = (int)(xseq + (unsigned)n_kb) - kXSlots - 1 - lane;
+                auto published = [&] { return lane >= kXSlots || x < 0 || (int)(ctl[S::cXTag + x % kXSlots] - (unsigned)(x + 1)) >= 0; };
+                if (!__all_sync(0xffffffffu, published())) {
+                    const bool in_time = wait_smem(published, ctl, a.wait_ns);
+                    if (!in_time && !ctl[S::cAbort]) raise_timeout(a, ctl);
+                    if (!__all_sync(0xffffffffu, in_time)) { stop = true; break; }
+                }
+                fence_cta();
+            }
             for (int si = 0; si < so.n_strips && !stop; si++) {
                 const int rp = so.strip(si);
                 int c0, c1;
@@ -649,10 +662,10 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
             }
             __syncwarp();
             if (lane == 0) {
-                fence_cta();
                 ctl[S::cXCnt + slot] = (unsigned)it.uses;
-                ctl[S::cXTag + slot] = it.xs + 1u;
                 mbar_arrive(bars + 256 + 8 * slot);                        // wakes the consumers that sleep on this slot
+                fence_cta();
+                ctl[S::cXTag + slot] = it.xs + 1u;                         // (after the barrier: the producer and the next use go by it)
             }
             return true;
         };
@@ -708,16 +721,10 @@ gemv1_kernel(const __grid_constant__ InlineOps inl, const Args a)
             const int kb = (int)((e.y >> 10) & 31u), sslot = (int)((e.y >> 15) & 7u), variant = (int)((e.y >> 18) & 15u);
             const int tsel = (int)((e.y >> 22) & 3u);                        // 0: both tiles, 1 / 2: tile 0 / 1 only
             // ---- its weights and its activations
-            const bool held = ctl[S::cXTag + xslot] == e.z;                  // the slot holds (or is about to publish) this blob
             bool ok = wait_mbar(bars + 8 * stage, (uint32_t)parity, ctl, a.wait_ns);
             // (a hardware wake-up: at the start of a dependency phase every consumer sleeps here and must not
             // take issue slots from the pre-processing warps; the slot's barrier completes once per publication)
-            const uint32_t xbar = bars + 256 + 8 * xslot, xparity = ((e.z - 1u) / kXSlots) & 1u;
-            if (ok) ok = wait_mbar(xbar, xparity, ctl, a.wait_ns);
-            // A warp whose item is that far ahead of the activation warps that the slot's blob before this one is not published yet
-            // has read the parity of the blob before that: only the barrier of a slot that holds this blob counts
-            if (ok && !held)
-                ok = wait_smem([&] { return ctl[S::cXTag + xslot] == e.z; }, ctl, a.wait_ns) && wait_mbar(xbar, xparity, ctl, a.wait_ns);
+            if (ok) ok = wait_mbar(bars + 256 + 8 * xslot, ((e.z - 1u) / kXSlots) & 1u, ctl, a.wait_ns);
             if (!__all_sync(0xffffffffu, ok)) {
                 if (lane == 0 && !ctl[S::cAbort]) raise_timeout(a, ctl);
                 let_copies_land();
