@@ -50,8 +50,8 @@ __device__ __forceinline__ unsigned long long global_ns()
     return t;
 }
 // Orders this thread's accesses, and those it has seen, before its later ones.  (__threadfence is a sequentially consistent fence, more
-// than any of the flags and counters here need: with it four 7B blocks in order take 161.3 us at 4 bits and 228 nested at 6, with
-// these 160.7 and 227, and fq_gemm on 4096 x 11008 at 77 tokens 21.3 and 21.0.)
+// than the flags and counters here need where an atomic that hands something over has one of these on both of its sides.  What the
+// difference gives, half a percent of four 7B blocks in order, is not beyond the scatter of the measurements.)
 __device__ __forceinline__ void fence_cta() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
 __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 __device__ __forceinline__ unsigned atom_add_acq_rel(unsigned* p, unsigned v)
