@@ -511,6 +511,7 @@ gemv_kernel(const __grid_constant__ GemvOp single, const StackArgs sa)
             if (live) blob_dispatch<BP>(d.variant, d.blob, xs, lane, tile, tot);
             __syncwarp();
             if (lane == 0) {
+                fence_cta();                                     // all lanes' reads of the activations before the count below
                 mbar_arrive(empty);                              // the place may be filled again
                 atomicSub(const_cast<int*>(&x_pending[slot]), 1);   // one warp fewer needs the activation slot
             }
